@@ -34,6 +34,7 @@
 #include "batch.cuh"
 #include "profile.cuh"
 #include "stencil_ep.cuh"
+#include "stencil_fx.cuh"
 #include "beam.cuh"
 #include "stencil_v2.cuh"
 #include <algorithm>
@@ -89,6 +90,7 @@ struct Level {
     EpsSlot* eps_aux;
     ChebTable* cheb;
     bool pv_valid;
+    FxTiling fx;  // FP64 3D: tiling of the fixed-point kernel
 };
 
 }  // namespace jfnk
@@ -235,6 +237,9 @@ static size_t plan(P& p, char* base, const jfnk_options* o) {
     if (const char* e = getenv("JFNK_ZM3D_MIN_N_F32")) p.zm_min_n32 = atoi(e);
     if (const char* e = getenv("JFNK_EP3D_CLUSTER_MIN_N")) p.cl_min_n32 = atoi(e);
     if (const char* e = getenv("JFNK_EP3D_CLUSTER_MAX_N")) p.cl_max_n32 = atoi(e);
+    // an explicit choice of another FP64 kernel stands
+    const bool fx = !getenv("JFNK_EP3D_MAX_N_F64") && !getenv("JFNK_ZM3D_MIN_N_F64") && !getenv("JFNK_V2_THREADS_F64");
+    for (Level& L : p.lv) L.fx = fx ? fx3d_tiling(L.g) : FxTiling{};
     // the cluster kernels' attributes are set here, outside any graph capture
     if (p.cl_max_n32 > 0 && !ep3d_cluster_init()) p.cl_max_n32 = 0;
     if (const char* e = getenv("JFNK_V2_THREADS_F64")) p.v2_threads64 = atoi(e);
@@ -372,6 +377,7 @@ static StencilArgs<T> base_args(P& p, int l) {
     a.cl_max_n = sizeof(T) == 4 ? p.cl_max_n32 : 0;
     a.v2_threads = sizeof(T) == 8 ? p.v2_threads64 : p.v2_threads32;
     a.v3 = sizeof(T) == 4 ? p.v3_f32 : 0;
+    if (sizeof(T) == 8) a.fx = L.fx;
     return a;
 }
 

@@ -1,0 +1,20 @@
+// FP64 residual kernels of the 3D diffusion problems with the element
+// arithmetic in 64-bit fixed point (fx64.cuh): one launch per action, no
+// scratch.
+#pragma once
+#include "stencil.cuh"
+
+namespace jfnk {
+
+// The tiling for a grid; no CTAs where the kernel does not apply (scalar 3D
+// grids up to n = 1024 only).
+FxTiling fx3d_tiling(const Grid& g);
+
+// True when the fixed-point kernel takes this FP64 call: a.fx is set, and the
+// outputs are apart from the vectors whose neighbouring values other threads
+// still read.
+bool fx3d_use(const StencilArgs<double>& a, Mode mode);
+
+jfnk_status launch_fx3d(Prob prob, Mode mode, const StencilArgs<double>& a, cudaStream_t st);
+
+}  // namespace jfnk
