@@ -7,6 +7,7 @@
 #include "batch.cuh"
 #include "reduce.cuh"
 #include "stencil_body.cuh"
+#include "stencil_fx2d.cuh"
 
 namespace jfnk {
 
@@ -29,13 +30,13 @@ __global__ void __launch_bounds__(512) stencil2d_batched_kernel(const StencilArg
     }
 }
 
-template <typename T>
-jfnk_status launch_stencil2d_batched(Mode mode, const StencilArgs<T>* dev_args, const BTile* dev_tiles, int ntiles,
-                                     int bx, cudaStream_t st, int grid) {
+template <>
+jfnk_status launch_stencil2d_batched<float>(Mode mode, const StencilArgs<float>* dev_args, const BTile* dev_tiles,
+                                            int ntiles, int bx, cudaStream_t st, int grid) {
     if (ntiles <= 0) return JFNK_OK;
     const int g = (grid > 0 && grid < ntiles) ? grid : ntiles;
-    const size_t smem = sizeof(T) * (2 * (bx + 1) + 4 * bx);
-#define JFNK_B2(MM) stencil2d_batched_kernel<T, MM><<<g, bx, smem, st>>>(dev_args, dev_tiles, ntiles)
+    const size_t smem = sizeof(float) * (2 * (bx + 1) + 4 * bx);
+#define JFNK_B2(MM) stencil2d_batched_kernel<float, MM><<<g, bx, smem, st>>>(dev_args, dev_tiles, ntiles)
     switch (mode) {
         case Mode::F: JFNK_B2(Mode::F); break;
         case Mode::JV: JFNK_B2(Mode::JV); break;
@@ -48,10 +49,34 @@ jfnk_status launch_stencil2d_batched(Mode mode, const StencilArgs<T>* dev_args, 
     JFNK_LAUNCH_CHECK();
     return JFNK_OK;
 }
-template jfnk_status launch_stencil2d_batched<double>(Mode, const StencilArgs<double>*, const BTile*, int, int,
-                                                      cudaStream_t, int);
-template jfnk_status launch_stencil2d_batched<float>(Mode, const StencilArgs<float>*, const BTile*, int, int,
-                                                     cudaStream_t, int);
+
+// FP64: one CTA per (instance, strip, row chunk), element arithmetic in fixed
+// point (stencil_fx2d.cuh); the tile's x0 is the strip.
+template <Mode M>
+__global__ void __launch_bounds__(32 * kFx2Warps) fx2d_batched_kernel(const StencilArgs<double>* __restrict__ args,
+                                                                      const BTile* __restrict__ tiles) {
+    __shared__ double red_sm[32];
+    const BTile t = tiles[blockIdx.x];
+    fx2d_cta<Prob::BRATU2, M>(args[t.inst], t.x0, t.y0, t.y1, t.bid, t.nblk, red_sm);
+}
+
+template <>
+jfnk_status launch_stencil2d_batched<double>(Mode mode, const StencilArgs<double>* dev_args, const BTile* dev_tiles,
+                                             int ntiles, int, cudaStream_t st, int) {
+    if (ntiles <= 0) return JFNK_OK;
+#define JFNK_B2(MM) fx2d_batched_kernel<MM><<<ntiles, 32 * kFx2Warps, 0, st>>>(dev_args, dev_tiles)
+    switch (mode) {
+        case Mode::F: JFNK_B2(Mode::F); break;
+        case Mode::JV: JFNK_B2(Mode::JV); break;
+        case Mode::BMJ: JFNK_B2(Mode::BMJ); break;
+        case Mode::CHEB0: JFNK_B2(Mode::CHEB0); break;
+        case Mode::CHEB: JFNK_B2(Mode::CHEB); break;
+        case Mode::CHEBLAST: JFNK_B2(Mode::CHEBLAST); break;
+    }
+#undef JFNK_B2
+    JFNK_LAUNCH_CHECK();
+    return JFNK_OK;
+}
 
 // ---------------------------------------------------------------------------
 // batched vector operations

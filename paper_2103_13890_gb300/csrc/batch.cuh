@@ -79,7 +79,8 @@ struct BScal {
     int* status;
 };
 
-// grid > 0 (< ntiles): persistent launch of `grid` CTAs looping over the tiles
+// FP32: bx threads a CTA; grid > 0 (< ntiles): persistent launch of `grid` CTAs
+// looping over the tiles.  FP64: one CTA per tile, bx and grid unused.
 template <typename T>
 jfnk_status launch_stencil2d_batched(Mode mode, const StencilArgs<T>* dev_args, const BTile* dev_tiles, int ntiles,
                                      int bx, cudaStream_t st, int grid = 0);

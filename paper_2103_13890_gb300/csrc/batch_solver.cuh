@@ -41,7 +41,7 @@ struct Arena {
     }
 };
 
-// Tiling of the batched 2D kernel: threads per CTA, target CTA count of a
+// Tiling of the batched FP32 2D kernel: threads per CTA, target CTA count of a
 // launch (sets the row-chunk length), persistent grid size (0: one CTA per tile).
 struct TileCfg {
     int bx = 160;
@@ -50,7 +50,7 @@ struct TileCfg {
 };
 
 struct BCtx {
-    TileCfg tile[2];  // [0] FP32, [1] FP64 launches
+    TileCfg tile;  // FP32 launches
     std::vector<P*> ps;
     std::vector<double*> u;
     int B = 0;
@@ -130,6 +130,26 @@ static std::vector<BTile> tiles_for(const std::vector<Grid>& gs, int bx = kBatch
     return t;
 }
 
+// FP64 tiles (stencil_fx2d.cuh): x0 is the strip of node columns
+static std::vector<BTile> tiles_fx2d(const std::vector<Grid>& gs) {
+    long long total = 0;
+    for (const Grid& g : gs) total += (long long)fx2d_strips(g.n) * g.ny;
+    const int rows = fx2d_cta_rows(total);
+    std::vector<BTile> t;
+    for (int k = 0; k < (int)gs.size(); ++k) {
+        const Grid& g = gs[k];
+        const int strips = fx2d_strips(g.n);
+        // (an instance's reduction scratch holds 2 kMaxRedBlocks partials)
+        const int most = std::max(1, 2 * kMaxRedBlocks / strips);
+        const int rk = std::max(rows, (g.ny + most - 1) / most);
+        const int ch = (g.ny + rk - 1) / rk;
+        for (int c = 0; c < ch; ++c)
+            for (int s = 0; s < strips; ++s)
+                t.push_back(BTile{k, s, c * rk, std::min(c * rk + rk, g.ny), 0, c * strips + s, strips * ch, 0});
+    }
+    return t;
+}
+
 template <typename T>
 static jfnk_status bstencil(BCtx& b, Arena& A, Mode m, const std::vector<int>& S, int lvl_from_coarse,
                             const std::vector<StencilArgs<T>>& args) {
@@ -137,8 +157,8 @@ static jfnk_status bstencil(BCtx& b, Arena& A, Mode m, const std::vector<int>& S
     std::vector<Grid> gs;
     for (int i : S) gs.push_back(b.ps[i]->lv[lvl_from_coarse].g);
     jfnk_status err = JFNK_OK;
-    const TileCfg& tc = b.tile[sizeof(T) == 8 ? 1 : 0];
-    const std::vector<BTile> tiles = tiles_for(gs, tc.bx, tc.target);
+    const TileCfg& tc = b.tile;
+    const std::vector<BTile> tiles = sizeof(T) == 8 ? tiles_fx2d(gs) : tiles_for(gs, tc.bx, tc.target);
     const StencilArgs<T>* da = stage(b, A, args, err);
     const BTile* dt = stage(b, A, tiles, err);
     if (err != JFNK_OK) return err;
@@ -515,12 +535,11 @@ static jfnk_status bjv64(BCtx& b, const std::vector<int>& S, const std::vector<c
     std::vector<Grid> gs;
     for (int i : S) gs.push_back(b.ps[i]->lv[b.ps[i]->L].g);
     jfnk_status err = JFNK_OK;
-    const TileCfg& tc = b.tile[1];
-    const std::vector<BTile> tiles = tiles_for(gs, tc.bx, tc.target);
+    const std::vector<BTile> tiles = tiles_fx2d(gs);
     const StencilArgs<double>* da = stage(b, b.dyn, args, err);
     const BTile* dt = stage(b, b.dyn, tiles, err);
     JFNK_TRY(err);
-    return launch_stencil2d_batched<double>(Mode::JV, da, dt, (int)tiles.size(), tc.bx, b.st, tc.grid);
+    return launch_stencil2d_batched<double>(Mode::JV, da, dt, (int)tiles.size(), 0, b.st);
 }
 
 // F_i = F(x_i), A_i = A(x_i) (FP64, finest) and ||F_i|| into res slot 0
@@ -540,12 +559,11 @@ static jfnk_status bresidual64(BCtx& b, const std::vector<int>& S, const std::ve
         p.nFplain[p.L]++;
     }
     jfnk_status err = JFNK_OK;
-    const TileCfg& tc = b.tile[1];
-    const std::vector<BTile> tiles = tiles_for(gs, tc.bx, tc.target);
+    const std::vector<BTile> tiles = tiles_fx2d(gs);
     const StencilArgs<double>* da = stage(b, b.dyn, args, err);
     const BTile* dt = stage(b, b.dyn, tiles, err);
     JFNK_TRY(err);
-    JFNK_TRY(launch_stencil2d_batched<double>(Mode::F, da, dt, (int)tiles.size(), tc.bx, b.st, tc.grid));
+    JFNK_TRY(launch_stencil2d_batched<double>(Mode::F, da, dt, (int)tiles.size(), 0, b.st));
     std::vector<const void*> xv(F.begin(), F.end());
     std::vector<double*> outs;
     for (int i : S) outs.push_back(b.res + (size_t)i * kResStride);
@@ -1057,13 +1075,12 @@ static void tile_cache_store(const std::string& key, const TileCfg& c, double ms
     fclose(f);
 }
 
-template <typename T>
 static jfnk_status tune_tiles(BCtx& b) {
-    const int ti = sizeof(T) == 8 ? 1 : 0;
+    using T = float;
     std::vector<int> ns;
     for (P* p : b.ps) ns.push_back(p->lv[p->L].g.n);
     std::sort(ns.begin(), ns.end());
-    std::string key = std::string("bratu2d_") + (ti ? "f64" : "f32");
+    std::string key = "bratu2d_f32";
     for (size_t k = 0; k < ns.size();) {
         size_t e = k;
         while (e < ns.size() && ns[e] == ns[k]) ++e;
@@ -1072,7 +1089,7 @@ static jfnk_status tune_tiles(BCtx& b) {
     }
     auto it = tile_cache().find(key);
     if (it != tile_cache().end()) {
-        b.tile[ti] = it->second;
+        b.tile = it->second;
         return JFNK_OK;
     }
     std::vector<int> all(b.B);
@@ -1083,13 +1100,8 @@ static jfnk_status tune_tiles(BCtx& b) {
         P& p = *b.ps[i];
         gs.push_back(p.lv[p.L].g);
         StencilArgs<T> a = base_args<T>(p, p.L);
-        if (ti) {
-            a.u = (const T*)b.u[i];
-            a.out = (T*)p.Ftrial;
-        } else {
-            a.u = as<T>(p.lv[p.L].x);
-            a.out = as<T>(p.lv[p.L].t);
-        }
+        a.u = as<T>(p.lv[p.L].x);
+        a.out = as<T>(p.lv[p.L].t);
         args.push_back(a);
     }
     int dev = 0, sms = kNumSMs;
@@ -1127,7 +1139,7 @@ static jfnk_status tune_tiles(BCtx& b) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    b.tile[ti] = best;
+    b.tile = best;
     tile_cache_store(key, best, best_ms / 3.0);
     return JFNK_OK;
 }
@@ -1144,8 +1156,7 @@ static jfnk_status bsolve(BCtx& b, jfnk_stats* stats) {
     std::vector<long long> ci0(B, 0);
     for (int i = 0; i < B; ++i)
         JFNK_CUDA_TRY(cudaMemcpyAsync(&ci0[i], b.ps[i]->coarse_iters, sizeof(long long), cudaMemcpyDeviceToHost, b.st));
-    JFNK_TRY(tune_tiles<double>(b));
-    if (sizeof(T) == 4) JFNK_TRY(tune_tiles<T>(b));
+    if (sizeof(T) == 4) JFNK_TRY(tune_tiles(b));
     auto Fs = [&](const std::vector<int>& S, bool trial) {
         std::vector<double*> F, A;
         for (int i : S) {

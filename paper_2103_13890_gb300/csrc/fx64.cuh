@@ -1,5 +1,5 @@
-// 64-bit fixed-point evaluation of the 3D nonlinear-diffusion element, for the
-// FP64 kernels.
+// 64-bit fixed-point evaluation of the 3D nonlinear-diffusion, 2D Bratu and 2D
+// minimal-surface elements, for the FP64 kernels.
 //
 // What bounds an FP64 element kernel on this GPU is the FP64 pipe: 2
 // operations per clock and SM.  The integer pipe adds 64-bit integers at ~52
@@ -25,6 +25,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include "fx_tables.cuh"
+
 #ifndef __CUDACC__
 #include <cmath>
 #ifndef __host__
@@ -37,6 +39,11 @@
 namespace jfnk {
 
 typedef long long fx_t;
+
+#ifdef __CUDACC__
+static __device__ const fx_t kFxExp2Dev[256] = {JFNK_FX_EXP2_TABLE};
+#endif
+static const fx_t kFxExp2Host[256] = {JFNK_FX_EXP2_TABLE};
 
 __host__ __device__ __forceinline__ int fx_hi(fx_t a) { return (int)(a >> 32); }
 __host__ __device__ __forceinline__ unsigned int fx_lo(fx_t a) { return (unsigned int)a; }
@@ -186,6 +193,8 @@ __host__ __device__ __forceinline__ FxScale fx_scale_kappa(const FxScale& sc, do
 // field (lower 10): 0 for zero, 1 (and no significand) below 2^-422, kFxBad for
 // what the fixed-point path leaves to FP64 (non-finite, 2^54 and above), else
 // the biased exponent - 600.
+constexpr int kFxTiny = -4000;  // exponent of a vanishing part
+constexpr int kFxFp64 = 8000;   // marks contributions held as doubles
 constexpr int kFxBias = 600, kFxBad = 1023, kFxMask = 1023;
 constexpr int kFxMinExp = 1023 - 300 - kFxBias, kFxMaxExp = 1023 + 54 - kFxBias;
 __host__ __device__ __forceinline__ fx_t fx_pack(double w) {
@@ -313,6 +322,201 @@ __host__ __device__ __forceinline__ void fx_nd3(const fx_t p[8], int xm, const F
     r[4] = f0_01 - f1_01; r[5] = f0_01 + f1_01;
     r[6] = f0_11 - f1_11; r[7] = f0_11 + f1_11;
     X = sc.ex + 3 + f - k - s;
+}
+
+// ---------------------------------------------------------------------------
+// 2D elements.  Corner index a + 2b; the three gradient modes are left-aligned
+// as in 3D.
+// ---------------------------------------------------------------------------
+struct FxModes2 {
+    fx_t m00, m10, m01, m11;  // m00 at 2^-k; the others at 2^-(k + s), below 2^62
+    int k, s;
+};
+__host__ __device__ __forceinline__ FxModes2 fx_modes2(const fx_t p[4], int xm) {
+    FxModes2 m;
+    m.k = 55 - (xm + kFxBias - 1022);
+    fx_t u[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) u[c] = fx_sar(p[c] & ~(fx_t)kFxMask, 8 + xm - fx_exp(p[c]));
+    const fx_t p0 = u[0] + u[1], q0 = u[1] - u[0], p1 = u[2] + u[3], q1 = u[3] - u[2];
+    m.m00 = p0 + p1;
+    m.m10 = q0 + q1;
+    m.m01 = p1 - p0;
+    m.m11 = q1 - q0;
+    auto mag = [](fx_t a) { return (unsigned int)(fx_hi(a) ^ (fx_hi(a) >> 31)); };
+    const unsigned int top = mag(m.m10) | mag(m.m01) | mag(m.m11);
+    if (top) {
+        m.s = fx_clz(top) - 2;
+    } else {
+        auto low = [](fx_t a) { return fx_lo(a) ^ (unsigned int)(fx_hi(a) >> 31); };
+        m.s = 30 + fx_clz(low(m.m10) | low(m.m01) | low(m.m11));
+    }
+    m.m10 = fx_shl(m.m10, m.s);
+    m.m01 = fx_shl(m.m01, m.s);
+    m.m11 = fx_shl(m.m11, m.s);
+    return m;
+}
+
+// exp(U 2^-57) for |U| < 2^61: V 2^(N - 58), V in [2^58, 2^59].
+//   exp(u) = 2^N 2^(j/256) exp(z), 256 N + j = floor(256 u / ln 2) (a little
+//   below it at times), 0 <= z < 1.01 ln 2 / 256; exp(z) by its Taylor
+//   polynomial of degree 5 (next term z^6 / 720 < 2^-60), the terms from z^3 on
+//   in 32 bits (z^2 / 2 < 2^-18 times them).  Error below 2^-55 of exp(u).
+__host__ __device__ __forceinline__ fx_t fx_exp_table(int j) {
+#ifdef __CUDA_ARCH__
+    return __ldg(&kFxExp2Dev[j]);
+#else
+    return kFxExp2Host[j];
+#endif
+}
+__host__ __device__ __forceinline__ fx_t fx_exp(fx_t U, int& N) {
+    const int n = (fx_mulhi_s(fx_hi(U), 1549082005) - 64) >> 15;  // 256 / ln 2 2^22; U's upper word is u 2^25
+    // z 2^70: ln 2 / 256 2^70 = 0x2c5c85fdf473de6b
+    const unsigned long long zs = ((unsigned long long)U << 13) - (unsigned long long)(long long)n * 0x2c5c85fdf473de6bULL;
+    const unsigned int zh = (unsigned int)(zs >> 32), zl = (unsigned int)zs;   // zh = z 2^38
+    const unsigned long long zz = (unsigned long long)zh * zh + 2ULL * fx_mulhi_u(zh, zl);  // z^2 2^76
+    // S = z/3 + z^2/12 + z^3/60 = z (1/3 + z (1/12 + z/60))
+    const unsigned int t1 = 1431655765u + fx_mulhi_u(zh, 4473924u);   // 1/12 + z/60, times 2^34
+    const unsigned int t2 = 1431655765u + (fx_mulhi_u(zh, t1) >> 8);  // 1/3 + z t1, times 2^32
+    const unsigned int S = (unsigned int)(((unsigned long long)zh * t2) >> 30);  // times 2^40
+    // z^2/2 (1 + S): at 2^70
+    const unsigned long long q = (zz >> 7) + (((unsigned long long)(unsigned int)(zz >> 27) * S) >> 20);
+    // (1 + z + q) 2^61 times 2^(j/256) 2^61
+    const fx_t F = ((fx_t)1 << 61) + (fx_t)((zs + q) >> 9);
+    N = n >> 8;
+    return fx_mul(F, fx_split(fx_exp_table(n & 255)));
+}
+
+// Source multipliers of the Bratu element: A^k |lh| 2^62 2^-ex, lh = lambda h^2 / 16.
+struct FxBratu {
+    FxMul b0, b1, b2;
+    int ex;
+    bool neg;
+};
+__host__ __device__ __forceinline__ FxBratu fx_bratu(double lh) {
+    FxBratu s;
+    s.neg = dbl_hi(lh) < 0;
+    const double a = s.neg ? -lh : lh;
+    if (a == 0.0) {
+        s.b0 = s.b1 = s.b2 = FxMul{0, 0};
+        s.ex = kFxTiny;
+        return s;
+    }
+    s.b0 = fx_significand(a, s.ex);  // m 2^62
+    s.b1 = fx_split(fx_shl(fx_mul(kFxA1, s.b0), 1));
+    s.b2 = fx_split(fx_shl(fx_mul(kFxA2, s.b0), 1));
+    return s;
+}
+__host__ __device__ __forceinline__ bool fx_bratu_ok(double lh) {
+    return lh == 0.0 || fx_scale_ok(lh) || fx_scale_ok(-lh);
+}
+// elem_bratu2 takes |u| < 16
+__host__ __device__ __forceinline__ bool fx_bratu_exp_ok(int x) { return x >= kFxMinExp && x < 1023 + 4 - kFxBias; }
+
+// elem_bratu2 in fixed point; r[4] times 2^X, below 2^62.4
+__host__ __device__ __forceinline__ void fx_bratu2(const fx_t p[4], int xm, const FxBratu& b, fx_t r[4], int& X) {
+    const FxModes2 m = fx_modes2(p, xm);
+    const FxMul A1 = fx_split(kFxA1), A2 = fx_split(kFxA2);
+    // u at the points, times 2^57
+    const fx_t T10 = fx_mul(m.m10, A1), T01 = fx_mul(m.m01, A1), T11 = fx_mul(m.m11, A2);
+    const int e = 55 - m.k, sh = m.s - 1 - e;
+    const fx_t U0 = e > 0 ? fx_shl(m.m00, e) : fx_sar(m.m00, -e);
+    int N[4];
+    fx_t V[4];
+    V[0] = fx_exp(U0 + fx_sar(T11 - T10 - T01, sh), N[0]);   // (sx, sy) = (-, -)
+    V[1] = fx_exp(U0 + fx_sar(T10 - T01 - T11, sh), N[1]);   // (+, -)
+    V[2] = fx_exp(U0 + fx_sar(T01 - T10 - T11, sh), N[2]);   // (-, +)
+    V[3] = fx_exp(U0 + fx_sar(T10 + T01 + T11, sh), N[3]);   // (+, +)
+    const int n01 = N[0] > N[1] ? N[0] : N[1], n23 = N[2] > N[3] ? N[2] : N[3];
+    const int nm = n01 > n23 ? n01 : n23;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) V[q] = fx_sar(V[q], nm - N[q]);
+    const fx_t s0 = V[0] + V[1], s1 = V[2] + V[3], d0 = V[1] - V[0], d1 = V[3] - V[2];
+    // lh A^k E at 2^(nm + ex - 56)
+    fx_t E00 = fx_mul(s1 + s0, b.b0), E01 = fx_mul(s1 - s0, b.b1), E10 = fx_mul(d1 + d0, b.b1), E11 = fx_mul(d1 - d0, b.b2);
+    const int xs = nm + b.ex - 56, xg = -m.k - m.s - 1;
+    X = (xs > xg ? xs : xg) + 1;
+    const int ss = X - xs, sg = X - xg;
+    const fx_t G10 = fx_sar(m.m10, sg + 1), G01 = fx_sar(m.m01, sg + 1), G11 = fx_sar(fx_mul(m.m11, fx_split(0x5555555555555555LL)), sg);
+    E00 = fx_sar(E00, ss);
+    E10 = fx_sar(E10, ss);
+    E01 = fx_sar(E01, ss);
+    E11 = fx_sar(E11, ss);
+    const fx_t R00 = b.neg ? E00 : -E00;
+    const fx_t R10 = b.neg ? G10 + E10 : G10 - E10;
+    const fx_t R01 = b.neg ? G01 + E01 : G01 - E01;
+    const fx_t R11 = b.neg ? G11 + E11 : G11 - E11;
+    const fx_t g00 = R00 - R01, g01 = R00 + R01, g10 = R10 - R11, g11 = R10 + R11;
+    r[0] = g00 - g10;
+    r[1] = g00 + g10;
+    r[2] = g01 - g11;
+    r[3] = g01 + g11;
+}
+
+// 1 / sqrt(S 2^(F - 61)) times 2^61, for 0 < S < 2^62, F even and a result of at
+// most 1: a 24-bit start from the hardware reciprocal square root and one
+// third-order Newton step (error 5/16 e^3, e < 2^-21).
+__host__ __device__ __forceinline__ fx_t fx_rsqrt(fx_t S, int F) {
+    int n = fx_hi(S) ? fx_clz((unsigned int)fx_hi(S)) : 32 + fx_clz(fx_lo(S));
+    n = (n - 3) | 1;  // odd, and m = S 2^n in [2^60, 2^62)
+    const fx_t m = n > 0 ? fx_shl(S, n) : S >> 1;
+    const float f = (float)fx_hi(m) * 0x1p-28f;  // m 2^-60 in [1, 4)
+#ifdef __CUDA_ARCH__
+    const unsigned int y0 = __float2uint_rn(rsqrtf(f) * 0x1p31f);
+#else
+    const unsigned int y0 = (unsigned int)std::lrint(1.0f / std::sqrt(f) * 0x1p31f);
+#endif
+    const fx_t e = ((fx_t)1 << 58) - fx_mul(m, fx_split((fx_t)((unsigned long long)y0 * y0)));  // (1 - m y0^2) 2^58
+    const int e40 = (int)(e >> 18);
+    const fx_t c4 = (e + ((fx_t)e40 * e40 * 3 >> 24)) * 8;  // (e/2 + 3/8 e^2) 2^62
+    const fx_t y = fx_shl(y0, 30) + (fx_t)fx_hi(c4) * (fx_t)y0 + fx_mulhi_u(fx_lo(c4), y0);
+    // S 2^(F - 61) = (m 2^-60) 2^(F - 1 - n)
+    return fx_sar(y, (F - 1 - n) / 2);
+}
+
+// inv_h2 of the minimal-surface element, and the corner range it takes
+struct FxMinsurf {
+    FxMul m;
+    int ex;
+};
+__host__ __device__ __forceinline__ FxMinsurf fx_minsurf(double inv_h2) {
+    FxMinsurf s;
+    s.m = fx_significand(inv_h2, s.ex);
+    return s;
+}
+// elem_minsurf2 in fixed point; r[4] times 2^X, below 2^62.7.  False where a
+// slope reaches 64 (left to FP64, as the coefficients then differ by more than
+// their common scale should hold).
+__host__ __device__ __forceinline__ bool fx_minsurf2(const fx_t p[4], int xm, const FxMinsurf& ih, fx_t r[4], int& X) {
+    const FxModes2 m = fx_modes2(p, xm);
+    const FxMul A1 = fx_split(kFxA1);
+    // h grad u at 2^-(k + s)
+    const fx_t gx0 = m.m10 >> 1, gy0 = m.m01 >> 1, gd = fx_mul(m.m11, A1);
+    const fx_t gxm = gx0 - gd, gxp = gx0 + gd, gym = gy0 - gd, gyp = gy0 + gd;
+    auto sq = [](fx_t g) -> fx_t {  // g^2 / 2^64
+        const FxMul s = fx_split(g);
+        return (fx_t)s.h * s.h + (fx_t)fx_mulhi_s(s.h, s.l) * 2;
+    };
+    const fx_t axm = sq(gxm), axp = sq(gxp), aym = sq(gym), ayp = sq(gyp);
+    // (a + b) inv_h2 = p 2^xa, p < 2^59
+    const int xa = ih.ex + 66 - 2 * (m.k + m.s);
+    int F = xa + 59;
+    if (F > 12) return false;
+    F = F > 0 ? (F + 1) & ~1 : 0;
+    const fx_t one = (fx_t)1 << (61 - F);
+    const int sh = F - (xa + 59);
+    auto coef = [&](fx_t a, fx_t b) -> fx_t { return fx_rsqrt(one + fx_sar(fx_shl(fx_mul(a + b, ih.m), 2), sh), F); };
+    const fx_t cmm = coef(axm, aym), cpm = coef(axm, ayp), cmp = coef(axp, aym), cpp = coef(axp, ayp);
+    const fx_t Xm = fx_mul(gxm, fx_split(cmm + cpm)), Xp = fx_mul(gxp, fx_split(cmp + cpp));
+    const fx_t Ym = fx_mul(gym, fx_split(cmm + cmp)), Yp = fx_mul(gyp, fx_split(cpm + cpp));
+    const fx_t P1 = Xm + Xp, P2 = Ym + Yp;
+    const fx_t P3 = fx_shl(fx_mul((Xp - Xm) + (Yp - Ym), A1), 1);
+    r[0] = P3 - P1 - P2;
+    r[1] = P1 - P2 - P3;
+    r[2] = P2 - P1 - P3;
+    r[3] = P1 + P2 + P3;
+    X = -m.k - m.s;
+    return true;
 }
 
 // an integer times 2^X as a double (correctly rounded; X keeps it normal)

@@ -35,6 +35,7 @@
 #include "profile.cuh"
 #include "stencil_ep.cuh"
 #include "stencil_fx.cuh"
+#include "stencil_fx2d.cuh"
 #include "beam.cuh"
 #include "stencil_v2.cuh"
 #include <algorithm>

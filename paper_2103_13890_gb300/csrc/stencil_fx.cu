@@ -35,8 +35,6 @@ namespace jfnk {
 #define FX_B 2
 #endif
 constexpr int kFxThreads = FX_T, kFxBlocks = FX_B;  // largest CTA, CTAs per SM
-constexpr int kFxZero = -4000;  // exponent of zero contributions
-constexpr int kFxFp64 = 8000;   // marks contributions held as doubles
 
 // FP64 evaluation of the element at (x, y, z), for values outside the
 // fixed-point range (non-finite or huge values, magnitudes near underflow,
@@ -116,7 +114,7 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx3d_kernel(const Stenc
                 epilogue<double, M>(a, z * sz + sidx, false, 0.0, 0.0, ck, red);
         };
         fx_t p[8], carry[4] = {0, 0, 0, 0};  // corners; contributions to the upper face ...
-        int xl = 0, Xc = kFxZero;            // ... times 2^Xc, or doubles (kFxFp64)
+        int xl = 0, Xc = kFxTiny;            // ... times 2^Xc, or doubles (kFxFp64)
         auto face = [&](int z, fx_t* q) -> int {
             const fx_t* Wz = W + (z & 1) * np + corner;
             q[0] = Wz[0];
@@ -145,7 +143,7 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx3d_kernel(const Stenc
                 const int xm = max(xl, xu);
                 const bool fits = fx_exp_ok(xm) && (!KAPPA || fx_scale_ok(kap));
                 fx_t r[8];
-                int Xr = kFxZero;
+                int Xr = kFxTiny;
                 if (fits) {
                     if (KAPPA)
                         fx_nd3(p, xm, fx_scale_kappa(sc0, kap), r, Xr);
@@ -239,24 +237,25 @@ static bool overlap(const void* p, const void* q, size_t bytes) {
     return p && q && x < y + bytes && y < x + bytes;
 }
 
-bool fx3d_use(const StencilArgs<double>& a, Mode mode) {
-    if (a.fx.ctas == 0) return false;
-    if (!fx_scale_ok(a.node_scale)) return false;
+bool fx_outputs_alias(const StencilArgs<double>& a, Mode mode) {
     const size_t bytes = sizeof(double) * (size_t)a.g.size;
     const void* in[2] = {a.u, mode == Mode::F ? nullptr : a.v};
-    const void* out[5] = {a.out, a.out2, nullptr, nullptr, nullptr};
+    const void* out[3] = {a.out, nullptr, nullptr};
     if (mode == Mode::CHEB || mode == Mode::CHEBLAST) {
-        out[0] = out[1] = nullptr;
-        out[2] = a.r;
-        out[3] = a.s;
-        out[4] = a.dnew;
-    } else if (mode != Mode::F && mode != Mode::CHEB0) {
-        out[1] = nullptr;
+        out[0] = a.r;
+        out[1] = a.s;
+        out[2] = a.dnew;
+    } else if (mode == Mode::F || mode == Mode::CHEB0) {
+        out[1] = a.out2;
     }
     for (const void* i : in)
         for (const void* o : out)
-            if (overlap(i, o, bytes)) return false;
-    return true;
+            if (overlap(i, o, bytes)) return true;
+    return false;
+}
+
+bool fx3d_use(const StencilArgs<double>& a, Mode mode) {
+    return a.fx.ctas > 0 && fx_scale_ok(a.node_scale) && !fx_outputs_alias(a, mode);
 }
 
 template <Prob P, Mode M>

@@ -6,7 +6,8 @@
 //      accepted range, corners of equal and of very different size, kappa over
 //      its range.  Worst case of the bit budget: 2^7 units on a largest
 //      contribution of at least 2^54, i.e. 2^-47 of it.
-//   2. fields assembled over 6^3 elements: the error's 2-norm is at most 1.5
+//   2. the 2D elements likewise.
+//   3. fields assembled over 6^3 elements: the error's 2-norm is at most 1.5
 //      times that of the FP64 element (a quarter to a hundredth where the
 //      field is smooth or random).
 // Prints violations and "ok <cases>".
@@ -65,8 +66,69 @@ static std::mt19937_64 rng(11);
 static double uni() { return std::uniform_real_distribution<double>(-1, 1)(rng); }
 static double nrm() { return std::normal_distribution<double>()(rng); }
 
+// 2D elements: Bratu (par = lambda h^2 / 16) or minimal surface (par = 1 / h^2)
+static void reference2(bool ms, const double w[4], Q par, Q r[4]) {
+    const Q a = 1 / (2 * std::sqrt((Q)3));
+    for (int c = 0; c < 4; ++c) r[c] = 0;
+    for (int q = 0; q < 4; ++q) {
+        const Q px = (q & 1) ? (Q)0.5 + a : (Q)0.5 - a, py = (q & 2) ? (Q)0.5 + a : (Q)0.5 - a;
+        Q N[4], gx[4], gy[4], u = 0, x = 0, y = 0;
+        for (int c = 0; c < 4; ++c) {
+            const Q lx = (c & 1) ? px : 1 - px, ly = (c & 2) ? py : 1 - py;
+            N[c] = lx * ly;
+            gx[c] = (c & 1) ? ly : -ly;
+            gy[c] = (c & 2) ? lx : -lx;
+            u += N[c] * w[c];
+            x += gx[c] * ((Q)w[c] - w[0]);  // (the gradients' weights sum to zero)
+            y += gy[c] * ((Q)w[c] - w[0]);
+        }
+        const Q k = ms ? 1 / std::sqrt(1 + (x * x + y * y) * par) : (Q)1;
+        for (int c = 0; c < 4; ++c) {
+            r[c] += k * (x * gx[c] + y * gy[c]) / 4;
+            if (!ms) r[c] -= 4 * par * std::exp(u) * N[c];
+        }
+    }
+}
+
+// single 2D elements: errors against the element's largest contribution or
+// source.  Bit budget: 2^6 units on at least 2^55 (exp 2^-55, rsqrt 2^-54).
+static int check2(int& cases) {
+    int bad = 0;
+    for (int ms = 0; ms < 2; ++ms)
+        for (int ex : {-299, -100, -30, -6, -1, 0, 1, 3})
+            for (int it = 0; it < 400; ++it) {
+                const double par = ms ? std::ldexp(1.0 + std::fabs(uni()), (it % 4 == 0 ? 12 : 3) - 2 * ex)
+                                      : (it % 7 ? 1 : -1) * std::ldexp(std::fabs(uni()), -(int)(rng() % 30));
+                double w[4];
+                fx_t p[4], r[4];
+                int xm = 0, X = 0;
+                for (int c = 0; c < 4; ++c) {
+                    w[c] = std::ldexp(it % 3 == 0 ? uni() : it % 3 == 1 ? ((it >> (c + 2)) & 1 ? 0.999 : -0.999) : 0.7 + 1e-10 * uni(), ex);
+                    p[c] = fx_pack(w[c]);
+                    xm = std::max(xm, fx_exp(p[c]));
+                }
+                ++cases;
+                Q q[4], big = 0, err = 0;
+                reference2(ms, w, par, q);
+                if (ms) {
+                    if (!fx_exp_ok(xm) || !fx_minsurf2(p, xm, fx_minsurf(par), r, X)) continue;  // left to FP64
+                } else {
+                    if (!fx_exp_ok(xm) || !fx_bratu_exp_ok(xm)) { printf("2D refused: %d\n", ex), ++bad; continue; }
+                    fx_bratu2(p, xm, fx_bratu(par), r, X);
+                    big = std::fabs((Q)par) * std::exp((Q)std::max({w[0], w[1], w[2], w[3]}));
+                }
+                for (int c = 0; c < 4; ++c) {
+                    big = std::max(big, std::fabs(q[c]));
+                    err = std::max(err, std::fabs(q[c] - (Q)fx_to_double(r[c], X)));
+                }
+                if (!(err <= 0x1p-49L * big)) printf("2D %d exponent %d case %d: %Lg of %Lg\n", ms, ex, it, err, big), ++bad;
+            }
+    return bad;
+}
+
 int main() {
     int bad = 0, cases = 0;
+    bad += check2(cases);
     const double scale = 3.0 / 16 / 100;
     const int exps[] = {-299, -120, -40, -8, -2, -1, 0, 1, 2, 9, 30, 53};
     for (int ex : exps)

@@ -5,10 +5,13 @@ sums of element integrals: each is within c 2^-53 of the sum of the magnitudes
 of an element's terms, c = 64 covering its ~45 roundings, which is what the
 tolerance takes from the "ep" result of |w| (the diffusion terms of a node sum
 to at most 8 x 16 times the largest corner value's share)."""
+import functools
+
 import numpy as np
 import pytest
 
 from gpu_common import dev, host, jf, kernel_path, torch
+from oracle import fem
 
 pytestmark = pytest.mark.gpu
 
@@ -103,3 +106,61 @@ def test_output_may_be_an_input(monkeypatch):
     w = v.clone()
     p.jvp(u, F, w, eps=1e-4, out=w)
     assert torch.equal(w, J)
+
+
+# ---- 2D: strips of 30 node columns, a warp each ---------------------------
+# Tolerance as above for the gradient part (stiffness entries up to 2/3, 4
+# elements of 4 corners; minimal surface: coefficient at most 1) plus the
+# source's lambda h^2 max exp(u).
+
+
+@functools.lru_cache(maxsize=None)
+def _case2d(kind, n, what):
+    rng = np.random.default_rng(n)
+    u = rng.uniform(-0.9, 0.9, size=(n + 1, n + 1)) / (n if kind == "minsurf2d" else 1)
+    if what in ("nan", "inf"):
+        u[n // 2, 1] = u[1, n // 3] = np.nan if what == "nan" else np.inf
+    elif what == "range":  # Bratu: |u| to 30; minimal surface: slopes to 1e4
+        u *= 33.0 if kind == "bratu2d" else 1e4
+    elif what == "tiny":
+        u *= 1e-130
+    elif what == "zero":
+        u[: n // 2 + 1] = 0
+    with np.errstate(all="ignore"):
+        return u, fem.residual(kind, u, 5.0, None, None)
+
+
+def _tol2d(kind, u, n):
+    m = np.max(np.abs(u[np.isfinite(u)]))
+    return 64 * EPS * (16 * 2 / 3 * m + (5.0 / n ** 2 * np.exp(m) if kind == "bratu2d" else 0.0))
+
+
+# one strip and part of a warp (2, 29..32), several strips, ragged rows
+@pytest.mark.parametrize("kind,n,what",
+                         [(k, n, "plain") for k in ("bratu2d", "minsurf2d") for n in (2, 3, 29, 30, 31, 32, 61, 95, 250)] +
+                         [(k, 48, w) for k in ("bratu2d", "minsurf2d") for w in ("nan", "inf", "range", "tiny", "zero")])
+def test_2d_matches_oracle(kind, n, what):
+    u, G = _case2d(kind, n, what)
+    p = jf().Problem(kind, n, 1, lam=5.0)
+    F = host(p.residual(dev(u)))
+    fine = np.isfinite(G)
+    assert np.array_equal(fine, np.isfinite(F))
+    tol = _tol2d(kind, u, n)
+    assert np.max(np.abs(F - G)[fine]) <= tol
+    if what == "plain":
+        v = np.random.default_rng(n + 1).normal(size=u.shape) * (0.1 / n if kind == "minsurf2d" else 1.0)
+        eps = 1e-4
+        inner = np.zeros_like(u)
+        inner[1:-1, 1:-1] = 1
+        K = (fem.residual(kind, u + eps * v * inner, 5.0, None, None) - G) / eps
+        J = host(p.jvp(dev(u), dev(G), dev(v), eps=eps))
+        assert np.max(np.abs(J - K)) <= 2 * tol / eps
+
+
+@pytest.mark.parametrize("lam", [0.0, -3.0, 1e-120])
+def test_2d_bratu_lambda(lam):
+    n = 40
+    u, _ = _case2d("bratu2d", n, "plain")
+    F = host(jf().Problem("bratu2d", n, 1, lam=lam).residual(dev(u)))
+    G = fem.residual("bratu2d", u, lam, None, None)
+    assert np.max(np.abs(F - G)) <= _tol2d("bratu2d", u, n)
