@@ -51,6 +51,9 @@ struct CoarseArgs {
     LbfgsState* lb;
 };
 
+// method 1 (coarse_cg.cu)
+template <typename T>
+jfnk_status launch_coarse_cgqn(Prob prob, const CoarseArgs<T>& a, cudaStream_t st);
 template <typename T>
 jfnk_status launch_coarse(Prob prob, const CoarseArgs<T>& a, cudaStream_t st);
 // count instances (2D Bratu, same coarse grid as a0), args in device memory
