@@ -14,57 +14,25 @@ namespace jfnk {
 constexpr int kBThreads = 256;
 
 // ---------------------------------------------------------------------------
-// 2D element-residual kernel over (instance, row segment, row chunk) tiles
+// 2D element-residual kernel over (instance, strip, row chunk) tiles: one CTA a
+// tile (stencil_fx2d.cuh), a warp per part of its rows; the tile's x0 is the
+// strip.
 // ---------------------------------------------------------------------------
-// Persistent over the work list: CTA b processes tiles b, b + gridDim.x, ...
-// (gridDim.x = ntiles gives one tile per CTA).
+constexpr int kB2Threads = 256;
+
 template <typename T, Mode M>
-__global__ void __launch_bounds__(512) stencil2d_batched_kernel(const StencilArgs<T>* __restrict__ args,
-                                                                 const BTile* __restrict__ tiles, int ntiles) {
-    extern __shared__ unsigned char smem_raw[];
-    __shared__ double red_sm[32];
-    for (int k = blockIdx.x; k < ntiles; k += gridDim.x) {
-        const BTile t = tiles[k];
-        stencil2d_body<T, M>(args[t.inst], t.x0, t.y0, t.y1, t.txo, t.bid, t.nblk, smem_raw, red_sm);
-        __syncthreads();  // shared rows are reused by the next tile
-    }
-}
-
-template <>
-jfnk_status launch_stencil2d_batched<float>(Mode mode, const StencilArgs<float>* dev_args, const BTile* dev_tiles,
-                                            int ntiles, int bx, cudaStream_t st, int grid) {
-    if (ntiles <= 0) return JFNK_OK;
-    const int g = (grid > 0 && grid < ntiles) ? grid : ntiles;
-    const size_t smem = sizeof(float) * (2 * (bx + 1) + 4 * bx);
-#define JFNK_B2(MM) stencil2d_batched_kernel<float, MM><<<g, bx, smem, st>>>(dev_args, dev_tiles, ntiles)
-    switch (mode) {
-        case Mode::F: JFNK_B2(Mode::F); break;
-        case Mode::JV: JFNK_B2(Mode::JV); break;
-        case Mode::BMJ: JFNK_B2(Mode::BMJ); break;
-        case Mode::CHEB0: JFNK_B2(Mode::CHEB0); break;
-        case Mode::CHEB: JFNK_B2(Mode::CHEB); break;
-        case Mode::CHEBLAST: JFNK_B2(Mode::CHEBLAST); break;
-    }
-#undef JFNK_B2
-    JFNK_LAUNCH_CHECK();
-    return JFNK_OK;
-}
-
-// FP64: one CTA per (instance, strip, row chunk), element arithmetic in fixed
-// point (stencil_fx2d.cuh); the tile's x0 is the strip.
-template <Mode M>
-__global__ void __launch_bounds__(32 * kFx2Warps) fx2d_batched_kernel(const StencilArgs<double>* __restrict__ args,
-                                                                      const BTile* __restrict__ tiles) {
+__global__ void __launch_bounds__(kB2Threads) fx2d_batched_kernel(const StencilArgs<T>* __restrict__ args,
+                                                                  const BTile* __restrict__ tiles) {
     __shared__ double red_sm[32];
     const BTile t = tiles[blockIdx.x];
     fx2d_cta<Prob::BRATU2, M>(args[t.inst], t.x0, t.y0, t.y1, t.bid, t.nblk, red_sm);
 }
 
-template <>
-jfnk_status launch_stencil2d_batched<double>(Mode mode, const StencilArgs<double>* dev_args, const BTile* dev_tiles,
-                                             int ntiles, int, cudaStream_t st, int) {
+template <typename T>
+jfnk_status launch_stencil2d_batched(Mode mode, const StencilArgs<T>* dev_args, const BTile* dev_tiles, int ntiles,
+                                     int bx, cudaStream_t st) {
     if (ntiles <= 0) return JFNK_OK;
-#define JFNK_B2(MM) fx2d_batched_kernel<MM><<<ntiles, 32 * kFx2Warps, 0, st>>>(dev_args, dev_tiles)
+#define JFNK_B2(MM) fx2d_batched_kernel<T, MM><<<ntiles, bx, 0, st>>>(dev_args, dev_tiles)
     switch (mode) {
         case Mode::F: JFNK_B2(Mode::F); break;
         case Mode::JV: JFNK_B2(Mode::JV); break;
@@ -77,6 +45,10 @@ jfnk_status launch_stencil2d_batched<double>(Mode mode, const StencilArgs<double
     JFNK_LAUNCH_CHECK();
     return JFNK_OK;
 }
+template jfnk_status launch_stencil2d_batched<double>(Mode, const StencilArgs<double>*, const BTile*, int, int,
+                                                      cudaStream_t);
+template jfnk_status launch_stencil2d_batched<float>(Mode, const StencilArgs<float>*, const BTile*, int, int,
+                                                     cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // batched vector operations
@@ -86,7 +58,7 @@ __device__ __forceinline__ bool b_inner(const Grid& g, long long i) { return gri
 __device__ __forceinline__ void b_finish_eps(const BVec& d, double nrm) {
     if (!d.slot) return;
     double e = eps_formula(d.ep.mode, d.ep.n_unknowns, *d.ep.xstat, nrm);
-    double inv = e > 0.0 ? 1.0 / e : 0.0;
+    double inv = e > 0.0 ? 1.0 / (d.ep.unit ? e * nrm : e) : 0.0;  // unit: see RedOut::EPS_UNIT
     d.slot->e = e;
     d.slot->inv = inv;
     d.slot->ef = (float)e;
@@ -98,6 +70,39 @@ __device__ __forceinline__ uint64_t b_splitmix(uint64_t z) {
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
     return z ^ (z >> 31);
 }
+
+// A thread's running sum of |v| or v^2.  FP32 entries are summed as an FP32 pair
+// (Knuth's two-sum; squares as product and its FMA remainder), 44 bits or more
+// without the FP64 pipe, on which the conversion, product and sum of every
+// entry would run at 2 a clock and SM.
+template <typename T>
+struct BSum;
+template <>
+struct BSum<double> {
+    double s = 0.0;
+    __device__ void abs(double v) { s += fabs(v); }
+    __device__ void sq(double v) { s += v * v; }
+    __device__ double value() const { return s; }
+};
+template <>
+struct BSum<float> {
+    float h = 0.f, l = 0.f;
+    __device__ void add(float v, float rest) {
+        const float t = h + v, b = t - h;
+        l += ((h - (t - b)) + (v - b)) + rest;
+        h = t;
+    }
+    __device__ void abs(float v) { add(fabsf(v), 0.f); }
+    __device__ void sq(float v) {
+        const float p = v * v;
+        add(p, isfinite(p) ? fmaf(v, v, -p) : 0.f);
+    }
+    __device__ double value() const { return isfinite(h) ? (double)h + (double)l : (double)h; }
+};
+
+// b times the FP64 scalar whose FP32 parts are th + tl, rounded once
+__device__ __forceinline__ double b_scaled(double b, double ti, double, double) { return b * ti; }
+__device__ __forceinline__ float b_scaled(float b, double, float th, float tl) { return fmaf(b, th, b * tl); }
 
 template <typename T, BOp OP>
 __global__ void __launch_bounds__(kBThreads) bvec_kernel(const BVec* __restrict__ descs, const BItem* __restrict__ items) {
@@ -135,24 +140,28 @@ __global__ void __launch_bounds__(kBThreads) bvec_kernel(const BVec* __restrict_
             ((T*)d.y)[i] = v;
         }
     } else if (OP == BOp::STAT || OP == BOp::CHEB_START) {
-        double acc = 0.0;
+        BSum<T> acc;
         const double ti = (OP == BOp::CHEB_START) ? d.cheb->theta_inv : 0.0;
+        const T th = (T)ti, tl = (T)(ti - (double)th);
         for (long long i = i0; i < d.g.size; i += stride) {
             const bool in = b_inner(d.g, i);
             if (OP == BOp::STAT) {
                 if (!in) continue;
-                const double v = (double)((const T*)d.x)[i];
-                acc += d.what == 0 ? fabs(v) : v * v;
+                const T v = ((const T*)d.x)[i];
+                if (d.what == 0)
+                    acc.abs(v);
+                else
+                    acc.sq(v);
             } else {
                 const T bv = in ? ((const T*)d.x)[i] : T(0);
-                const T dv = (T)((double)bv * ti);
+                const T dv = b_scaled(bv, ti, th, tl);
                 ((T*)d.y)[i] = bv;        // r
                 ((T*)d.y2)[i] = dv;       // d
                 ((T*)d.x2)[i] = T(0);     // s (written through x2's address)
-                acc += (double)dv * (double)dv;
+                acc.sq(dv);
             }
         }
-        const double bs = block_sum(acc, sm);
+        const double bs = block_sum(acc.value(), sm);
         double tot = 0.0;
         if (grid_sum_last_seg(bs, d.partials, d.counter, &tot, sm, it.bid, it.nblk) && threadIdx.x == 0) {
             const double r = (OP == BOp::STAT && d.what == 0) ? tot : sqrt(tot);
@@ -292,10 +301,7 @@ __global__ void bscalar_kernel(BScalar op, const BScal* __restrict__ descs, int 
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     const BScal& d = descs[i];
-    if (op == BScalar::RATIO) {
-        const double b = *d.x2;
-        *d.out = b > 0.0 ? *d.x / b : 0.0;
-    } else if (op == BScalar::CHEB_TABLE) {
+    if (op == BScalar::CHEB_TABLE) {
         const double l = *d.x;
         if ((!(l > 0.0) || !isfinite(l)) && d.status) atomicOr(d.status, 2);
         double theta, c1, c2;

@@ -9,12 +9,11 @@
 
 namespace jfnk {
 
-// 2D row-segment tile of one instance
+// node rows [y0, y1) of a strip of node columns (stencil_fx2d.cuh) of one instance
 struct BTile {
     int inst;
-    int x0, y0, y1, txo;
-    int bid, nblk;  // index among the instance's CTAs, their count
-    int pad;
+    int x0, y0, y1;  // x0: the strip
+    int bid, nblk;   // index among the instance's CTAs, their count
 };
 
 // work item of a batched vector operation
@@ -64,7 +63,6 @@ enum class BOp : int {
 
 // Tiny per-instance scalar kernels (one thread per instance)
 enum class BScalar : int {
-    RATIO = 0,       // *out = *x / *x2    (lambda = ||Jv|| / ||v||)
     CHEB_TABLE = 1,  // cheb table from *x with [a, b] and degree m
     SET_EPS = 2,     // slot from a
 };
@@ -79,11 +77,10 @@ struct BScal {
     int* status;
 };
 
-// FP32: bx threads a CTA; grid > 0 (< ntiles): persistent launch of `grid` CTAs
-// looping over the tiles.  FP64: one CTA per tile, bx and grid unused.
+// one CTA of bx threads per tile
 template <typename T>
 jfnk_status launch_stencil2d_batched(Mode mode, const StencilArgs<T>* dev_args, const BTile* dev_tiles, int ntiles,
-                                     int bx, cudaStream_t st, int grid = 0);
+                                     int bx, cudaStream_t st);
 
 template <typename T>
 jfnk_status launch_bvec(BOp op, const BVec* dev_desc, const BItem* dev_items, int nitems, cudaStream_t st);

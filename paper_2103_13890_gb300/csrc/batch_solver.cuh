@@ -41,16 +41,15 @@ struct Arena {
     }
 };
 
-// Tiling of the batched FP32 2D kernel: threads per CTA, target CTA count of a
-// launch (sets the row-chunk length), persistent grid size (0: one CTA per tile).
+// Tiling of the batched 2D kernel: threads per CTA, warps a launch is cut into
+// (sets the row-chunk length).
 struct TileCfg {
-    int bx = 160;
-    int target = 608;
-    int grid = 0;
+    int bx = 32 * kFx2Warps;
+    int target = kFx2Slots64;
 };
 
 struct BCtx {
-    TileCfg tile;  // FP32 launches
+    TileCfg tile[2];  // [0] FP32, [1] FP64 launches
     std::vector<P*> ps;
     std::vector<double*> u;
     int B = 0;
@@ -64,6 +63,8 @@ struct BCtx {
     // cached V-cycle program
     std::vector<int> prog_set;
     cudaGraphExec_t graph = nullptr;
+    std::vector<long long> graph_nF;  // evaluations per instance and level of one replay
+    long long graph_launches = 0;
     ~BCtx() {
         if (graph) cudaGraphExecDestroy(graph);
     }
@@ -98,43 +99,44 @@ static D* stage(BCtx& b, Arena& A, const std::vector<D>& v, jfnk_status& err) {
     return ptr;
 }
 
-static std::vector<BItem> vec_items(const std::vector<long long>& sizes, int cap = 32) {
+// two arrays of one operation; uploaded at once, with one copy
+template <class D, class E>
+static void stage2(BCtx& b, Arena& A, const std::vector<D>& v, const std::vector<E>& w, const D*& dv, const E*& dw,
+                   jfnk_status& err) {
+    if (&A == &b.dyn && b.immediate) {
+        const size_t at = ((v.size() * sizeof(D)) + 255) & ~size_t(255);
+        std::vector<char> both(at + w.size() * sizeof(E));
+        memcpy(both.data(), v.data(), v.size() * sizeof(D));
+        memcpy(both.data() + at, w.data(), w.size() * sizeof(E));
+        const char* ptr = stage(b, A, both, err);
+        dv = reinterpret_cast<const D*>(ptr);
+        dw = reinterpret_cast<const E*>(ptr + at);
+        return;
+    }
+    dv = stage(b, A, v, err);
+    dw = stage(b, A, w, err);
+}
+
+// blocks per instance: about 8 entries a thread, and about 8 blocks per SM over
+// the launch, but no more than the dot products' scratch holds (kDotBlocks)
+static std::vector<BItem> vec_items(const std::vector<long long>& sizes) {
+    long long total = 0;
+    for (long long s : sizes) total += s;
+    const long long per = std::max(2048LL, (total + 8 * kNumSMs - 1) / (8 * kNumSMs));
     std::vector<BItem> it;
     for (int k = 0; k < (int)sizes.size(); ++k) {
-        long long nb = (sizes[k] + 255) / 256;
-        nb = std::max(1LL, std::min<long long>(nb, cap));
+        const long long nb = std::max(1LL, std::min<long long>((sizes[k] + per - 1) / per, kDotBlocks));
         for (int q = 0; q < nb; ++q) it.push_back(BItem{k, q, (int)nb, 0});
     }
     return it;
 }
 
-// tiles of the 2D kernel for grids g[k]: row segments of <= bx-1 nodes, row
-// chunks sized so that the launch has about `target` tiles
-constexpr int kBatchBX = 160;
-static std::vector<BTile> tiles_for(const std::vector<Grid>& gs, int bx = kBatchBX, int target = 608) {
-    long long rows = 0;
-    for (const Grid& g : gs) rows += (long long)g.ny * ((g.nx + bx - 2) / (bx - 1));
-    const int yc = (int)std::max(4LL, (rows + target - 1) / target);
-    std::vector<BTile> t;
-    for (int k = 0; k < (int)gs.size(); ++k) {
-        const Grid& g = gs[k];
-        const int segs = (g.nx + bx - 2) / (bx - 1);
-        const int txo = (g.nx + segs - 1) / segs;
-        const int ch = (g.ny + yc - 1) / yc;
-        const int nblk = segs * ch;
-        int bid = 0;
-        for (int c = 0; c < ch; ++c)
-            for (int sg = 0; sg < segs; ++sg)
-                t.push_back(BTile{k, sg * txo, c * yc, std::min(c * yc + yc, g.ny), txo, bid++, nblk, 0});
-    }
-    return t;
-}
-
-// FP64 tiles (stencil_fx2d.cuh): x0 is the strip of node columns
-static std::vector<BTile> tiles_fx2d(const std::vector<Grid>& gs) {
+// tiles of the 2D kernel for grids g[k]: rows per CTA so that the launch's warps
+// (`warps` a CTA) number about `slots`
+static std::vector<BTile> tiles_for(const std::vector<Grid>& gs, int warps, int slots) {
     long long total = 0;
     for (const Grid& g : gs) total += (long long)fx2d_strips(g.n) * g.ny;
-    const int rows = fx2d_cta_rows(total);
+    const int rows = fx2d_cta_rows(total, slots, warps);
     std::vector<BTile> t;
     for (int k = 0; k < (int)gs.size(); ++k) {
         const Grid& g = gs[k];
@@ -145,7 +147,7 @@ static std::vector<BTile> tiles_fx2d(const std::vector<Grid>& gs) {
         const int ch = (g.ny + rk - 1) / rk;
         for (int c = 0; c < ch; ++c)
             for (int s = 0; s < strips; ++s)
-                t.push_back(BTile{k, s, c * rk, std::min(c * rk + rk, g.ny), 0, c * strips + s, strips * ch, 0});
+                t.push_back(BTile{k, s, c * rk, std::min(c * rk + rk, g.ny), c * strips + s, strips * ch});
     }
     return t;
 }
@@ -157,13 +159,14 @@ static jfnk_status bstencil(BCtx& b, Arena& A, Mode m, const std::vector<int>& S
     std::vector<Grid> gs;
     for (int i : S) gs.push_back(b.ps[i]->lv[lvl_from_coarse].g);
     jfnk_status err = JFNK_OK;
-    const TileCfg& tc = b.tile;
-    const std::vector<BTile> tiles = sizeof(T) == 8 ? tiles_fx2d(gs) : tiles_for(gs, tc.bx, tc.target);
-    const StencilArgs<T>* da = stage(b, A, args, err);
-    const BTile* dt = stage(b, A, tiles, err);
+    const TileCfg& tc = b.tile[sizeof(T) == 8 ? 1 : 0];
+    const std::vector<BTile> tiles = tiles_for(gs, tc.bx / 32, tc.target);
+    const StencilArgs<T>* da = nullptr;
+    const BTile* dt = nullptr;
+    stage2(b, A, args, tiles, da, dt, err);
     if (err != JFNK_OK) return err;
     if (b.dry) return JFNK_OK;
-    return launch_stencil2d_batched<T>(m, da, dt, (int)tiles.size(), tc.bx, b.st, tc.grid);
+    return launch_stencil2d_batched<T>(m, da, dt, (int)tiles.size(), tc.bx, b.st);
 }
 
 template <typename T>
@@ -171,8 +174,9 @@ static jfnk_status bvec(BCtx& b, Arena& A, BOp op, const std::vector<BVec>& d, c
     if (d.empty()) return JFNK_OK;
     jfnk_status err = JFNK_OK;
     const std::vector<BItem> items = vec_items(sizes);
-    const BVec* dd = stage(b, A, d, err);
-    const BItem* di = stage(b, A, items, err);
+    const BVec* dd = nullptr;
+    const BItem* di = nullptr;
+    stage2(b, A, d, items, dd, di, err);
     if (err != JFNK_OK) return err;
     if (b.dry) return JFNK_OK;
     return launch_bvec<T>(op, dd, di, (int)items.size(), b.st);
@@ -430,12 +434,22 @@ static jfnk_status bvcycle_run(BCtx& b, const std::vector<int>& act) {
             cudaStream_t keep = b.st;
             b.st = lp.cap_stream;
             for (int i = 0; i < b.B; ++i) memcpy(&nF0[i * JFNK_MAX_LEVELS], b.ps[i]->nF, sizeof(long long) * JFNK_MAX_LEVELS);
+            const long long l0 = g_launches;
             JFNK_CUDA_TRY(cudaStreamBeginCapture(lp.cap_stream, cudaStreamCaptureModeThreadLocal));
             s = bvcycle<T>(b, A, act);
             cudaGraph_t g = nullptr;
             cudaError_t e = cudaStreamEndCapture(lp.cap_stream, &g);
             b.st = keep;
-            for (int i = 0; i < b.B; ++i) memcpy(b.ps[i]->nF, &nF0[i * JFNK_MAX_LEVELS], sizeof(long long) * JFNK_MAX_LEVELS);
+            // the captured launches have not run: what a replay evaluates and launches
+            b.graph_nF.assign(nF0.size(), 0);
+            for (int i = 0; i < b.B; ++i)
+                for (int l = 0; l < JFNK_MAX_LEVELS; ++l) {
+                    const size_t q = (size_t)i * JFNK_MAX_LEVELS + l;
+                    b.graph_nF[q] = b.ps[i]->nF[l] - nF0[q];
+                    b.ps[i]->nF[l] = nF0[q];
+                }
+            b.graph_launches = g_launches - l0;
+            g_launches = l0;
             if (s != JFNK_OK) {
                 if (e == cudaSuccess && g) cudaGraphDestroy(g);
                 A.replay = false;
@@ -448,11 +462,9 @@ static jfnk_status bvcycle_run(BCtx& b, const std::vector<int>& act) {
             A.off = 0;
         }
         JFNK_CUDA_TRY(cudaGraphLaunch(b.graph, b.st));
-        // count the evaluations of the replayed cycle (dry bookkeeping pass)
-        b.dry = true;
-        A.off = 0;
-        s = bvcycle<T>(b, A, act);
-        b.dry = false;
+        for (int i = 0; i < b.B; ++i)
+            for (int l = 0; l < JFNK_MAX_LEVELS; ++l) b.ps[i]->nF[l] += b.graph_nF[(size_t)i * JFNK_MAX_LEVELS + l];
+        g_launches += b.graph_launches;
     } else {
         s = bvcycle<T>(b, A, act);
     }
@@ -535,11 +547,12 @@ static jfnk_status bjv64(BCtx& b, const std::vector<int>& S, const std::vector<c
     std::vector<Grid> gs;
     for (int i : S) gs.push_back(b.ps[i]->lv[b.ps[i]->L].g);
     jfnk_status err = JFNK_OK;
-    const std::vector<BTile> tiles = tiles_fx2d(gs);
+    const TileCfg& tc = b.tile[1];
+    const std::vector<BTile> tiles = tiles_for(gs, tc.bx / 32, tc.target);
     const StencilArgs<double>* da = stage(b, b.dyn, args, err);
     const BTile* dt = stage(b, b.dyn, tiles, err);
     JFNK_TRY(err);
-    return launch_stencil2d_batched<double>(Mode::JV, da, dt, (int)tiles.size(), 0, b.st);
+    return launch_stencil2d_batched<double>(Mode::JV, da, dt, (int)tiles.size(), tc.bx, b.st);
 }
 
 // F_i = F(x_i), A_i = A(x_i) (FP64, finest) and ||F_i|| into res slot 0
@@ -559,11 +572,12 @@ static jfnk_status bresidual64(BCtx& b, const std::vector<int>& S, const std::ve
         p.nFplain[p.L]++;
     }
     jfnk_status err = JFNK_OK;
-    const std::vector<BTile> tiles = tiles_fx2d(gs);
+    const TileCfg& tc = b.tile[1];
+    const std::vector<BTile> tiles = tiles_for(gs, tc.bx / 32, tc.target);
     const StencilArgs<double>* da = stage(b, b.dyn, args, err);
     const BTile* dt = stage(b, b.dyn, tiles, err);
     JFNK_TRY(err);
-    JFNK_TRY(launch_stencil2d_batched<double>(Mode::F, da, dt, (int)tiles.size(), 0, b.st));
+    JFNK_TRY(launch_stencil2d_batched<double>(Mode::F, da, dt, (int)tiles.size(), tc.bx, b.st));
     std::vector<const void*> xv(F.begin(), F.end());
     std::vector<double*> outs;
     for (int i : S) outs.push_back(b.res + (size_t)i * kResStride);
@@ -668,11 +682,12 @@ static jfnk_status bsetup(BCtx& b, const std::vector<int>& S, int newton_step) {
         std::vector<EpsParams> ep;
         std::vector<EpsSlot*> slots;
         std::vector<double*> n0;
-        std::vector<BVec> start, sc;
+        std::vector<BVec> start;
         for (int i : R) {
             Level& L = b.ps[i]->lv[c];
             pv.push_back(L.pv);
             ep.push_back(eps_params(*b.ps[i], c, o.eps_mode_pc));
+            ep.back().unit = 1;
             slots.push_back(L.eps_aux);
             n0.push_back(L.nrm0);
             BVec v = bv0();
@@ -680,62 +695,33 @@ static jfnk_status bsetup(BCtx& b, const std::vector<int>& S, int newton_step) {
             v.y = L.pv;
             v.key = o.seed + (uint64_t)c * 0xD1B54A32D192ED03ULL;
             start.push_back(v);
-            BVec w = bv0();
-            w.g = L.g;
-            w.x = w.y = L.pv;
-            w.dsc = L.nrm0;
-            sc.push_back(w);
         }
         if (newton_step == 0 || !b.ps[R[0]]->lv[c].pv_valid) JFNK_TRY(bvec<T>(b, A, BOp::SPLITMIX, start, z));
-        // v <- v / ||v||
         JFNK_TRY(bstat(b, R, c, 1, pv, n0, slots, ep, sizeof(T) == 8));
-        JFNK_TRY(bvec<T>(b, A, BOp::SCALE_INV_T, sc, z));
     }
-    // one iteration on level c for instances Ra: w = J v (FD), lambda = ||w|| / ||v||,
-    // v <- w / ||w||
+    // one iteration on level c for instances Ra along unit vectors, without
+    // normalisation passes (RedOut::EPS_UNIT, as in jfnk_solve): the action's own
+    // output norm is lambda and its output the next v
     auto iterate = [&](int c, const std::vector<int>& Ra) -> jfnk_status {
-        std::vector<const void*> pv;
-        std::vector<double*> n0;
-        std::vector<EpsSlot*> slots;
-        std::vector<EpsParams> ep;
-        std::vector<BVec> sc;
-        std::vector<long long> z;
         std::vector<StencilArgs<T>> args;
-        std::vector<BScal> rat;
         for (int i : Ra) {
             P& p = *b.ps[i];
             Level& L = p.lv[c];
-            pv.push_back(L.pv);
-            n0.push_back(L.nrm0);
-            slots.push_back(L.eps_aux);
-            ep.push_back(eps_params(p, c, o.eps_mode_pc));
-            BVec v = bv0();
-            v.g = L.g;
-            v.x = v.y = L.pw;
-            v.dsc = L.nrm1;
-            sc.push_back(v);
-            z.push_back(L.g.size);
             StencilArgs<T> a = base_args<T>(p, c);
             a.u = as<T>(L.x);
             a.v = as<T>(L.pv);
             a.eps = L.eps_aux;
             a.Au = as<T>(L.Ax);
             a.out = as<T>(L.pw);
-            a.red = RedOut::NORM;
-            a.red_norm = L.nrm1;
+            a.red = RedOut::EPS_UNIT;
+            a.red_norm = L.lam;
+            a.red_eps = L.eps_aux;
+            a.epsp = eps_params(p, c, o.eps_mode_pc);
+            a.epsp.unit = 1;
             args.push_back(a);
             p.nF[c]++;
-            BScal r;
-            memset(&r, 0, sizeof(r));
-            r.out = L.lam;
-            r.x = L.nrm1;
-            r.x2 = L.nrm0;
-            rat.push_back(r);
         }
-        JFNK_TRY(bstat(b, Ra, c, 1, pv, n0, slots, ep, sizeof(T) == 8));
         JFNK_TRY(bstencil<T>(b, A, Mode::JV, Ra, c, args));
-        JFNK_TRY(bscalar(b, A, BScalar::RATIO, rat));
-        JFNK_TRY(bvec<T>(b, A, BOp::SCALE_INV_T, sc, z));
         for (int i : Ra) std::swap(b.ps[i]->lv[c].pv, b.ps[i]->lv[c].pw);
         return JFNK_OK;
     };
@@ -1040,11 +1026,11 @@ static jfnk_status bfgmres(BCtx& b, const std::vector<int>& S, const std::vector
 
 // ---------------------------------------------------------------------------
 // Tile autotuner: the first batched solve of a given mix of grid sizes times
-// the residual kernel of the finest grids for a few (threads per CTA, target
-// CTA count, persistent grid) candidates with CUDA events and keeps the
-// fastest, per precision.  Results are cached in the process and, when the
-// environment variable JFNK_TUNE_CACHE names a file, in that file (one line
-// per key: "key bx target grid ms").
+// the FP32 residual kernel of the finest grids for a few (threads per CTA, warps
+// a launch is cut into) candidates with CUDA events and keeps the fastest.
+// Results are cached in the process and, when the environment variable
+// JFNK_TUNE_CACHE names a file, in that file (one line per key:
+// "key bx target 0 ms").
 static std::map<std::string, TileCfg>& tile_cache() {
     static std::map<std::string, TileCfg> m;
     static bool loaded = false;
@@ -1056,8 +1042,10 @@ static std::map<std::string, TileCfg>& tile_cache() {
             if (f) {
                 char key[512];
                 TileCfg c;
+                int unused;
                 double ms;
-                while (fscanf(f, "%511s %d %d %d %lf", key, &c.bx, &c.target, &c.grid, &ms) == 5) m[key] = c;
+                while (fscanf(f, "%511s %d %d %d %lf", key, &c.bx, &c.target, &unused, &ms) == 5)
+                    if (c.bx >= 32 && c.bx <= 256 && c.bx % 32 == 0 && c.target > 0) m[key] = c;
                 fclose(f);
             }
         }
@@ -1071,7 +1059,7 @@ static void tile_cache_store(const std::string& key, const TileCfg& c, double ms
     if (!path) return;
     FILE* f = fopen(path, "a");
     if (!f) return;
-    fprintf(f, "%s %d %d %d %.6f\n", key.c_str(), c.bx, c.target, c.grid, ms);
+    fprintf(f, "%s %d %d 0 %.6f\n", key.c_str(), c.bx, c.target, ms);
     fclose(f);
 }
 
@@ -1080,7 +1068,7 @@ static jfnk_status tune_tiles(BCtx& b) {
     std::vector<int> ns;
     for (P* p : b.ps) ns.push_back(p->lv[p->L].g.n);
     std::sort(ns.begin(), ns.end());
-    std::string key = "bratu2d_f32";
+    std::string key = "bratu2d_strips_f32";
     for (size_t k = 0; k < ns.size();) {
         size_t e = k;
         while (e < ns.size() && ns[e] == ns[k]) ++e;
@@ -1089,7 +1077,7 @@ static jfnk_status tune_tiles(BCtx& b) {
     }
     auto it = tile_cache().find(key);
     if (it != tile_cache().end()) {
-        b.tile = it->second;
+        b.tile[0] = it->second;
         return JFNK_OK;
     }
     std::vector<int> all(b.B);
@@ -1104,42 +1092,35 @@ static jfnk_status tune_tiles(BCtx& b) {
         a.out = as<T>(p.lv[p.L].t);
         args.push_back(a);
     }
-    int dev = 0, sms = kNumSMs;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaEvent_t e0, e1;
     JFNK_CUDA_TRY(cudaEventCreate(&e0));
     JFNK_CUDA_TRY(cudaEventCreate(&e1));
     TileCfg best;
     double best_ms = -1.0;
     jfnk_status err = JFNK_OK;
-    for (int bx : {128, 160, 256}) {
-        for (int target : {304, 608, 1216}) {
-            const std::vector<BTile> tiles = tiles_for(gs, bx, target);
+    for (int bx : {64, 128, 256}) {
+        for (int target : {kFx2Slots32 / 2, kFx2Slots32, 2 * kFx2Slots32}) {
+            const std::vector<BTile> tiles = tiles_for(gs, bx / 32, target);
             const StencilArgs<T>* da = stage(b, b.dyn, args, err);
             const BTile* dt = stage(b, b.dyn, tiles, err);
             JFNK_TRY(err);
-            const int per_sm = std::max(1, 2048 / bx);
-            for (int grid : {0, sms * per_sm}) {
-                TileCfg c{bx, target, grid};
-                JFNK_TRY(launch_stencil2d_batched<T>(Mode::F, da, dt, (int)tiles.size(), bx, b.st, grid));
-                JFNK_CUDA_TRY(cudaEventRecord(e0, b.st));
-                for (int r = 0; r < 3; ++r)
-                    JFNK_TRY(launch_stencil2d_batched<T>(Mode::F, da, dt, (int)tiles.size(), bx, b.st, grid));
-                JFNK_CUDA_TRY(cudaEventRecord(e1, b.st));
-                JFNK_CUDA_TRY(cudaEventSynchronize(e1));
-                float ms = 0.f;
-                JFNK_CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
-                if (best_ms < 0.0 || ms < best_ms) {
-                    best_ms = ms;
-                    best = c;
-                }
+            JFNK_TRY(launch_stencil2d_batched<T>(Mode::F, da, dt, (int)tiles.size(), bx, b.st));
+            JFNK_CUDA_TRY(cudaEventRecord(e0, b.st));
+            for (int r = 0; r < 3; ++r)
+                JFNK_TRY(launch_stencil2d_batched<T>(Mode::F, da, dt, (int)tiles.size(), bx, b.st));
+            JFNK_CUDA_TRY(cudaEventRecord(e1, b.st));
+            JFNK_CUDA_TRY(cudaEventSynchronize(e1));
+            float ms = 0.f;
+            JFNK_CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
+            if (best_ms < 0.0 || ms < best_ms) {
+                best_ms = ms;
+                best = TileCfg{bx, target};
             }
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    b.tile = best;
+    b.tile[0] = best;
     tile_cache_store(key, best, best_ms / 3.0);
     return JFNK_OK;
 }

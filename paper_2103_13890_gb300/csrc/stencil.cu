@@ -200,8 +200,8 @@ static jfnk_status launch_stencil_impl(Prob prob, Mode mode, const StencilArgs<T
     if (prob == Prob::BEAM3) return launch_beam<T>(mode, a, st);
     if constexpr (sizeof(T) == 8) {
         if (!is_2d(prob) && fx3d_use(a, mode)) return launch_fx3d(prob, mode, a, st);
-        if (fx2d_use(prob, a, mode)) return launch_fx2d(prob, mode, a, st);
     }
+    if (fx2d_use<T>(prob, a, mode)) return launch_fx2d<T>(prob, mode, a, st);
     if (!is_2d(prob) && ep3d_use(a)) return launch_ep3d<T>(prob, mode, false, a, st);
     if (!is_2d(prob) && a.face != nullptr && a.v2_threads >= 0 && v2_applicable(a.g)) {
         if constexpr (sizeof(T) == 4) {

@@ -237,8 +237,9 @@ static bool overlap(const void* p, const void* q, size_t bytes) {
     return p && q && x < y + bytes && y < x + bytes;
 }
 
-bool fx_outputs_alias(const StencilArgs<double>& a, Mode mode) {
-    const size_t bytes = sizeof(double) * (size_t)a.g.size;
+template <typename T>
+bool fx_outputs_alias(const StencilArgs<T>& a, Mode mode) {
+    const size_t bytes = sizeof(T) * (size_t)a.g.size;
     const void* in[2] = {a.u, mode == Mode::F ? nullptr : a.v};
     const void* out[3] = {a.out, nullptr, nullptr};
     if (mode == Mode::CHEB || mode == Mode::CHEBLAST) {
@@ -253,6 +254,8 @@ bool fx_outputs_alias(const StencilArgs<double>& a, Mode mode) {
             if (overlap(i, o, bytes)) return true;
     return false;
 }
+template bool fx_outputs_alias<double>(const StencilArgs<double>&, Mode);
+template bool fx_outputs_alias<float>(const StencilArgs<float>&, Mode);
 
 bool fx3d_use(const StencilArgs<double>& a, Mode mode) {
     return a.fx.ctas > 0 && fx_scale_ok(a.node_scale) && !fx_outputs_alias(a, mode);

@@ -12,7 +12,8 @@ FxTiling fx3d_tiling(const Grid& g);
 
 // True when an output of the action overlaps u or v, whose neighbouring values
 // the one-launch kernels still read while others write.
-bool fx_outputs_alias(const StencilArgs<double>& a, Mode mode);
+template <typename T>
+bool fx_outputs_alias(const StencilArgs<T>& a, Mode mode);
 
 // True when the fixed-point kernel takes this FP64 call: a.fx is set, and the
 // outputs are apart from the vectors whose neighbouring values other threads

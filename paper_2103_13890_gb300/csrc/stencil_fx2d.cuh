@@ -1,4 +1,4 @@
-// FP64 residual kernels of the 2D problems with the element arithmetic in
+// Residual kernels of the 2D problems; in FP64 the element arithmetic runs in
 // 64-bit fixed point (fx64.cuh).
 //
 // A warp owns a strip of 30 node columns and marches along y on its own: lane l
@@ -23,15 +23,18 @@ namespace jfnk {
 
 constexpr int kFx2Strip = 30;     // node columns a warp completes
 constexpr int kFx2Warps = 4;      // per CTA
-constexpr int kFx2Slots = 152 * 20;  // resident warps (96 registers a thread)
+// warps a launch is cut into, about what is resident: FP64 96 registers a thread
+constexpr int kFx2Slots64 = 152 * 20, kFx2Slots32 = 152 * 40;
 
 __host__ __device__ inline int fx2d_strips(int n) { return (n - 1 + kFx2Strip - 1) / kFx2Strip; }
 
-// True when the kernels take this FP64 call: outputs apart from the vectors
-// whose neighbouring values other lanes still read, and no node factor.
-bool fx2d_use(Prob prob, const StencilArgs<double>& a, Mode mode);
+// True when the kernels take this call: outputs apart from the vectors whose
+// neighbouring values other lanes still read, and (FP64) no node factor.
+template <typename T>
+bool fx2d_use(Prob prob, const StencilArgs<T>& a, Mode mode);
 
-jfnk_status launch_fx2d(Prob prob, Mode mode, const StencilArgs<double>& a, cudaStream_t st);
+template <typename T>
+jfnk_status launch_fx2d(Prob prob, Mode mode, const StencilArgs<T>& a, cudaStream_t st);
 
 #ifdef __CUDACC__
 
@@ -150,9 +153,70 @@ __device__ __forceinline__ void fx2d_warp(const StencilArgs<double>& a, int stri
     }
 }
 
-// A CTA's part: node rows [y0, y1) of a strip, shared out among its warps.
+// The same in FP32, element arithmetic in FP32.  Bound by instruction
+// issue: 146 instructions an element at 67 % of the issue slots on 4097^2 nodes
+// (fetching rows 2 to 4 ahead instead of 1 changed nothing).  Residual against
+// the row-segment kernel: 1025^2 14.5 -> 10.3 us, 2049^2 37.1 -> 25.0 us, 4097^2
+// 127 -> 101 us.
 template <Prob P, Mode M>
-__device__ __forceinline__ void fx2d_cta(const StencilArgs<double>& a, int strip, int y0, int y1, unsigned int bid,
+__device__ __forceinline__ void fx2d_warp(const StencilArgs<float>& a, int strip, int y0, int y1, float& red) {
+    const unsigned int all = 0xffffffffu;
+    const int n = a.g.n;
+    const int lane = threadIdx.x & 31;
+    const int x = strip * kFx2Strip + lane;
+    const bool col = x <= n;
+    const bool inner_x = x > 0 && x < n;
+    const bool out_x = col && (lane == 0 ? x == 0 : lane < 31 || x == n);
+    float eps = 0.f, inv_eps = 0.f;
+    if (M != Mode::F) {
+        eps = eps_of<float>(a.eps);
+        inv_eps = inv_eps_of<float>(a.eps);
+    }
+    ChebK<float> ck = {0.f, 0.f, 0.f};
+    if (M == Mode::CHEB0 || M == Mode::CHEB || M == Mode::CHEBLAST) ck = cheb_of<float>(a.cheb, a.cheb_step);
+    float ru = 0.f, rv = 0.f;
+    auto fetch = [&](int y) {
+        if (!col || y < 0 || y > n) return;
+        const long long i = JFNK_IDX((long long)y * a.g.sy + x, a.g.size);
+        ru = a.u[i];
+        if (M != Mode::F) rv = (inner_x && y > 0 && y < n) ? a.v[i] : 0.f;
+    };
+    float p[4] = {0.f, 0.f, 0.f, 0.f}, carry[2] = {0.f, 0.f};
+    auto row = [&](float* q) {
+        q[0] = M != Mode::F ? ru + eps * rv : ru;
+        q[1] = __shfl_down_sync(all, q[0], 1);
+    };
+    fetch(y0 - 1);
+    row(p);
+    fetch(y0);
+    for (int j = y0 - 1; j < y1; ++j) {
+        row(p + 2);
+        fetch(j + 2);
+        const bool out = out_x && j >= y0, inner = out && inner_x && j > 0 && j < n;
+        const long long idx = (long long)j * a.g.sy + x;
+        EpiIn1<float> e;
+        if (inner) epi1_load<float, M>(a, idx, e);
+        float r[4];
+        if (P == Prob::MINSURF2)
+            elem_minsurf2<float>(p, a.lh, r);
+        else
+            elem_bratu2<float>(p, a.lh, r);
+        // (rows and columns outside the grid only feed nodes that are not inner)
+        const float left = __shfl_up_sync(all, carry[1] + r[1], 1);
+        if (inner)
+            epilogue_pf<float, M>(a, idx, true, (left + (carry[0] + r[0])) * a.node_scale, inv_eps, ck, e, red);
+        else if (out)
+            epilogue<float, M>(a, idx, false, 0.f, 0.f, ck, red);
+        carry[0] = r[2];
+        carry[1] = r[3];
+        p[0] = p[2];
+        p[1] = p[3];
+    }
+}
+
+// A CTA's part: node rows [y0, y1) of a strip, shared out among its warps.
+template <Prob P, Mode M, typename T>
+__device__ __forceinline__ void fx2d_cta(const StencilArgs<T>& a, int strip, int y0, int y1, unsigned int bid,
                                          unsigned int nb, double* red_sm) {
     const int warps = blockDim.x >> 5, w = threadIdx.x >> 5;
     const int per = (y1 - y0 + warps - 1) / warps;
@@ -165,9 +229,9 @@ __device__ __forceinline__ void fx2d_cta(const StencilArgs<double>& a, int strip
 
 // Rows a CTA takes so that `rows` (strips x node rows, over all grids of a
 // launch) fill the resident warps once.
-inline int fx2d_cta_rows(long long rows) {
-    const long long per = (rows + kFx2Slots - 1) / kFx2Slots;
-    return kFx2Warps * (int)(per < 1 ? 1 : per);
+inline int fx2d_cta_rows(long long rows, int slots, int warps = kFx2Warps) {
+    const long long per = (rows + slots - 1) / slots;
+    return warps * (int)(per < 1 ? 1 : per);
 }
 
 }  // namespace jfnk
