@@ -164,6 +164,97 @@ __host__ __device__ __forceinline__ void elem_nd3(const T u[8], T kap, T r[8]) {
     r[6] = f0_11 - f1_11; r[7] = f0_11 + f1_11;
 }
 
+// The same element for kernels that march along z, in 131 operations a layer:
+// the x/y butterflies of a face's corner values are shared by the elements on
+// both sides, and on the test side the two elements' face modes are added
+// before the x/y butterflies.  No mode is scaled by itself: with the gradients
+// taken over A, the powers of A enter the butterflies as multiply-adds, and the
+// common factors 1/8 (gradient), 1/64 (coefficient, formed as 64 + (8u)^2) and
+// A^2 = 1/3 are left to the node factor (kNd3FaceScale).
+constexpr double kNd3FaceScale = 1.0 / (8.0 * 64.0 * 3.0);
+
+// face corners q[a + 2b] -> modes m[p + 2q] (8 operations)
+template <typename T>
+__host__ __device__ __forceinline__ void nd3_face(const T q[4], T m[4]) {
+    const T p0 = q[0] + q[1], d0 = q[1] - q[0], p1 = q[2] + q[3], d1 = q[3] - q[2];
+    m[0] = p0 + p1;
+    m[2] = p1 - p0;
+    m[1] = d0 + d1;
+    m[3] = d1 - d0;
+}
+// lower and upper face modes a, b -> test-side face modes lo, up (the modes
+// p + 2q = 3 over A); lo[0] is returned negated
+template <typename T, bool KAPPA>
+__host__ __device__ __forceinline__ void nd3_faces(const T a[4], const T b[4], T kap, T lo[4], T up[4]) {
+    const T A = T(0.57735026918962576451), B = T(-0.57735026918962576451);
+    const T M000 = a[0] + b[0], M001 = b[0] - a[0], M100 = a[1] + b[1], M101 = b[1] - a[1];
+    const T M010 = a[2] + b[2], M011 = b[2] - a[2], M110 = a[3] + b[3], M111 = b[3] - a[3];
+    // z signs; index [sz]
+    const T P0z[2] = {madd(M001, B, M000), madd(M001, A, M000)}, Y0z[2] = {madd(M011, B, M010), madd(M011, A, M010)};
+    const T X0z[2] = {madd(M101, B, M100), madd(M101, A, M100)}, X1z[2] = {madd(M111, B, M110), madd(M111, A, M110)};
+    const T Z0x[2] = {madd(M101, B, M001), madd(M101, A, M001)}, Z1x[2] = {madd(M111, B, M011), madd(M111, A, M011)};
+    T GX[2][2], GY[2][2], GZ[2][2], c[2][2][2];  // [sy][sz], [sx][sz], [sx][sy]; [sx][sy][sz]
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        GX[0][k] = madd(X1z[k], B, X0z[k]);
+        GX[1][k] = madd(X1z[k], A, X0z[k]);
+        GY[0][k] = madd(X1z[k], B, Y0z[k]);
+        GY[1][k] = madd(X1z[k], A, Y0z[k]);
+        GZ[k][0] = madd(Z1x[k], B, Z0x[k]);
+        GZ[k][1] = madd(Z1x[k], A, Z0x[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const T p = madd(Y0z[k], j ? A : B, P0z[k]);
+            const T um = madd(GX[j][k], B, p), up8 = madd(GX[j][k], A, p);  // 8 u
+            c[0][j][k] = madd(um, um, T(64));
+            c[1][j][k] = madd(up8, up8, T(64));
+        }
+    T FX[2][2], FY[2][2], FZ[2][2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            FX[i][j] = GX[i][j] * (c[1][i][j] + c[0][i][j]);
+            FY[i][j] = GY[i][j] * (c[i][1][j] + c[i][0][j]);
+            FZ[i][j] = GZ[i][j] * (c[i][j][1] + c[i][j][0]);
+        }
+    T R100, R010, R001, X10, X01, X11, Y10, Y01, Y11, Z10, Z01, Z11;
+    h2_adj(FX, R100, X10, X01, X11);  // X_qr
+    h2_adj(FY, R010, Y10, Y01, Y11);  // Y_pr
+    h2_adj(FZ, R001, Z10, Z01, Z11);  // Z_pq
+    T S110 = X10 + Y10, S101 = X01 + Z10, S011 = Y01 + Z01, S111 = X11 + Y11 + Z11;
+    if (KAPPA) {
+        R100 = R100 * kap;
+        R010 = R010 * kap;
+        R001 = R001 * kap;
+        S110 = S110 * kap;
+        S101 = S101 * kap;
+        S011 = S011 * kap;
+        S111 = S111 * kap;
+    }
+    lo[0] = up[0] = R001;
+    lo[2] = madd(S011, B, R010);
+    up[2] = madd(S011, A, R010);
+    lo[1] = madd(S101, B, R100);
+    up[1] = madd(S101, A, R100);
+    lo[3] = madd(S111, B, S110);
+    up[3] = madd(S111, A, S110);
+}
+// a face's summed test-side modes -> its corner contributions r[a + 2b]
+template <typename T>
+__host__ __device__ __forceinline__ void nd3_face_adj(const T m[4], T r[4]) {
+    const T A = T(0.57735026918962576451), B = T(-0.57735026918962576451);
+    const T f00 = m[0] - m[2], f01 = m[0] + m[2];                      // x mode 0, b = 0 / 1
+    const T f10 = madd(m[3], B, m[1]), f11 = madd(m[3], A, m[1]);      // x mode 1
+    r[0] = f00 - f10;
+    r[1] = f00 + f10;
+    r[2] = f01 - f11;
+    r[3] = f01 + f11;
+}
+
 // ---------------------------------------------------------------------------
 // 3D vector-Jacobian product of the coefficient problem (adjoint).
 //   F_i = sum_e kap_e int_e (1+u^2) grad u . grad phi_i - int phi_i, so for a

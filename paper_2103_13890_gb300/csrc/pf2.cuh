@@ -49,6 +49,10 @@ __device__ __forceinline__ pf2 operator*(pf2 a, pf2 b) {
     return r;
 }
 __device__ __forceinline__ pf2 operator-(pf2 a) { return pf2(0.0) - a; }
+__device__ __forceinline__ pf2& operator+=(pf2& a, pf2 b) {
+    a = a + b;
+    return a;
+}
 // a b + c with one rounding per component
 __device__ __forceinline__ pf2 madd(pf2 a, pf2 b, pf2 c) {
     pf2 r;

@@ -36,6 +36,7 @@
 #include "stencil_ep.cuh"
 #include "stencil_fx.cuh"
 #include "stencil_fx2d.cuh"
+#include "stencil_t3.cuh"
 #include "beam.cuh"
 #include "stencil_v2.cuh"
 #include <algorithm>
@@ -92,6 +93,7 @@ struct Level {
     ChebTable* cheb;
     bool pv_valid;
     FxTiling fx;  // FP64 3D: tiling of the fixed-point kernel
+    FxTiling t3;  // FP32 3D: tiling of the z-marching kernel
 };
 
 }  // namespace jfnk
@@ -238,9 +240,16 @@ static size_t plan(P& p, char* base, const jfnk_options* o) {
     if (const char* e = getenv("JFNK_ZM3D_MIN_N_F32")) p.zm_min_n32 = atoi(e);
     if (const char* e = getenv("JFNK_EP3D_CLUSTER_MIN_N")) p.cl_min_n32 = atoi(e);
     if (const char* e = getenv("JFNK_EP3D_CLUSTER_MAX_N")) p.cl_max_n32 = atoi(e);
-    // an explicit choice of another FP64 kernel stands
+    // an explicit choice of another kernel stands
     const bool fx = !getenv("JFNK_EP3D_MAX_N_F64") && !getenv("JFNK_ZM3D_MIN_N_F64") && !getenv("JFNK_V2_THREADS_F64");
-    for (Level& L : p.lv) L.fx = fx ? fx3d_tiling(L.g) : FxTiling{};
+    bool t3 = true;
+    for (const char* e : {"JFNK_EP3D_MAX_N_F32", "JFNK_ZM3D_MIN_N_F32", "JFNK_V2_THREADS_F32", "JFNK_V3_F32",
+                          "JFNK_EP3D_CLUSTER_MIN_N", "JFNK_EP3D_CLUSTER_MAX_N"})
+        t3 = t3 && !getenv(e);
+    for (Level& L : p.lv) {
+        L.fx = fx ? fx3d_tiling(L.g) : FxTiling{};
+        L.t3 = t3 ? t3d_tiling(L.g) : FxTiling{};
+    }
     // the cluster kernels' attributes are set here, outside any graph capture
     if (p.cl_max_n32 > 0 && !ep3d_cluster_init()) p.cl_max_n32 = 0;
     if (const char* e = getenv("JFNK_V2_THREADS_F64")) p.v2_threads64 = atoi(e);
@@ -379,6 +388,7 @@ static StencilArgs<T> base_args(P& p, int l) {
     a.v2_threads = sizeof(T) == 8 ? p.v2_threads64 : p.v2_threads32;
     a.v3 = sizeof(T) == 4 ? p.v3_f32 : 0;
     if (sizeof(T) == 8) a.fx = L.fx;
+    if (sizeof(T) == 4) a.t3 = L.t3;
     return a;
 }
 

@@ -21,6 +21,7 @@
 #include "stencil_ep.cuh"
 #include "stencil_fx.cuh"
 #include "stencil_fx2d.cuh"
+#include "stencil_t3.cuh"
 #include "beam.cuh"
 #include "stencil_v2.cuh"
 #include "reduce.cuh"
@@ -200,6 +201,9 @@ static jfnk_status launch_stencil_impl(Prob prob, Mode mode, const StencilArgs<T
     if (prob == Prob::BEAM3) return launch_beam<T>(mode, a, st);
     if constexpr (sizeof(T) == 8) {
         if (!is_2d(prob) && fx3d_use(a, mode)) return launch_fx3d(prob, mode, a, st);
+    }
+    if constexpr (sizeof(T) == 4) {
+        if (!is_2d(prob) && t3d_use(a, mode, false)) return launch_t3d(prob, mode, false, a, st);
     }
     if (fx2d_use<T>(prob, a, mode)) return launch_fx2d<T>(prob, mode, a, st);
     if (!is_2d(prob) && ep3d_use(a)) return launch_ep3d<T>(prob, mode, false, a, st);

@@ -48,7 +48,7 @@ struct EpsParams {
     int unit = 0;        // 1: slots produced from a norm are for the unit direction (EPS_UNIT)
 };
 
-// Tiling of the FP64 fixed-point kernel (stencil_fx.cu)
+// Tiling of the z-marching kernels (stencil_fx.cu, stencil_t3.cu)
 struct FxTiling {
     int ex, ey;         // elements of a tile; it completes (ex - 1) x (ey - 1) nodes
     int tx, ty;         // tiles per direction
@@ -95,6 +95,7 @@ struct StencilArgs {
                              // thread-block cluster (stencil_ep.cu; cl_max_n 0: never)
     int v2_threads;      // cap on the CTA size of the halo-free kernel (0: 1024; < 0: not used)
     FxTiling fx;         // FP64: tiling of the fixed-point kernel (stencil_fx.cu; no CTAs: not used)
+    FxTiling t3;         // FP32: tiling of the z-marching kernel (stencil_t3.cu; no CTAs: not used)
     int v3;              // FP32: the halo-free kernel's two-elements-per-thread variant (0: not used;
                          // 1 / 2: one / two CTAs per SM; other: chosen per mode)
     // adjoint kernel: per-element (dF/dkappa_e)^T v times dk_scale (nullable)
