@@ -13,26 +13,42 @@ namespace jfnk {
 
 constexpr int kBThreads = 256;
 
+// The segment this CTA belongs to (every warp finds it for itself).
+__device__ __forceinline__ int b_segment(const BSeg* __restrict__ segs, int count) {
+    const int lane = threadIdx.x & 31;
+    int s = 0;
+    for (int base = 0; base < count; base += 32) {
+        const bool le = base + lane < count && segs[base + lane].first <= (int)blockIdx.x;
+        const unsigned int m = __ballot_sync(0xffffffffu, le);
+        s += __popc(m);
+        if (m != 0xffffffffu) break;
+    }
+    return s - 1;
+}
+
 // ---------------------------------------------------------------------------
-// 2D element-residual kernel over (instance, strip, row chunk) tiles: one CTA a
-// tile (stencil_fx2d.cuh), a warp per part of its rows; the tile's x0 is the
-// strip.
+// 2D element-residual kernel over (instance, strip, row chunk): a CTA takes a
+// chunk of a strip's node rows (stencil_fx2d.cuh).
 // ---------------------------------------------------------------------------
 constexpr int kB2Threads = 256;
 
 template <typename T, Mode M>
 __global__ void __launch_bounds__(kB2Threads) fx2d_batched_kernel(const StencilArgs<T>* __restrict__ args,
-                                                                  const BTile* __restrict__ tiles) {
+                                                                  const BSeg* __restrict__ segs, int count) {
     __shared__ double red_sm[32];
-    const BTile t = tiles[blockIdx.x];
-    fx2d_cta<Prob::BRATU2, M>(args[t.inst], t.x0, t.y0, t.y1, t.bid, t.nblk, red_sm);
+    const int s = b_segment(segs, count);
+    const BSeg g = segs[s];
+    const int bid = blockIdx.x - g.first;
+    const int chunk = bid / g.strips, strip = bid - chunk * g.strips;
+    const int y0 = chunk * g.rows;
+    fx2d_cta<Prob::BRATU2, M>(args[s], strip, y0, min(y0 + g.rows, args[s].g.ny), bid, g.nblk, red_sm);
 }
 
 template <typename T>
-jfnk_status launch_stencil2d_batched(Mode mode, const StencilArgs<T>* dev_args, const BTile* dev_tiles, int ntiles,
-                                     int bx, cudaStream_t st) {
-    if (ntiles <= 0) return JFNK_OK;
-#define JFNK_B2(MM) fx2d_batched_kernel<T, MM><<<ntiles, bx, 0, st>>>(dev_args, dev_tiles)
+jfnk_status launch_stencil2d_batched(Mode mode, const StencilArgs<T>* dev_args, const BSeg* dev_segs, int count,
+                                     int blocks, int bx, cudaStream_t st) {
+    if (blocks <= 0) return JFNK_OK;
+#define JFNK_B2(MM) fx2d_batched_kernel<T, MM><<<blocks, bx, 0, st>>>(dev_args, dev_segs, count)
     switch (mode) {
         case Mode::F: JFNK_B2(Mode::F); break;
         case Mode::JV: JFNK_B2(Mode::JV); break;
@@ -45,9 +61,9 @@ jfnk_status launch_stencil2d_batched(Mode mode, const StencilArgs<T>* dev_args, 
     JFNK_LAUNCH_CHECK();
     return JFNK_OK;
 }
-template jfnk_status launch_stencil2d_batched<double>(Mode, const StencilArgs<double>*, const BTile*, int, int,
+template jfnk_status launch_stencil2d_batched<double>(Mode, const StencilArgs<double>*, const BSeg*, int, int, int,
                                                       cudaStream_t);
-template jfnk_status launch_stencil2d_batched<float>(Mode, const StencilArgs<float>*, const BTile*, int, int,
+template jfnk_status launch_stencil2d_batched<float>(Mode, const StencilArgs<float>*, const BSeg*, int, int, int,
                                                      cudaStream_t);
 
 // ---------------------------------------------------------------------------
@@ -105,10 +121,13 @@ __device__ __forceinline__ double b_scaled(double b, double ti, double, double) 
 __device__ __forceinline__ float b_scaled(float b, double, float th, float tl) { return fmaf(b, th, b * tl); }
 
 template <typename T, BOp OP>
-__global__ void __launch_bounds__(kBThreads) bvec_kernel(const BVec* __restrict__ descs, const BItem* __restrict__ items) {
+__global__ void __launch_bounds__(kBThreads) bvec_kernel(const BVec* __restrict__ descs, const BSeg* __restrict__ segs, int count) {
     __shared__ double sm[32];
-    const BItem it = items[blockIdx.x];
-    const BVec& d = descs[it.inst];
+    const int seg = b_segment(segs, count);
+    const BVec& d = descs[seg];
+    const struct {
+        int bid, nblk;
+    } it = {(int)blockIdx.x - segs[seg].first, segs[seg].nblk};
     const long long stride = (long long)it.nblk * blockDim.x;
     const long long i0 = (long long)it.bid * blockDim.x + threadIdx.x;
     if (OP == BOp::CAST_D2T) {
@@ -268,10 +287,10 @@ __global__ void __launch_bounds__(kBThreads) bvec_kernel(const BVec* __restrict_
 }
 
 template <typename T>
-jfnk_status launch_bvec(BOp op, const BVec* dev_desc, const BItem* dev_items, int nitems, cudaStream_t st) {
-    if (nitems <= 0) return JFNK_OK;
+jfnk_status launch_bvec(BOp op, const BVec* dev_desc, const BSeg* dev_segs, int count, int blocks, cudaStream_t st) {
+    if (blocks <= 0) return JFNK_OK;
 #define JFNK_BV(OPX)                                                                   \
-    case OPX: bvec_kernel<T, OPX><<<nitems, kBThreads, 0, st>>>(dev_desc, dev_items); break;
+    case OPX: bvec_kernel<T, OPX><<<blocks, kBThreads, 0, st>>>(dev_desc, dev_segs, count); break;
     switch (op) {
         JFNK_BV(BOp::CAST_D2T)
         JFNK_BV(BOp::CAST_T2D)
@@ -293,8 +312,8 @@ jfnk_status launch_bvec(BOp op, const BVec* dev_desc, const BItem* dev_items, in
     JFNK_LAUNCH_CHECK();
     return JFNK_OK;
 }
-template jfnk_status launch_bvec<float>(BOp, const BVec*, const BItem*, int, cudaStream_t);
-template jfnk_status launch_bvec<double>(BOp, const BVec*, const BItem*, int, cudaStream_t);
+template jfnk_status launch_bvec<float>(BOp, const BVec*, const BSeg*, int, int, cudaStream_t);
+template jfnk_status launch_bvec<double>(BOp, const BVec*, const BSeg*, int, int, cudaStream_t);
 
 // ---------------------------------------------------------------------------
 __global__ void bscalar_kernel(BScalar op, const BScal* __restrict__ descs, int count) {
@@ -315,6 +334,10 @@ __global__ void bscalar_kernel(BScalar op, const BScal* __restrict__ descs, int 
             d.cheb->c1f[k] = (float)c1;
             d.cheb->c2f[k] = (float)c2;
         }
+    } else if (op == BScalar::GATHER) {
+        for (int k = 0; k < d.m; ++k) d.out[k] = d.x[k];
+        d.out[kGatherIters] = *d.x2;
+        d.out[kGatherStatus] = (double)*d.status;
     } else if (op == BScalar::SET_EPS) {
         const double e = d.a;
         const double inv = e > 0.0 ? 1.0 / e : 0.0;

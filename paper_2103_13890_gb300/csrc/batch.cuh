@@ -1,6 +1,6 @@
 // Batched kernels: one launch applies a level operation to every active
 // instance of a batch of independent problems of uneven sizes.  Each CTA
-// reads a work item (instance, tile or block) and that instance's operands
+// finds its instance in a segment list and reads that instance's operands
 // from descriptor arrays in device memory; reductions complete per instance
 // (each instance's CTAs form one segment of the last-block reduction).
 #pragma once
@@ -9,16 +9,13 @@
 
 namespace jfnk {
 
-// node rows [y0, y1) of a strip of node columns (stencil_fx2d.cuh) of one instance
-struct BTile {
-    int inst;
-    int x0, y0, y1;  // x0: the strip
-    int bid, nblk;   // index among the instance's CTAs, their count
-};
-
-// work item of a batched vector operation
-struct BItem {
-    int inst, bid, nblk, pad;
+// One instance's CTAs in a batched launch: consecutive blocks from `first`.  A CTA
+// finds its instance among the segments (sorted by first) with one load a lane
+// and a ballot per 32 segments, so that a launch's work list is one entry per
+// instance and not one per CTA.
+struct BSeg {
+    int first, nblk;
+    int strips, rows;  // 2D kernel: strips of node columns, node rows a CTA (stencil_fx2d.cuh)
 };
 
 // per-instance operands of a batched vector operation
@@ -65,7 +62,9 @@ enum class BOp : int {
 enum class BScalar : int {
     CHEB_TABLE = 1,  // cheb table from *x with [a, b] and degree m
     SET_EPS = 2,     // slot from a
+    GATHER = 3,      // out[0..m) = x[0..m); out[kGatherIters] = *x2 (bits); out[kGatherStatus] = *status
 };
+constexpr int kGatherIters = JFNK_MAX_LEVELS, kGatherStatus = JFNK_MAX_LEVELS + 1;
 struct BScal {
     double* out;
     const double* x;
@@ -77,13 +76,13 @@ struct BScal {
     int* status;
 };
 
-// one CTA of bx threads per tile
+// `blocks` CTAs of bx threads over `count` instances
 template <typename T>
-jfnk_status launch_stencil2d_batched(Mode mode, const StencilArgs<T>* dev_args, const BTile* dev_tiles, int ntiles,
-                                     int bx, cudaStream_t st);
+jfnk_status launch_stencil2d_batched(Mode mode, const StencilArgs<T>* dev_args, const BSeg* dev_segs, int count,
+                                     int blocks, int bx, cudaStream_t st);
 
 template <typename T>
-jfnk_status launch_bvec(BOp op, const BVec* dev_desc, const BItem* dev_items, int nitems, cudaStream_t st);
+jfnk_status launch_bvec(BOp op, const BVec* dev_desc, const BSeg* dev_segs, int count, int blocks, cudaStream_t st);
 
 jfnk_status launch_bscalar(BScalar op, const BScal* dev_desc, int count, cudaStream_t st);
 

@@ -117,39 +117,39 @@ static void stage2(BCtx& b, Arena& A, const std::vector<D>& v, const std::vector
     dw = stage(b, A, w, err);
 }
 
-// blocks per instance: about 8 entries a thread, and about 8 blocks per SM over
-// the launch, but no more than the dot products' scratch holds (kDotBlocks)
-static std::vector<BItem> vec_items(const std::vector<long long>& sizes) {
+// Work list of a vector operation: about 8 entries a thread, and about 8 blocks
+// per SM over the launch, but no more per instance than the dot products'
+// scratch holds (kDotBlocks).  Returns the blocks of the launch.
+static int vec_segs(const std::vector<long long>& sizes, std::vector<BSeg>& segs) {
     long long total = 0;
     for (long long s : sizes) total += s;
     const long long per = std::max(2048LL, (total + 8 * kNumSMs - 1) / (8 * kNumSMs));
-    std::vector<BItem> it;
-    for (int k = 0; k < (int)sizes.size(); ++k) {
-        const long long nb = std::max(1LL, std::min<long long>((sizes[k] + per - 1) / per, kDotBlocks));
-        for (int q = 0; q < nb; ++q) it.push_back(BItem{k, q, (int)nb, 0});
+    int blocks = 0;
+    for (long long s : sizes) {
+        const int nb = (int)std::max(1LL, std::min<long long>((s + per - 1) / per, kDotBlocks));
+        segs.push_back(BSeg{blocks, nb, 0, 0});
+        blocks += nb;
     }
-    return it;
+    return blocks;
 }
 
-// tiles of the 2D kernel for grids g[k]: rows per CTA so that the launch's warps
-// (`warps` a CTA) number about `slots`
-static std::vector<BTile> tiles_for(const std::vector<Grid>& gs, int warps, int slots) {
+// Work list of the 2D kernel for grids g[k]: node rows per CTA so that the
+// launch's warps (`warps` a CTA) number about `slots`.
+static int grid_segs(const std::vector<Grid>& gs, int warps, int slots, std::vector<BSeg>& segs) {
     long long total = 0;
     for (const Grid& g : gs) total += (long long)fx2d_strips(g.n) * g.ny;
     const int rows = fx2d_cta_rows(total, slots, warps);
-    std::vector<BTile> t;
-    for (int k = 0; k < (int)gs.size(); ++k) {
-        const Grid& g = gs[k];
+    int blocks = 0;
+    for (const Grid& g : gs) {
         const int strips = fx2d_strips(g.n);
         // (an instance's reduction scratch holds 2 kMaxRedBlocks partials)
         const int most = std::max(1, 2 * kMaxRedBlocks / strips);
         const int rk = std::max(rows, (g.ny + most - 1) / most);
-        const int ch = (g.ny + rk - 1) / rk;
-        for (int c = 0; c < ch; ++c)
-            for (int s = 0; s < strips; ++s)
-                t.push_back(BTile{k, s, c * rk, std::min(c * rk + rk, g.ny), c * strips + s, strips * ch});
+        const int nb = strips * ((g.ny + rk - 1) / rk);
+        segs.push_back(BSeg{blocks, nb, strips, rk});
+        blocks += nb;
     }
-    return t;
+    return blocks;
 }
 
 template <typename T>
@@ -160,26 +160,28 @@ static jfnk_status bstencil(BCtx& b, Arena& A, Mode m, const std::vector<int>& S
     for (int i : S) gs.push_back(b.ps[i]->lv[lvl_from_coarse].g);
     jfnk_status err = JFNK_OK;
     const TileCfg& tc = b.tile[sizeof(T) == 8 ? 1 : 0];
-    const std::vector<BTile> tiles = tiles_for(gs, tc.bx / 32, tc.target);
+    std::vector<BSeg> segs;
+    const int blocks = grid_segs(gs, tc.bx / 32, tc.target, segs);
     const StencilArgs<T>* da = nullptr;
-    const BTile* dt = nullptr;
-    stage2(b, A, args, tiles, da, dt, err);
+    const BSeg* dt = nullptr;
+    stage2(b, A, args, segs, da, dt, err);
     if (err != JFNK_OK) return err;
     if (b.dry) return JFNK_OK;
-    return launch_stencil2d_batched<T>(m, da, dt, (int)tiles.size(), tc.bx, b.st);
+    return launch_stencil2d_batched<T>(m, da, dt, (int)segs.size(), blocks, tc.bx, b.st);
 }
 
 template <typename T>
 static jfnk_status bvec(BCtx& b, Arena& A, BOp op, const std::vector<BVec>& d, const std::vector<long long>& sizes) {
     if (d.empty()) return JFNK_OK;
     jfnk_status err = JFNK_OK;
-    const std::vector<BItem> items = vec_items(sizes);
+    std::vector<BSeg> segs;
+    const int blocks = vec_segs(sizes, segs);
     const BVec* dd = nullptr;
-    const BItem* di = nullptr;
-    stage2(b, A, d, items, dd, di, err);
+    const BSeg* di = nullptr;
+    stage2(b, A, d, segs, dd, di, err);
     if (err != JFNK_OK) return err;
     if (b.dry) return JFNK_OK;
-    return launch_bvec<T>(op, dd, di, (int)items.size(), b.st);
+    return launch_bvec<T>(op, dd, di, (int)segs.size(), blocks, b.st);
 }
 
 static jfnk_status bscalar(BCtx& b, Arena& A, BScalar op, const std::vector<BScal>& d) {
@@ -403,37 +405,34 @@ static jfnk_status bvcycle(BCtx& b, Arena& A, const std::vector<int>& act) {
     return JFNK_OK;
 }
 
-// Build (dry pass + upload) or reuse the V-cycle program for `act`, then run it.
+// Build (captured, or by a dry pass, and uploaded) or reuse the V-cycle program
+// for `act`, then run it.
 template <typename T>
 static jfnk_status bvcycle_run(BCtx& b, const std::vector<int>& act) {
     Arena& A = b.prog;
-    std::vector<long long> nF0(b.B * JFNK_MAX_LEVELS);
+    auto counts = [&](std::vector<long long>& c) {
+        c.resize((size_t)b.B * JFNK_MAX_LEVELS);
+        for (int i = 0; i < b.B; ++i) memcpy(&c[(size_t)i * JFNK_MAX_LEVELS], b.ps[i]->nF, sizeof(b.ps[i]->nF));
+    };
+    auto restore = [&](const std::vector<long long>& c) {
+        for (int i = 0; i < b.B; ++i) memcpy(b.ps[i]->nF, &c[(size_t)i * JFNK_MAX_LEVELS], sizeof(b.ps[i]->nF));
+    };
     if (act != b.prog_set) {
         if (b.graph) {
             cudaGraphExecDestroy(b.graph);
             b.graph = nullptr;
         }
+        b.prog_set.clear();
         A.reset();
-        for (int i = 0; i < b.B; ++i) memcpy(&nF0[i * JFNK_MAX_LEVELS], b.ps[i]->nF, sizeof(long long) * JFNK_MAX_LEVELS);
-        b.dry = true;
-        jfnk_status s = bvcycle<T>(b, A, act);
-        b.dry = false;
-        for (int i = 0; i < b.B; ++i) memcpy(b.ps[i]->nF, &nF0[i * JFNK_MAX_LEVELS], sizeof(long long) * JFNK_MAX_LEVELS);
-        JFNK_TRY(s);
-        JFNK_CUDA_TRY(cudaMemcpyAsync(A.dev, A.host.data(), A.off, cudaMemcpyHostToDevice, b.st));
-        JFNK_CUDA_TRY(cudaStreamSynchronize(b.st));
-        b.prog_set = act;
-    }
-    A.off = 0;
-    A.replay = true;
-    jfnk_status s = JFNK_OK;
-    if (b.o->use_graph) {
-        if (!b.graph) {
+        std::vector<long long> nF0;
+        counts(nF0);
+        jfnk_status s = JFNK_OK;
+        if (b.o->use_graph) {
+            // descriptors are placed and the launches that read them captured in one pass
             P& lp = *b.lead;
             if (!lp.cap_stream) JFNK_CUDA_TRY(cudaStreamCreateWithFlags(&lp.cap_stream, cudaStreamNonBlocking));
             cudaStream_t keep = b.st;
             b.st = lp.cap_stream;
-            for (int i = 0; i < b.B; ++i) memcpy(&nF0[i * JFNK_MAX_LEVELS], b.ps[i]->nF, sizeof(long long) * JFNK_MAX_LEVELS);
             const long long l0 = g_launches;
             JFNK_CUDA_TRY(cudaStreamBeginCapture(lp.cap_stream, cudaStreamCaptureModeThreadLocal));
             s = bvcycle<T>(b, A, act);
@@ -441,33 +440,40 @@ static jfnk_status bvcycle_run(BCtx& b, const std::vector<int>& act) {
             cudaError_t e = cudaStreamEndCapture(lp.cap_stream, &g);
             b.st = keep;
             // the captured launches have not run: what a replay evaluates and launches
-            b.graph_nF.assign(nF0.size(), 0);
-            for (int i = 0; i < b.B; ++i)
-                for (int l = 0; l < JFNK_MAX_LEVELS; ++l) {
-                    const size_t q = (size_t)i * JFNK_MAX_LEVELS + l;
-                    b.graph_nF[q] = b.ps[i]->nF[l] - nF0[q];
-                    b.ps[i]->nF[l] = nF0[q];
-                }
+            counts(b.graph_nF);
+            for (size_t q = 0; q < nF0.size(); ++q) b.graph_nF[q] -= nF0[q];
+            restore(nF0);
             b.graph_launches = g_launches - l0;
             g_launches = l0;
             if (s != JFNK_OK) {
                 if (e == cudaSuccess && g) cudaGraphDestroy(g);
-                A.replay = false;
                 return s;
             }
             JFNK_CUDA_TRY(e);
             cudaError_t ei = cudaGraphInstantiate(&b.graph, g, 0);
             cudaGraphDestroy(g);
             JFNK_CUDA_TRY(ei);
-            A.off = 0;
+        } else {
+            b.dry = true;
+            s = bvcycle<T>(b, A, act);
+            b.dry = false;
+            restore(nF0);
+            JFNK_TRY(s);
         }
+        JFNK_CUDA_TRY(cudaMemcpyAsync(A.dev, A.host.data(), A.off, cudaMemcpyHostToDevice, b.st));
+        JFNK_CUDA_TRY(cudaStreamSynchronize(b.st));
+        b.prog_set = act;
+    }
+    if (b.graph) {
         JFNK_CUDA_TRY(cudaGraphLaunch(b.graph, b.st));
         for (int i = 0; i < b.B; ++i)
             for (int l = 0; l < JFNK_MAX_LEVELS; ++l) b.ps[i]->nF[l] += b.graph_nF[(size_t)i * JFNK_MAX_LEVELS + l];
         g_launches += b.graph_launches;
-    } else {
-        s = bvcycle<T>(b, A, act);
+        return JFNK_OK;
     }
+    A.off = 0;
+    A.replay = true;
+    const jfnk_status s = bvcycle<T>(b, A, act);
     A.replay = false;
     return s;
 }
@@ -485,6 +491,30 @@ static jfnk_status read_res(BCtx& b, std::vector<double>& host) {
     JFNK_CUDA_TRY(cudaMemcpyAsync(host.data(), b.res, sizeof(double) * host.size(), cudaMemcpyDeviceToHost, b.st));
     JFNK_CUDA_TRY(cudaStreamSynchronize(b.st));
     return JFNK_OK;
+}
+
+// eigenvalue estimates of all levels, coarse iterations and status word of the
+// instances S, by one launch and one copy (BScalar::GATHER)
+static jfnk_status bgather(BCtx& b, const std::vector<int>& S, std::vector<double>& hr) {
+    std::vector<BScal> d;
+    for (int i : S) {
+        P& p = *b.ps[i];
+        BScal g;
+        memset(&g, 0, sizeof(g));
+        g.out = b.res + (size_t)i * kResStride;
+        g.x = p.lams;
+        g.x2 = reinterpret_cast<const double*>(p.coarse_iters);
+        g.m = p.L + 1;
+        g.status = p.status;
+        d.push_back(g);
+    }
+    JFNK_TRY(bscalar(b, b.dyn, BScalar::GATHER, d));
+    return read_res(b, hr);
+}
+static long long gathered_iters(const std::vector<double>& hr, int i) {
+    long long v;
+    memcpy(&v, &hr[(size_t)i * kResStride + kGatherIters], sizeof(v));
+    return v;
 }
 
 // out[i] = ||x_i|| (what 1) or sum |x_i| (what 0) over interior nodes; slot (optional) = FD step
@@ -548,11 +578,13 @@ static jfnk_status bjv64(BCtx& b, const std::vector<int>& S, const std::vector<c
     for (int i : S) gs.push_back(b.ps[i]->lv[b.ps[i]->L].g);
     jfnk_status err = JFNK_OK;
     const TileCfg& tc = b.tile[1];
-    const std::vector<BTile> tiles = tiles_for(gs, tc.bx / 32, tc.target);
-    const StencilArgs<double>* da = stage(b, b.dyn, args, err);
-    const BTile* dt = stage(b, b.dyn, tiles, err);
+    std::vector<BSeg> segs;
+    const int blocks = grid_segs(gs, tc.bx / 32, tc.target, segs);
+    const StencilArgs<double>* da = nullptr;
+    const BSeg* dt = nullptr;
+    stage2(b, b.dyn, args, segs, da, dt, err);
     JFNK_TRY(err);
-    return launch_stencil2d_batched<double>(Mode::JV, da, dt, (int)tiles.size(), tc.bx, b.st);
+    return launch_stencil2d_batched<double>(Mode::JV, da, dt, (int)segs.size(), blocks, tc.bx, b.st);
 }
 
 // F_i = F(x_i), A_i = A(x_i) (FP64, finest) and ||F_i|| into res slot 0
@@ -573,11 +605,13 @@ static jfnk_status bresidual64(BCtx& b, const std::vector<int>& S, const std::ve
     }
     jfnk_status err = JFNK_OK;
     const TileCfg& tc = b.tile[1];
-    const std::vector<BTile> tiles = tiles_for(gs, tc.bx / 32, tc.target);
-    const StencilArgs<double>* da = stage(b, b.dyn, args, err);
-    const BTile* dt = stage(b, b.dyn, tiles, err);
+    std::vector<BSeg> segs;
+    const int blocks = grid_segs(gs, tc.bx / 32, tc.target, segs);
+    const StencilArgs<double>* da = nullptr;
+    const BSeg* dt = nullptr;
+    stage2(b, b.dyn, args, segs, da, dt, err);
     JFNK_TRY(err);
-    JFNK_TRY(launch_stencil2d_batched<double>(Mode::F, da, dt, (int)tiles.size(), tc.bx, b.st));
+    JFNK_TRY(launch_stencil2d_batched<double>(Mode::F, da, dt, (int)segs.size(), blocks, tc.bx, b.st));
     std::vector<const void*> xv(F.begin(), F.end());
     std::vector<double*> outs;
     for (int i : S) outs.push_back(b.res + (size_t)i * kResStride);
@@ -736,11 +770,13 @@ static jfnk_status bsetup(BCtx& b, const std::vector<int>& S, int newton_step) {
         }
         if (!any) break;
         if (o.power_tol > 0.0) {
+            std::vector<int> running;  // (an instance may be named once per level)
             for (int c = 1; c <= cmax; ++c)
-                for (int i : Rl[c])
-                    JFNK_CUDA_TRY(cudaMemcpyAsync(&lam_now[c][i], b.ps[i]->lv[c].lam, sizeof(double),
-                                                  cudaMemcpyDeviceToHost, b.st));
-            JFNK_CUDA_TRY(cudaStreamSynchronize(b.st));
+                running.insert(running.end(), Rl[c].begin(), Rl[c].end());
+            std::vector<double> hr;
+            JFNK_TRY(bgather(b, running, hr));
+            for (int c = 1; c <= cmax; ++c)
+                for (int i : Rl[c]) lam_now[c][i] = hr[(size_t)i * kResStride + c];
             for (int c = 1; c <= cmax; ++c) {
                 std::vector<int> still;
                 for (int i : Rl[c]) {
@@ -1100,14 +1136,16 @@ static jfnk_status tune_tiles(BCtx& b) {
     jfnk_status err = JFNK_OK;
     for (int bx : {64, 128, 256}) {
         for (int target : {kFx2Slots32 / 2, kFx2Slots32, 2 * kFx2Slots32}) {
-            const std::vector<BTile> tiles = tiles_for(gs, bx / 32, target);
-            const StencilArgs<T>* da = stage(b, b.dyn, args, err);
-            const BTile* dt = stage(b, b.dyn, tiles, err);
+            std::vector<BSeg> segs;
+            const int blocks = grid_segs(gs, bx / 32, target, segs);
+            const StencilArgs<T>* da = nullptr;
+            const BSeg* dt = nullptr;
+            stage2(b, b.dyn, args, segs, da, dt, err);
             JFNK_TRY(err);
-            JFNK_TRY(launch_stencil2d_batched<T>(Mode::F, da, dt, (int)tiles.size(), bx, b.st));
+            JFNK_TRY(launch_stencil2d_batched<T>(Mode::F, da, dt, (int)segs.size(), blocks, bx, b.st));
             JFNK_CUDA_TRY(cudaEventRecord(e0, b.st));
             for (int r = 0; r < 3; ++r)
-                JFNK_TRY(launch_stencil2d_batched<T>(Mode::F, da, dt, (int)tiles.size(), bx, b.st));
+                JFNK_TRY(launch_stencil2d_batched<T>(Mode::F, da, dt, (int)segs.size(), blocks, bx, b.st));
             JFNK_CUDA_TRY(cudaEventRecord(e1, b.st));
             JFNK_CUDA_TRY(cudaEventSynchronize(e1));
             float ms = 0.f;
@@ -1135,8 +1173,9 @@ static jfnk_status bsolve(BCtx& b, jfnk_stats* stats) {
         for (int l = 0; l <= b.ps[i]->L; ++l) b.ps[i]->nF[l] = b.ps[i]->nFplain[l] = 0;
     }
     std::vector<long long> ci0(B, 0);
-    for (int i = 0; i < B; ++i)
-        JFNK_CUDA_TRY(cudaMemcpyAsync(&ci0[i], b.ps[i]->coarse_iters, sizeof(long long), cudaMemcpyDeviceToHost, b.st));
+    std::vector<double> hr;
+    JFNK_TRY(bgather(b, all, hr));
+    for (int i = 0; i < B; ++i) ci0[i] = gathered_iters(hr, i);
     if (sizeof(T) == 4) JFNK_TRY(tune_tiles(b));
     auto Fs = [&](const std::vector<int>& S, bool trial) {
         std::vector<double*> F, A;
@@ -1146,7 +1185,6 @@ static jfnk_status bsolve(BCtx& b, jfnk_stats* stats) {
         }
         return std::make_pair(F, A);
     };
-    std::vector<double> hr;
     {
         auto fa = Fs(all, false);
         std::vector<const double*> x(b.u.begin(), b.u.end());
@@ -1197,8 +1235,9 @@ static jfnk_status bsolve(BCtx& b, jfnk_stats* stats) {
         std::vector<int> its(B, 0);
         std::vector<ArnoldiSlope> asl(B);
         JFNK_TRY(bfgmres<T>(b, act, eta, its, asl));
+        JFNK_TRY(bgather(b, act, hr));
         for (int i : act) {
-            JFNK_TRY(check_status(*b.ps[i], b.st));
+            JFNK_TRY(status_word((int)hr[(size_t)i * kResStride + kGatherStatus]));
             S[i].linear_its += its[i];
             if (k < JFNK_MAX_HIST) S[i].lin_hist[k] = its[i];
         }
@@ -1333,18 +1372,16 @@ static jfnk_status bsolve(BCtx& b, jfnk_stats* stats) {
         }
     }
     jfnk_status result = JFNK_OK;
+    JFNK_TRY(bgather(b, all, hr));
     for (int i = 0; i < B; ++i) {
         P& p = *b.ps[i];
-        long long ci1 = 0;
-        JFNK_CUDA_TRY(cudaMemcpyAsync(&ci1, p.coarse_iters, sizeof(long long), cudaMemcpyDeviceToHost, b.st));
-        JFNK_CUDA_TRY(cudaStreamSynchronize(b.st));
-        p.nF[0] += ci1 - ci0[i];
+        p.nF[0] += gathered_iters(hr, i) - ci0[i];
         double ge = 0.0;
         for (int l = 0; l <= p.L && l < JFNK_MAX_LEVELS; ++l) {
             S[i].nF[l] = p.nF[l];
             S[i].nJv[l] = p.nF[l] - p.nFplain[l];
             ge += std::pow(2.0, -2.0 * (p.L - l)) * (double)p.nF[l];
-            if (l >= 1) JFNK_CUDA_TRY(cudaMemcpy(&S[i].lambda_max[l], p.lv[l].lam, sizeof(double), cudaMemcpyDeviceToHost));
+            if (l >= 1) S[i].lambda_max[l] = hr[(size_t)i * kResStride + l];
         }
         S[i].ge = ge;
         S[i].converged = conv(i) ? 1 : 0;

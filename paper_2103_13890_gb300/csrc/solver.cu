@@ -123,6 +123,7 @@ struct jfnk_problem {
     unsigned int* counters;
     int* status;
     long long* coarse_iters;
+    double* lams;  // the levels' lam, in one array (read with one copy)
     void* coarseV;
     double* coarseH;
     // CG-QN coarse solver: collected and kept secant pairs, compact-form state
@@ -212,11 +213,12 @@ static size_t plan(P& p, char* base, const jfnk_options* o) {
     p.nrm64 = pl.take<double>(8);
     p.xstat64 = pl.take<double>(8);
     p.coarse_iters = pl.take<long long>(8);
+    p.lams = pl.take<double>(JFNK_MAX_LEVELS);
     for (int l = 0; l <= p.L; ++l) {
         Level& L = p.lv[l];
         L.xstat_paper = pl.take<double>(1);
         L.xstat_fp32 = pl.take<double>(1);
-        L.lam = pl.take<double>(1);
+        L.lam = p.lams ? p.lams + l : nullptr;
         L.nrm0 = pl.take<double>(1);
         L.nrm1 = pl.take<double>(1);
         L.eps_s = pl.take<EpsSlot>(1);
@@ -679,8 +681,7 @@ static jfnk_status mg_setup_T(P& p, const jfnk_options& o, const double* u, int 
     for (int it = 0; it < o.power_iters && !active.empty(); ++it) {
         for (int l : active) JFNK_TRY(iterate(l));
         if (o.power_tol > 0.0) {
-            for (int l : active)
-                JFNK_CUDA_TRY(cudaMemcpyAsync(&lam_now[l], p.lv[l].lam, sizeof(double), cudaMemcpyDeviceToHost, st));
+            JFNK_CUDA_TRY(cudaMemcpyAsync(lam_now.data(), p.lams, sizeof(double) * (p.L + 1), cudaMemcpyDeviceToHost, st));
             JFNK_CUDA_TRY(cudaStreamSynchronize(st));
             std::vector<int> still;
             for (int l : active) {
@@ -975,15 +976,18 @@ static jfnk_status pcg(P& p, const jfnk_options& o, const double* u, double eta,
     return JFNK_OK;
 }
 
-static jfnk_status check_status(P& p, cudaStream_t st) {
-    int s = 0;
-    JFNK_CUDA_TRY(cudaMemcpyAsync(&s, p.status, sizeof(int), cudaMemcpyDeviceToHost, st));
-    JFNK_CUDA_TRY(cudaStreamSynchronize(st));
+static jfnk_status status_word(int s) {
     if (s) {
         set_error("device status word 0x%x (non-finite FD step or eigenvalue estimate)", s);
         return JFNK_ERR_NONFINITE;
     }
     return JFNK_OK;
+}
+static jfnk_status check_status(P& p, cudaStream_t st) {
+    int s = 0;
+    JFNK_CUDA_TRY(cudaMemcpyAsync(&s, p.status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    JFNK_CUDA_TRY(cudaStreamSynchronize(st));
+    return status_word(s);
 }
 
 template <typename T>
@@ -1116,7 +1120,9 @@ static jfnk_status solve_T(P& p, const jfnk_options& o, double* u, jfnk_stats* s
         set_error("Newton did not reach the tolerance in %d steps", k);
     }
     long long ci1 = 0;
+    double lams[JFNK_MAX_LEVELS];
     JFNK_CUDA_TRY(cudaMemcpyAsync(&ci1, p.coarse_iters, sizeof(long long), cudaMemcpyDeviceToHost, st));
+    JFNK_CUDA_TRY(cudaMemcpyAsync(lams, p.lams, sizeof(lams), cudaMemcpyDeviceToHost, st));
     JFNK_CUDA_TRY(cudaStreamSynchronize(st));
     p.nF[0] += ci1 - ci0;
     double ge = 0.0;
@@ -1124,11 +1130,7 @@ static jfnk_status solve_T(P& p, const jfnk_options& o, double* u, jfnk_stats* s
         S.nF[l] = p.nF[l];
         S.nJv[l] = p.nF[l] - p.nFplain[l];
         ge += std::pow(2.0, -(double)p.d * (p.L - l)) * (double)p.nF[l];
-        double lam = 0.0;
-        if (l >= 1) {
-            JFNK_CUDA_TRY(cudaMemcpy(&lam, p.lv[l].lam, sizeof(double), cudaMemcpyDeviceToHost));
-        }
-        S.lambda_max[l] = lam;
+        S.lambda_max[l] = l >= 1 ? lams[l] : 0.0;
     }
     S.ge = ge;
     if (p.lb) {
@@ -1700,12 +1702,14 @@ static jfnk_status adjoint_T(P& p, const jfnk_options& o, const double* u, const
         S.linear_its = its;
         S.lin_hist[0] = its;
         S.converged = 1;
+        double lams[JFNK_MAX_LEVELS];
+        JFNK_CUDA_TRY(cudaMemcpy(lams, p.lams, sizeof(lams), cudaMemcpyDeviceToHost));
         double ge = 0.0;
         for (int l = 0; l <= p.L && l < JFNK_MAX_LEVELS; ++l) {
             S.nF[l] = p.nF[l];
             S.nJv[l] = p.nF[l] - p.nFplain[l];
             ge += std::pow(2.0, -(double)p.d * (p.L - l)) * (double)p.nF[l];
-            if (l >= 1) JFNK_CUDA_TRY(cudaMemcpy(&S.lambda_max[l], p.lv[l].lam, sizeof(double), cudaMemcpyDeviceToHost));
+            if (l >= 1) S.lambda_max[l] = lams[l];
         }
         S.ge = ge;
         S.status = JFNK_OK;
