@@ -19,21 +19,45 @@
 
 #include "beam.cuh"
 #include "element.cuh"
+#include "fx_beam.cuh"
 #include "reduce.cuh"
 #include "stencil_body.cuh"
 
 namespace jfnk {
 
-constexpr int kBeamElemThreads = 128;
+constexpr int kBeamElemThreads = 64;
 constexpr int kBeamNodeThreads = 128;
 
+// The element's contributions; in FP64 factorised and partly in fixed point
+// (fx_beam.cuh), with elem_neohooke for what that does not take.
+static __device__ __noinline__ void neohooke_fp64(const double* u, double inv_h, double* r) {
+    double ue[24], q[24];
+    for (int k = 0; k < 24; ++k) ue[k] = u[k];
+    elem_neohooke<double>(ue, inv_h, q);
+    for (int k = 0; k < 24; ++k) r[k] = q[k];
+}
+__device__ __forceinline__ void beam_element(const double ue[24], double inv_h, const FxBeam& b, double r[24]) {
+    if (fx_scale_ok(inv_h) && fx_neohooke(ue, b, r)) return;
+    double us[24], rs[24];
+#pragma unroll
+    for (int k = 0; k < 24; ++k) us[k] = ue[k];
+    neohooke_fp64(us, inv_h, rs);
+#pragma unroll
+    for (int k = 0; k < 24; ++k) r[k] = rs[k];
+}
+__device__ __forceinline__ void beam_element(const float ue[24], float inv_h, const FxBeam&, float r[24]) {
+    elem_neohooke<float>(ue, inv_h, r);
+}
+
+// One thread per element, in storage order.
 template <typename T, Mode M>
-__global__ void __launch_bounds__(kBeamElemThreads) beam_elem_kernel(const StencilArgs<T> a) {
+__global__ void __launch_bounds__(kBeamElemThreads, 4) beam_elem_kernel(const StencilArgs<T> a) {
     const Grid g = a.g;
     const int ex = 10 * g.n, ey = g.n, ez = g.n;
-    const long long ne = (long long)ex * ey * ez;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
-    if (x >= ex) return;
+    const int ne = ex * ey * ez;  // (at most 10 x 256^3)
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= ne) return;
+    const int x = e % ex, yz = e / ex, y = yz % ey, z = yz / ey;
     T eps = T(0);
     if (M != Mode::F) eps = eps_of<T>(a.eps);
     T ue[24];
@@ -50,11 +74,10 @@ __global__ void __launch_bounds__(kBeamElemThreads) beam_elem_kernel(const Stenc
         }
     }
     T r[24];
-    elem_neohooke<T>(ue, a.lh, r);
-    const long long e = ((long long)z * ey + y) * ex + x;
+    beam_element(ue, a.lh, fx_beam(a.lh), r);
     T* C = a.face + e;
 #pragma unroll
-    for (int k = 0; k < 24; ++k) C[k * ne] = r[k];
+    for (int k = 0; k < 24; ++k) C[(long long)k * ne] = r[k];
 }
 
 template <typename T, Mode M>
@@ -104,9 +127,7 @@ static jfnk_status launch_beam_m(const StencilArgs<T>& a, cudaStream_t st) {
         set_error("beam element scratch too small (%lld < %lld)", a.face_cap, beam_scratch_count(g));
         return JFNK_ERR_WORKSPACE;
     }
-    const int ex = 10 * g.n;
-    const int bx = std::min(kBeamElemThreads, ((ex + 31) / 32) * 32);
-    beam_elem_kernel<T, M><<<dim3((ex + bx - 1) / bx, g.n, g.n), bx, 0, st>>>(a);
+    beam_elem_kernel<T, M><<<(int)((g.elements() + kBeamElemThreads - 1) / kBeamElemThreads), kBeamElemThreads, 0, st>>>(a);
     JFNK_LAUNCH_CHECK();
     const int nb = std::min(g.ny * g.nz, 2 * kMaxRedBlocks);
     beam_node_kernel<T, M><<<nb, kBeamNodeThreads, 0, st>>>(a);

@@ -5,6 +5,7 @@
 #pragma once
 #include "element.cuh"
 #include "fx64.cuh"
+#include "fx_beam.cuh"
 #include "stencil.cuh"
 
 namespace jfnk {
@@ -42,6 +43,22 @@ struct CoarseElem<double, Prob::NDK3> {
     __device__ explicit CoarseElem(double) : s(fx_scale(1.0)) {}
 };
 
+template <>
+struct CoarseElem<double, Prob::BEAM3> {
+    bool ok;
+    FxBeam b;
+    __device__ explicit CoarseElem(double inv_h) : ok(fx_scale_ok(inv_h)), b(fx_beam(ok ? inv_h : 1.0)) {}
+};
+
+// (out of line: it takes more registers than a coarse solver's thread has)
+static __device__ __noinline__ bool coarse_beam_fx(const double* u, const FxBeam& b, double* r) {
+    double ue[24], q[24];
+    for (int k = 0; k < 24; ++k) ue[k] = u[k];
+    if (!fx_neohooke(ue, b, q)) return false;
+    for (int k = 0; k < 24; ++k) r[k] = q[k];
+    return true;
+}
+
 template <typename T, Prob P>
 __device__ __forceinline__ void coarse_element_plain(const T* ue, T kap, T lh, T* r) {
     if (P == Prob::MINSURF2)
@@ -75,7 +92,9 @@ __device__ __forceinline__ void coarse_element(const Grid& g, const T* w, int x,
 #pragma unroll
             for (int i = 0; i < 3; ++i) ue[3 * c + i] = w[node * 3 + i];
         }
-        elem_neohooke<T>(ue, lh, r);
+        bool done = false;
+        if constexpr (sizeof(T) == 8) done = ce.ok && coarse_beam_fx(ue, ce.b, r);
+        if (!done) elem_neohooke<T>(ue, lh, r);
 #pragma unroll
         for (int k = 0; k < 24; ++k) C[k] = r[k];
     } else {
