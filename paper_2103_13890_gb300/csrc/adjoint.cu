@@ -98,20 +98,18 @@ __global__ void __launch_bounds__(KA_BX* KA_BY) vjp3d_kernel(const StencilArgs<T
         }
     }
     if (a.red == RedOut::NONE) return;
+    __shared__ EpsPre pre;
+    const bool step = a.red == RedOut::EPS;  // keeps the FD-step slot meaningful for mixed use
     double bs = block_sum(red, red_sm);
     double tot = 0.0;
-    if (grid_sum_last(bs, a.partials, a.counter, &tot, red_sm)) {
+    if (grid_sum_last(bs, a.partials, a.counter, &tot, [&] {
+            if (step) pre = eps_pre(a.epsp);
+        })) {
         if (threadIdx.x == 0 && threadIdx.y == 0) {
-            const double nrm = sqrt(tot);
-            if (a.red_norm) *a.red_norm = nrm;
-            if (a.red == RedOut::EPS) {  // keeps the FD-step slot meaningful for mixed use
-                double e = eps_formula(a.epsp.mode, a.epsp.n_unknowns, *a.epsp.xstat, nrm);
-                double inv = e > 0.0 ? 1.0 / e : 0.0;
-                a.red_eps->e = e;
-                a.red_eps->inv = inv;
-                a.red_eps->ef = (float)e;
-                a.red_eps->invf = (float)inv;
-            }
+            if (step)
+                set_eps_slot<false>(a.red_eps, pre, tot, false, nullptr, a.red_norm);
+            else if (a.red_norm)
+                *a.red_norm = sqrt(tot);
         }
     }
 }

@@ -71,16 +71,6 @@ template jfnk_status launch_stencil2d_batched<float>(Mode, const StencilArgs<flo
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ bool b_inner(const Grid& g, long long i) { return grid_unknown(g, i); }
 
-__device__ __forceinline__ void b_finish_eps(const BVec& d, double nrm) {
-    if (!d.slot) return;
-    double e = eps_formula(d.ep.mode, d.ep.n_unknowns, *d.ep.xstat, nrm);
-    double inv = e > 0.0 ? 1.0 / (d.ep.unit ? e * nrm : e) : 0.0;  // unit: see RedOut::EPS_UNIT
-    d.slot->e = e;
-    d.slot->inv = inv;
-    d.slot->ef = (float)e;
-    d.slot->invf = (float)inv;
-}
-
 __device__ __forceinline__ uint64_t b_splitmix(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
@@ -180,12 +170,17 @@ __global__ void __launch_bounds__(kBThreads) bvec_kernel(const BVec* __restrict_
                 acc.sq(dv);
             }
         }
+        __shared__ EpsPre pre;
+        const bool norm = OP != BOp::STAT || d.what != 0;
         const double bs = block_sum(acc.value(), sm);
         double tot = 0.0;
-        if (grid_sum_last_seg(bs, d.partials, d.counter, &tot, sm, it.bid, it.nblk) && threadIdx.x == 0) {
-            const double r = (OP == BOp::STAT && d.what == 0) ? tot : sqrt(tot);
-            if (d.out) *d.out = r;
-            b_finish_eps(d, r);
+        if (grid_sum_last_seg(bs, d.partials, d.counter, &tot, it.bid, it.nblk, [&] {
+                if (d.slot && norm) pre = eps_pre(d.ep);
+            }) && threadIdx.x == 0) {
+            if (d.slot && norm)
+                set_eps_slot<false>(d.slot, pre, tot, d.ep.unit != 0, nullptr, d.out);
+            else if (d.out)
+                *d.out = norm ? sqrt(tot) : tot;
         }
     } else if (OP == BOp::RESTRICT) {
         const Grid gc = d.gc, gf = d.g;

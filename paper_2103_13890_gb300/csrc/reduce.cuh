@@ -28,8 +28,11 @@ __device__ __forceinline__ double block_sum(TA v, double* sm) {
     __syncthreads();
     double t = 0.0;
     if (tid < 32) {
-        t = (tid < (nt + 31) / 32) ? sm[tid] : 0.0;
-        t = warp_sum(t);
+        // (a shuffled FP64 addition costs about 100 clocks: only the steps needed)
+        const int nw = (nt + 31) / 32;
+        t = (tid < nw) ? sm[tid] : 0.0;
+        for (int o = nw > 16 ? 16 : nw > 8 ? 8 : nw > 4 ? 4 : nw > 2 ? 2 : nw > 1 ? 1 : 0; o > 0; o >>= 1)
+            t += __shfl_xor_sync(0xffffffffu, t, o);
     }
     __syncthreads();
     return t;
@@ -38,13 +41,21 @@ __device__ __forceinline__ double block_sum(TA v, double* sm) {
 // Last-block completion over a segment of nb CTAs (bid = this CTA's index in
 // it).  Thread 0 of every block passes its block sum; returns true in every
 // thread of the last block of the segment, with the total in *total (thread
-// 0).  The completion counter is reset by the last block.
+// 0).  The completion counter is reset by the last block.  `early` runs in one
+// thread of the last block while the others sum the partials, and is visible to
+// thread 0 on return.  (At most 4 warps sum: an FP64 addition takes an SM
+// quarter 64 clocks a warp.  Blocks have at least one whole warp.)
+template <typename F>
 __device__ __forceinline__ bool grid_sum_last_seg(double blocksum, double* partials, unsigned int* counter,
-                                                  double* total, double* sm, unsigned int bid, unsigned int nb) {
+                                                  double* total, unsigned int bid, unsigned int nb, F early) {
+    __shared__ double s_part[4];
     const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
     const int nt = blockDim.x * blockDim.y * blockDim.z;
     if (nb == 1) {  // the only block: no partials, no completion counter
-        if (tid == 0) *total = blocksum;
+        if (tid == 0) {
+            early();
+            *total = blocksum;
+        }
         return true;
     }
     __shared__ int s_last;
@@ -57,10 +68,19 @@ __device__ __forceinline__ bool grid_sum_last_seg(double blocksum, double* parti
     __syncthreads();
     if (!s_last) return false;
     __threadfence();
-    double s = 0.0;
-    for (unsigned int i = tid; i < nb; i += nt) s += __ldcg(&partials[i]);
-    s = block_sum(s, sm);
+    const int act = nt >= 128 ? 128 : nt & ~31;
+    if (tid < act) {
+        double s = 0.0;
+#pragma unroll 4
+        for (unsigned int i = tid; i < nb; i += act) s += __ldcg(&partials[i]);
+        s = warp_sum(s);
+        if ((tid & 31) == 0) s_part[tid >> 5] = s;
+    }
+    if (tid == (act < nt ? act : 0)) early();
+    __syncthreads();
     if (tid == 0) {
+        double s = s_part[0];
+        for (int w = 1; w < act / 32; ++w) s += s_part[w];
         *total = s;
         *counter = 0u;
     }
@@ -68,11 +88,16 @@ __device__ __forceinline__ bool grid_sum_last_seg(double blocksum, double* parti
 }
 
 // The whole grid as one segment.
+template <typename F>
 __device__ __forceinline__ bool grid_sum_last(double blocksum, double* partials, unsigned int* counter,
-                                              double* total, double* sm) {
-    return grid_sum_last_seg(blocksum, partials, counter, total, sm,
+                                              double* total, F early) {
+    return grid_sum_last_seg(blocksum, partials, counter, total,
                              blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z),
-                             gridDim.x * gridDim.y * gridDim.z);
+                             gridDim.x * gridDim.y * gridDim.z, early);
+}
+__device__ __forceinline__ bool grid_sum_last(double blocksum, double* partials, unsigned int* counter,
+                                              double* total) {
+    return grid_sum_last(blocksum, partials, counter, total, [] {});
 }
 
 }  // namespace jfnk

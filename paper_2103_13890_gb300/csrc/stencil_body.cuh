@@ -186,14 +186,18 @@ template <typename T>
 __device__ __forceinline__ void stencil_reduce(const StencilArgs<T>& a, float red, double* sm, unsigned int bid,
                                                unsigned int nb) {
     if (a.red == RedOut::NONE) return;
+    __shared__ EpsPre pre;
+    const bool eps = a.red == RedOut::EPS || a.red == RedOut::EPS_UNIT;
     double bs = block_sum(red, sm);
     double tot = 0.0;
-    if (grid_sum_last_seg(bs, a.partials, a.counter, &tot, sm, bid, nb)) {
+    if (grid_sum_last_seg(bs, a.partials, a.counter, &tot, bid, nb, [&] {
+            if (eps) pre = eps_pre(a.epsp);
+        })) {
         if (threadIdx.x == 0 && threadIdx.y == 0) {
-            double nrm = sqrt(tot);
-            if (a.red_norm) *a.red_norm = nrm;
-            if (a.red == RedOut::EPS || a.red == RedOut::EPS_UNIT)
-                set_eps_slot(a.red_eps, a.epsp, nrm, a.red == RedOut::EPS_UNIT, a.status);
+            if (eps)
+                set_eps_slot(a.red_eps, pre, tot, a.red == RedOut::EPS_UNIT, a.status, a.red_norm);
+            else if (a.red_norm)
+                *a.red_norm = sqrt(tot);
         }
     }
 }

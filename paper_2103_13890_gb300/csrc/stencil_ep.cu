@@ -376,12 +376,15 @@ __global__ void __launch_bounds__(kEpSmallThreads) ep3d_small_kernel(const Stenc
             epilogue<T, M>(a, idx, inner, val, inv_eps, ck, red);
     }
     if (a.red == RedOut::NONE) return;
+    __shared__ EpsPre pre;
+    const bool step = a.red == RedOut::EPS || a.red == RedOut::EPS_UNIT;
+    if (step && threadIdx.x == 32) pre = eps_pre(a.epsp);
     const double bs = block_sum(red, red_sm);
     if (threadIdx.x == 0) {
-        const double nrm = sqrt(bs);
-        if (a.red_norm) *a.red_norm = nrm;
-        if (a.red == RedOut::EPS || a.red == RedOut::EPS_UNIT)
-            set_eps_slot(a.red_eps, a.epsp, nrm, a.red == RedOut::EPS_UNIT, a.status);
+        if (step)
+            set_eps_slot(a.red_eps, pre, bs, a.red == RedOut::EPS_UNIT, a.status, a.red_norm);
+        else if (a.red_norm)
+            *a.red_norm = sqrt(bs);
     }
 }
 
@@ -470,7 +473,10 @@ __global__ void __launch_bounds__(kEpClusterThreads) ep3d_cluster_kernel(const S
         }
         epilogue<T, M>(a, (int)JFNK_IDX(Z * sz + Y * sy + X, a.g.size), inner, val, inv_eps, ck, red);
     }
+    __shared__ EpsPre pre;
+    const bool step = a.red == RedOut::EPS || a.red == RedOut::EPS_UNIT;
     if (a.red != RedOut::NONE) {
+        if (step && rank == 0 && threadIdx.x == 32) pre = eps_pre(a.epsp);
         const double bs = block_sum(red, red_sm);
         if (threadIdx.x == 0) *cluster.map_shared_rank(&bsums[rank], 0) = bs;
     }
@@ -480,10 +486,10 @@ __global__ void __launch_bounds__(kEpClusterThreads) ep3d_cluster_kernel(const S
     if (a.red != RedOut::NONE && rank == 0 && threadIdx.x == 0) {
         double tot = 0.0;
         for (int q = 0; q < ncta; ++q) tot += bsums[q];
-        const double nrm = sqrt(tot);
-        if (a.red_norm) *a.red_norm = nrm;
-        if (a.red == RedOut::EPS || a.red == RedOut::EPS_UNIT)
-            set_eps_slot(a.red_eps, a.epsp, nrm, a.red == RedOut::EPS_UNIT, a.status);
+        if (step)
+            set_eps_slot(a.red_eps, pre, tot, a.red == RedOut::EPS_UNIT, a.status, a.red_norm);
+        else if (a.red_norm)
+            *a.red_norm = sqrt(tot);
     }
 }
 

@@ -677,15 +677,18 @@ __global__ void __launch_bounds__(256) stencil3d_fixup_kernel(const StencilArgs<
     if (!s_last) return;
     __threadfence();
     const int total_blocks = main_blocks + gridDim.x;
+    __shared__ EpsPre pre;
+    const bool step = a.red == RedOut::EPS || a.red == RedOut::EPS_UNIT;
+    if (step && tid == 32) pre = eps_pre(a.epsp);
     double s = 0.0;
     for (int b = tid; b < total_blocks; b += blockDim.x) s += __ldcg(&a.partials[b]);
     s = block_sum(s, red_sm);
     if (tid == 0) {
         *a.counter = 0u;
-        const double nrm = sqrt(s);
-        if (a.red_norm) *a.red_norm = nrm;
-        if (a.red == RedOut::EPS || a.red == RedOut::EPS_UNIT)
-            set_eps_slot(a.red_eps, a.epsp, nrm, a.red == RedOut::EPS_UNIT, a.status);
+        if (step)
+            set_eps_slot(a.red_eps, pre, s, a.red == RedOut::EPS_UNIT, a.status, a.red_norm);
+        else if (a.red_norm)
+            *a.red_norm = sqrt(s);
     }
 }
 

@@ -22,6 +22,19 @@ static int vec_blocks(long long len) {
 
 __device__ __forceinline__ bool grid_inner(const Grid& g, long long i) { return grid_unknown(g, i); }
 
+// Results of a norm (what 1) or a sum of magnitudes (what 0): out, norm_out and,
+// from a norm, the FD step of the vector.
+__device__ __forceinline__ void finish_stat(int what, double tot, double* out, double* norm_out, const EpsPre& pre,
+                                            const EpsParams& ep, EpsSlot* slot) {
+    if (slot && what != 0) {
+        set_eps_slot(slot, pre, tot, ep.unit != 0, nullptr, out, norm_out);
+        return;
+    }
+    const double r = what == 0 ? tot : sqrt(tot);
+    if (out) *out = r;
+    if (norm_out) *norm_out = r;
+}
+
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void masked_stat_kernel(Grid g, const T* x, int what, double* out, double* partials,
@@ -37,14 +50,13 @@ __global__ void masked_stat_kernel(Grid g, const T* x, int what, double* out, do
         const double t = (what == 0) ? fabs(v) : v * v;
         if (grid_inner(g, i)) acc += t;
     }
+    __shared__ EpsPre pre;
     double bs = block_sum(acc, sm);
     double tot = 0.0;
-    if (grid_sum_last(bs, partials, counter, &tot, sm) && threadIdx.x == 0) {
-        double r = (what == 0) ? tot : sqrt(tot);
-        if (out) *out = r;
-        if (norm_out) *norm_out = r;
-        if (slot) set_eps_slot(slot, ep, r, ep.unit != 0, nullptr);
-    }
+    if (grid_sum_last(bs, partials, counter, &tot, [&] {
+            if (slot) pre = eps_pre(ep);
+        }) && threadIdx.x == 0)
+        finish_stat(what, tot, out, norm_out, pre, ep, slot);
 }
 
 // Scalar grids (nc = 1): the interior is (n-1)^(d-1) rows of n-1 contiguous
@@ -106,14 +118,13 @@ __global__ void __launch_bounds__(kVecThreads) masked_stat_rows_kernel(Grid g, c
     double acc = 0.0;
     for (unsigned int r = blockIdx.x * kRowWarps + (threadIdx.x >> 5); r < nrows; r += wstride)
         acc += row_stat<T, WHAT>(x + JFNK_IDX(interior_row_base(g, r), g.size - g.nx + 1), g.nx, lane);
+    __shared__ EpsPre pre;
     double bs = block_sum(acc, sm);
     double tot = 0.0;
-    if (grid_sum_last(bs, partials, counter, &tot, sm) && threadIdx.x == 0) {
-        double res = (WHAT == 0) ? tot : sqrt(tot);
-        if (out) *out = res;
-        if (norm_out) *norm_out = res;
-        if (slot) set_eps_slot(slot, ep, res, ep.unit != 0, nullptr);
-    }
+    if (grid_sum_last(bs, partials, counter, &tot, [&] {
+            if (slot) pre = eps_pre(ep);
+        }) && threadIdx.x == 0)
+        finish_stat(WHAT, tot, out, norm_out, pre, ep, slot);
 }
 
 // at most kVecBlocks blocks (8 per SM); up to 2048 blocks, one row a warp at
@@ -269,7 +280,7 @@ __global__ void sumsq_kernel(const double* __restrict__ w, long long len, double
     }
     double bs = block_sum(acc, sm);
     double tot = 0.0;
-    if (grid_sum_last(bs, partials, counter, &tot, sm) && threadIdx.x == 0) *nrm_out = sqrt(tot);
+    if (grid_sum_last(bs, partials, counter, &tot) && threadIdx.x == 0) *nrm_out = sqrt(tot);
 }
 
 __global__ void scale_inv_kernel(double* __restrict__ y, const double* __restrict__ x, long long len,
@@ -488,16 +499,11 @@ __global__ void cheb_start_zero_kernel(Grid g, const T* __restrict__ b, T* __res
         d[i] = dv;
         acc += (double)dv * (double)dv;
     }
+    __shared__ EpsPre pre;
     double bs = block_sum(acc, sm);
     double tot = 0.0;
-    if (grid_sum_last(bs, partials, counter, &tot, sm) && threadIdx.x == 0) {
-        double e = eps_formula(ep.mode, ep.n_unknowns, *ep.xstat, sqrt(tot));
-        double inv = e > 0.0 ? 1.0 / e : 0.0;
-        slot->e = e;
-        slot->inv = inv;
-        slot->ef = (float)e;
-        slot->invf = (float)inv;
-    }
+    if (grid_sum_last(bs, partials, counter, &tot, [&] { pre = eps_pre(ep); }) && threadIdx.x == 0)
+        set_eps_slot<false>(slot, pre, tot, false, nullptr);
 }
 
 // The same over the rows of a scalar grid (every row, so that the boundary
@@ -534,16 +540,11 @@ __global__ void __launch_bounds__(kVecThreads) cheb_start_zero_rows_kernel(
         }
         acc += (double)f;
     }
+    __shared__ EpsPre pre;
     double bs = block_sum(acc, sm);
     double tot = 0.0;
-    if (grid_sum_last(bs, partials, counter, &tot, sm) && threadIdx.x == 0) {
-        double e = eps_formula(ep.mode, ep.n_unknowns, *ep.xstat, sqrt(tot));
-        double inv = e > 0.0 ? 1.0 / e : 0.0;
-        slot->e = e;
-        slot->inv = inv;
-        slot->ef = (float)e;
-        slot->invf = (float)inv;
-    }
+    if (grid_sum_last(bs, partials, counter, &tot, [&] { pre = eps_pre(ep); }) && threadIdx.x == 0)
+        set_eps_slot<false>(slot, pre, tot, false, nullptr);
 }
 
 template <typename T>
