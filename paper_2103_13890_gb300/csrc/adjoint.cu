@@ -15,6 +15,7 @@
 #include "stencil.cuh"
 #include "stencil_body.cuh"
 #include "stencil_ep.cuh"
+#include "stencil_fx.cuh"
 #include "stencil_t3.cuh"
 
 namespace jfnk {
@@ -148,7 +149,9 @@ static jfnk_status launch_vjp_k(Mode mode, const StencilArgs<T>& a, cudaStream_t
 
 template <typename T>
 jfnk_status launch_vjp(Prob prob, Mode mode, const StencilArgs<T>& a, cudaStream_t st) {
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 8) {
+        if ((prob == Prob::NDK3 || prob == Prob::ND3) && fx3d_use(a, mode, true)) return launch_fx3d(prob, mode, true, a, st);
+    } else {
         if ((prob == Prob::NDK3 || prob == Prob::ND3) && t3d_use(a, mode, true)) return launch_t3d(prob, mode, true, a, st);
     }
     if ((prob == Prob::NDK3 || prob == Prob::ND3) && ep3d_use(a, true)) return launch_ep3d<T>(prob, mode, true, a, st);

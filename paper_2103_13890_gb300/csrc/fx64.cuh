@@ -1,5 +1,5 @@
-// 64-bit fixed-point evaluation of the 3D nonlinear-diffusion, 2D Bratu and 2D
-// minimal-surface elements, for the FP64 kernels.
+// 64-bit fixed-point evaluation of the 3D nonlinear-diffusion (residual and
+// vector-Jacobian product), 2D Bratu and 2D minimal-surface elements, for the FP64 kernels.
 //
 // What bounds an FP64 element kernel on this GPU is the FP64 pipe: 2
 // operations per clock and SM.  The integer pipe adds 64-bit integers at ~52
@@ -151,14 +151,19 @@ __host__ __device__ __forceinline__ fx_t fx_mul(fx_t a, FxMul b) {
     return (fx_t)fx_hi(a) * b.h + t;
 }
 
+// a b / 2^64 of two split numbers, less than 2 off
+__host__ __device__ __forceinline__ fx_t fx_mul(FxMul a, FxMul b) {
+    return (fx_t)a.h * b.h + fx_madhi_s(a.h, b.l, fx_mulhi_s(a.l, b.h));
+}
+
 // 1/sqrt 3, 1/3 and 1/(3 sqrt 3), times 2^63
 constexpr fx_t kFxA1 = 0x49e69d1640cc7135LL, kFxA2 = 0x2aaaaaaaaaaaaaabLL, kFxA3 = 0x18a2345cc04425bcLL;
 
 // Test-side multipliers of an element: A^k times a positive scale (the node
-// factor, and kappa), its power of two apart.  b_k = A^k m 2^63, scale = m 2^ex
-// with m in [1/2, 1).
+// factor, and kappa), its power of two apart.  b_k = A^k m 2^63 (b0: m 2^62),
+// scale = m 2^ex with m in [1/2, 1).
 struct FxScale {
-    FxMul b1, b2, b3;
+    FxMul b0, b1, b2, b3;
     int ex;
 };
 // a positive normal double as m 2^62 (exact) and ex
@@ -169,6 +174,7 @@ __host__ __device__ __forceinline__ FxMul fx_significand(double x, int& ex) {
 __host__ __device__ __forceinline__ FxScale fx_scale(double scale) {
     FxScale s;
     const FxMul m = fx_significand(scale, s.ex);
+    s.b0 = m;
     s.b1 = fx_split(fx_shl(fx_mul(kFxA1, m), 2));
     s.b2 = fx_split(fx_shl(fx_mul(kFxA2, m), 2));
     s.b3 = fx_split(fx_shl(fx_mul(kFxA3, m), 2));
@@ -180,8 +186,10 @@ __host__ __device__ __forceinline__ FxScale fx_scale_kappa(const FxScale& sc, do
     FxScale s;
     int ex;
     const FxMul m = fx_significand(kap, ex);
+    const fx_t v0 = fx_mul(fx_value(sc.b0), m);
     const fx_t v1 = fx_mul(fx_value(sc.b1), m), v2 = fx_mul(fx_value(sc.b2), m), v3 = fx_mul(fx_value(sc.b3), m);
     const int l = v2 < (kFxA2 >> 3) ? 3 : 2;  // the product of the significands back to [1/2, 1)
+    s.b0 = fx_split(fx_shl(v0, l));
     s.b1 = fx_split(fx_shl(v1, l));
     s.b2 = fx_split(fx_shl(v2, l));
     s.b3 = fx_split(fx_shl(v3, l));
@@ -235,22 +243,24 @@ __host__ __device__ __forceinline__ void fx_h2_adj(const fx_t F[2][2], fx_t& w00
     w11 = D1 - D0;
 }
 
-// elem_nd3 (element.cuh) in fixed point: p[8] packed corner values with largest
-// exponent field xm (fx_exp_ok), r[8] the contributions as integers times 2^X,
-// the scale of `sc` applied.  Upper bounds: W 2^55, M 2^58, M' 2^62, S' 2^61,
-// G 2^61.6, U 2^60, K 2^61, F 2^59.6, X 2^61.1, X+Y+Z 2^62.5, r 2^62.6.
-__host__ __device__ __forceinline__ void fx_nd3(const fx_t p[8], int xm, const FxScale& sc, fx_t r[8], int& X) {
-    const int e = xm + kFxBias - 1022;  // |w| < 2^e
-    const int k = 55 - e;               // W = w 2^k
+// Modes of an element's packed corner values p[8] with largest exponent field xm:
+// W = w 2^k, M = T (x) T (x) T W; S = A^(p+q+r) M 2^(s-1) of the gradient modes, left-aligned
+// by s (|M 2^s| < 2^62).
+struct FxModes3 {
+    fx_t M000, S001, S010, S100, S011, S101, S110, S111;
+    int k, s;
+};
+__host__ __device__ __forceinline__ FxModes3 fx_modes3(const fx_t p[8], int xm) {
+    FxModes3 m;
+    m.k = 55 - (xm + kFxBias - 1022);
     fx_t u[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) u[c] = fx_sar(p[c] & ~(fx_t)kFxMask, 8 + xm - fx_exp(p[c]));
-    // modes (as in elem_nd3)
     const fx_t p0 = u[0] + u[1], q0 = u[1] - u[0], p1 = u[2] + u[3], q1 = u[3] - u[2];
     const fx_t p2 = u[4] + u[5], q2 = u[5] - u[4], p3 = u[6] + u[7], q3 = u[7] - u[6];
     const fx_t a00 = p0 + p1, a01 = p1 - p0, b00 = p2 + p3, b01 = p3 - p2;
     const fx_t a10 = q0 + q1, a11 = q1 - q0, b10 = q2 + q3, b11 = q3 - q2;
-    const fx_t M000 = a00 + b00;
+    m.M000 = a00 + b00;
     fx_t M[7] = {b00 - a00, a01 + b01, a10 + b10, b01 - a01, b10 - a10, a11 + b11, b11 - a11};
     // left-align the gradient modes: |M| < 2^(64 - clz), M' = M 2^s < 2^62
     unsigned int top = 0;
@@ -266,20 +276,36 @@ __host__ __device__ __forceinline__ void fx_nd3(const fx_t p[8], int xm, const F
         s = 30 + fx_clz(low);
     }
     const FxMul A1 = fx_split(kFxA1), A2 = fx_split(kFxA2), A3 = fx_split(kFxA3);
-    const fx_t S001 = fx_mul(fx_shl(M[0], s), A1), S010 = fx_mul(fx_shl(M[1], s), A1), S100 = fx_mul(fx_shl(M[2], s), A1);
-    const fx_t S011 = fx_mul(fx_shl(M[3], s), A2), S101 = fx_mul(fx_shl(M[4], s), A2), S110 = fx_mul(fx_shl(M[5], s), A2);
-    const fx_t S111 = fx_mul(fx_shl(M[6], s), A3);
+    m.s = s;
+    m.S001 = fx_mul(fx_shl(M[0], s), A1);
+    m.S010 = fx_mul(fx_shl(M[1], s), A1);
+    m.S100 = fx_mul(fx_shl(M[2], s), A1);
+    m.S011 = fx_mul(fx_shl(M[3], s), A2);
+    m.S101 = fx_mul(fx_shl(M[4], s), A2);
+    m.S110 = fx_mul(fx_shl(M[5], s), A2);
+    m.S111 = fx_mul(fx_shl(M[6], s), A3);
+    return m;
+}
+
+// elem_nd3 (element.cuh) in fixed point: p[8] packed corner values with largest
+// exponent field xm (fx_exp_ok), r[8] the contributions as integers times 2^X,
+// the scale of `sc` applied.  Upper bounds: W 2^55, M 2^58, M' 2^62, S' 2^61,
+// G 2^61.6, U 2^60, K 2^61, F 2^59.6, X 2^61.1, X+Y+Z 2^62.5, r 2^62.6.
+__host__ __device__ __forceinline__ void fx_nd3(const fx_t p[8], int xm, const FxScale& sc, fx_t r[8], int& X) {
+    const int e = xm + kFxBias - 1022;  // |w| < 2^e
+    const FxModes3 m = fx_modes3(p, xm);
+    const int k = m.k, s = m.s;
     fx_t P0[2][2], GX[2][2], GY[2][2], GZ[2][2];
-    fx_h2_fwd(0, S010, S001, S011, P0);     // [sy][sz], without the constant mode
-    fx_h2_fwd(S100, S110, S101, S111, GX);  // [sy][sz]
-    fx_h2_fwd(S010, S110, S011, S111, GY);  // [sx][sz]
-    fx_h2_fwd(S001, S101, S011, S111, GZ);  // [sx][sy]
+    fx_h2_fwd(0, m.S010, m.S001, m.S011, P0);     // [sy][sz], without the constant mode
+    fx_h2_fwd(m.S100, m.S110, m.S101, m.S111, GX);  // [sy][sz]
+    fx_h2_fwd(m.S010, m.S110, m.S011, m.S111, GY);  // [sx][sz]
+    fx_h2_fwd(m.S001, m.S101, m.S011, m.S111, GZ);  // [sx][sy]
     // 1 + u^2 at the points: U = u 2^(60 - max(e, 0)), K = (1 + u^2) 2^(60 - f)
     // with f = 2 max(e, 0); U carries 2^31 and K 2^30, so that the sum of two K
     // carries 2^31, which turns the lower words into rounded signed ones
     const int ep = e > 0 ? e : 0, f = 2 * ep;
     const fx_t one = (f > 60 ? 0 : (fx_t)1 << (60 - f)) + (fx_t)0x40000000LL;
-    const fx_t U0 = fx_sar(fx_shl(M000, 2), ep - e) + (fx_t)0x80000000LL;
+    const fx_t U0 = fx_sar(fx_shl(m.M000, 2), ep - e) + (fx_t)0x80000000LL;
     const int shu = s - 3 + ep - e;
     fx_t K[2][2][2];
 #pragma unroll
@@ -322,6 +348,111 @@ __host__ __device__ __forceinline__ void fx_nd3(const fx_t p[8], int xm, const F
     r[4] = f0_01 - f1_01; r[5] = f0_01 + f1_01;
     r[6] = f0_11 - f1_11; r[7] = f0_11 + f1_11;
     X = sc.ex + 3 + f - k - s;
+}
+
+// elem_vjp3 (element.cuh) in fixed point, without the coefficient's derivative:
+// p[8] packed corner values of u with largest exponent field xu (below
+// kFxMaxExp), q[8] of the covector w with xw (fx_exp_ok), r[8] times 2^X as above.
+// The flux terms are those of fx_nd3 with the gradients of w; the source terms
+// 2 u (grad u . grad w) have the exponent of a triple product, and the modes of
+// both are summed at the larger of the two exponents.  Upper bounds: 4 dot
+// 2^62.8, src 2^58.8, E 2^61.8, r 2^62.7.
+__host__ __device__ __forceinline__ void fx_vjp3(const fx_t p[8], int xu, const fx_t q[8], int xw, const FxScale& sc,
+                                                 fx_t r[8], int& X) {
+    if (xu < kFxMinExp) xu = kFxMinExp;  // (u = 0, or so small that only 1 + u^2 = 1 is left of it)
+    const int e = xu + kFxBias - 1022;
+    const int ep = e > 0 ? e : 0, f = 2 * ep;
+    const FxModes3 mw = fx_modes3(q, xw);
+    fx_t G[2][2];
+    FxMul WX[2][2], WY[2][2], WZ[2][2];
+    auto split = [&](FxMul o[2][2]) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) o[c >> 1][c & 1] = fx_split(G[c >> 1][c & 1]);
+    };
+    fx_h2_fwd(mw.S100, mw.S110, mw.S101, mw.S111, G);  // [sy][sz]
+    split(WX);
+    fx_h2_fwd(mw.S010, mw.S110, mw.S011, mw.S111, G);  // [sx][sz]
+    split(WY);
+    fx_h2_fwd(mw.S001, mw.S101, mw.S011, mw.S111, G);  // [sx][sy]
+    split(WZ);
+    const FxModes3 mu = fx_modes3(p, xu);
+    // u at the points (as in fx_nd3), and the three parts of grad u . grad w
+    FxMul U[2][2][2];
+    fx_t DX[2][2], DY[2][2], DZ[2][2];
+    auto dots = [&](const FxMul w[2][2], fx_t o[2][2]) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) o[c >> 1][c & 1] = fx_mul(fx_split(G[c >> 1][c & 1]), w[c >> 1][c & 1]);
+    };
+    fx_h2_fwd(mu.S010, mu.S110, mu.S011, mu.S111, G);
+    dots(WY, DY);
+    fx_h2_fwd(mu.S001, mu.S101, mu.S011, mu.S111, G);
+    dots(WZ, DZ);
+    fx_h2_fwd(mu.S100, mu.S110, mu.S101, mu.S111, G);
+    dots(WX, DX);
+    {
+        fx_t P0[2][2];
+        fx_h2_fwd(0, mu.S010, mu.S001, mu.S011, P0);
+        const fx_t U0 = fx_sar(fx_shl(mu.M000, 2), ep - e);
+        const int shu = mu.s - 3 + ep - e;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int i = c >> 2, j = c >> 1 & 1, l = c & 1;
+            U[i][j][l] = fx_split(U0 + fx_sar(i ? P0[j][l] + G[j][l] : P0[j][l] - G[j][l], shu));
+        }
+    }
+    const fx_t one = (f > 60 ? 0 : (fx_t)1 << (60 - f)) + (fx_t)0x40000000LL;  // (see fx_nd3)
+    fx_t K[2][2][2], S[2][2][2];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const int i = c >> 2, j = c >> 1 & 1, l = c & 1;
+        const FxMul u = U[i][j][l];
+        const int uh = u.h * 4;
+        K[i][j][l] = one + ((fx_t)uh * uh + (fx_t)(fx_mulhi_s(uh, u.l) * 2) * 4);
+        S[i][j][l] = fx_mul(fx_split(fx_shl(DX[j][l] + DY[i][l] + DZ[i][j], 2)), u);
+    }
+    auto ksum = [](fx_t a, fx_t b) -> FxMul {
+        const fx_t c = a + b;
+        return {fx_hi(c), (int)(fx_lo(c) ^ 0x80000000u)};
+    };
+    fx_t FX[2][2], FY[2][2], FZ[2][2], E0[2][2], E1[2][2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            FX[i][j] = fx_mul(WX[i][j], ksum(K[1][i][j], K[0][i][j]));  // [sy][sz]
+            FY[i][j] = fx_mul(WY[i][j], ksum(K[i][1][j], K[i][0][j]));  // [sx][sz]
+            FZ[i][j] = fx_mul(WZ[i][j], ksum(K[i][j][1], K[i][j][0]));  // [sx][sy]
+            E0[i][j] = S[i][j][1] + S[i][j][0];
+            E1[i][j] = S[i][j][1] - S[i][j][0];
+        }
+    fx_t X00, X10, X01, X11, Y00, Y10, Y01, Y11, Z00, Z10, Z01, Z11;
+    fx_h2_adj(FX, X00, X10, X01, X11);  // X_qr
+    fx_h2_adj(FY, Y00, Y10, Y01, Y11);  // Y_pr
+    fx_h2_adj(FZ, Z00, Z10, Z01, Z11);  // Z_pq
+    fx_t E000, E100, E010, E110, E001, E101, E011, E111;
+    fx_h2_adj(E0, E000, E100, E010, E110);
+    fx_h2_adj(E1, E001, E101, E011, E111);
+    // exponents of the flux modes and of twice the source modes; the common one
+    const int xf = 2 + f - mw.k - mw.s, xs = 63 + ep - mw.k - mw.s - mu.k - mu.s;
+    const int xc = (xf > xs ? xf : xs) + 1;
+    const int hf = xc - xf, hs = xc - xs;
+    const fx_t R000 = fx_shl(fx_mul(fx_sar(E000, hs), sc.b0), 1);
+    const fx_t R100 = fx_mul(fx_sar(X00, hf) + fx_sar(E100, hs), sc.b1);
+    const fx_t R010 = fx_mul(fx_sar(Y00, hf) + fx_sar(E010, hs), sc.b1);
+    const fx_t R001 = fx_mul(fx_sar(Z00, hf) + fx_sar(E001, hs), sc.b1);
+    const fx_t R110 = fx_mul(fx_sar(X10 + Y10, hf) + fx_sar(E110, hs), sc.b2);
+    const fx_t R101 = fx_mul(fx_sar(X01 + Z10, hf) + fx_sar(E101, hs), sc.b2);
+    const fx_t R011 = fx_mul(fx_sar(Y01 + Z01, hf) + fx_sar(E011, hs), sc.b2);
+    const fx_t R111 = fx_mul(fx_sar(X11 + Y11 + Z11, hf) + fx_sar(E111, hs), sc.b3);
+    const fx_t e00_0 = R000 - R001, e00_1 = R000 + R001, e01_0 = R010 - R011, e01_1 = R010 + R011;
+    const fx_t e10_0 = R100 - R101, e10_1 = R100 + R101, e11_0 = R110 - R111, e11_1 = R110 + R111;
+    const fx_t f0_00 = e00_0 - e01_0, f0_10 = e00_0 + e01_0, f0_01 = e00_1 - e01_1, f0_11 = e00_1 + e01_1;
+    const fx_t f1_00 = e10_0 - e11_0, f1_10 = e10_0 + e11_0, f1_01 = e10_1 - e11_1, f1_11 = e10_1 + e11_1;
+    r[0] = f0_00 - f1_00; r[1] = f0_00 + f1_00;
+    r[2] = f0_10 - f1_10; r[3] = f0_10 + f1_10;
+    r[4] = f0_01 - f1_01; r[5] = f0_01 + f1_01;
+    r[6] = f0_11 - f1_11; r[7] = f0_11 + f1_11;
+    X = sc.ex + 1 + xc;
 }
 
 // ---------------------------------------------------------------------------

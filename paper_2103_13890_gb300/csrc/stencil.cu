@@ -200,7 +200,7 @@ template <typename T>
 static jfnk_status launch_stencil_impl(Prob prob, Mode mode, const StencilArgs<T>& a, cudaStream_t st) {
     if (prob == Prob::BEAM3) return launch_beam<T>(mode, a, st);
     if constexpr (sizeof(T) == 8) {
-        if (!is_2d(prob) && fx3d_use(a, mode)) return launch_fx3d(prob, mode, a, st);
+        if (!is_2d(prob) && fx3d_use(a, mode, false)) return launch_fx3d(prob, mode, false, a, st);
     }
     if constexpr (sizeof(T) == 4) {
         if (!is_2d(prob) && t3d_use(a, mode, false)) return launch_t3d(prob, mode, false, a, st);

@@ -1,5 +1,5 @@
-// FP64 residual of the 3D diffusion problems, element arithmetic in 64-bit
-// fixed point (fx64.cuh).
+// FP64 residual and vector-Jacobian product of the 3D diffusion problems, element
+// arithmetic in 64-bit fixed point (fx64.cuh).
 //
 // One launch per action.  A CTA takes a tile of element columns and marches it
 // along z; thread (tx, ty) evaluates one element per layer.  The values
@@ -30,11 +30,7 @@
 
 namespace jfnk {
 
-#ifndef FX_T
-#define FX_T 288
-#define FX_B 2
-#endif
-constexpr int kFxThreads = FX_T, kFxBlocks = FX_B;  // largest CTA, CTAs per SM
+constexpr int kFxThreads = 288, kFxBlocks = 2;  // largest CTA, CTAs per SM
 
 // FP64 evaluation of the element at (x, y, z), for values outside the
 // fixed-point range (non-finite or huge values, magnitudes near underflow,
@@ -55,7 +51,28 @@ __device__ __noinline__ void nd3_fp64(const StencilArgs<double>& a, double eps, 
     for (int c = 0; c < 8; ++c) r[c] *= a.node_scale;
 }
 
-template <Prob P, Mode M>
+// The same for the vector-Jacobian product, w = v at the unknowns.
+template <bool KAPPA>
+__device__ __noinline__ void vjp3_fp64(const StencilArgs<double>& a, int x, int y, int z, double kap, double* r) {
+    const int n = a.g.n;
+    double u[8], w[8], dk;
+    for (int c = 0; c < 8; ++c) {
+        const int X = x + (c & 1), Y = y + ((c >> 1) & 1), Z = z + (c >> 2);
+        const long long i = JFNK_IDX((long long)Z * a.g.sz + (long long)Y * a.g.sy + X, a.g.size);
+        const bool bnd = X == 0 || X == n || Y == 0 || Y == n || Z == 0 || Z == n;
+        u[c] = a.u[i];
+        w[c] = bnd ? 0.0 : a.v[i];
+    }
+    elem_vjp3<double>(u, w, kap, r, dk);
+    for (int c = 0; c < 8; ++c) r[c] *= a.node_scale;
+}
+
+// ADJ: J^T v in place of the FD action; the planes of v are staged beside those
+// of u.  About 1.8 times the instructions of a residual: 129^3 with kappa 0.228 ms
+// against 1.068 ms of the FP64-pipe kernels, 257^3 1.54 against 8.43 ms.  (96
+// registers spill some 20 values; one CTA an SM with 168 registers and none: 0.250
+// and 1.78 ms.)
+template <Prob P, Mode M, bool ADJ>
 __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx3d_kernel(const StencilArgs<double> a) {
     const FxTiling& t = a.fx;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -64,11 +81,12 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx3d_kernel(const Stenc
     const int n = a.g.n;
     const int sy = (int)a.g.sy, sz = (int)a.g.sz;
     const int npx = t.ex + 1, np = npx * (t.ey + 1), ne = t.ex * t.ey;
-    fx_t* const W = reinterpret_cast<fx_t*>(smem_raw);       // [2][np] node planes, packed values
-    double* const C = reinterpret_cast<double*>(W + 2 * np);                         // [2][3][ne] contributions to the neighbour columns
+    fx_t* const W = reinterpret_cast<fx_t*>(smem_raw);        // [2][np] node planes, packed values
+    fx_t* const V = W + (ADJ ? 2 * np : 0);                   // [2][np] those of the direction (ADJ)
+    double* const C = reinterpret_cast<double*>(V + 2 * np);  // [2][3][ne] contributions to the neighbour columns
     const int tid = threadIdx.x;
     double eps = 0.0, inv_eps = 0.0;
-    if (M != Mode::F) {
+    if (!ADJ && M != Mode::F) {
         eps = eps_of<double>(a.eps);
         inv_eps = inv_eps_of<double>(a.eps);
     }
@@ -108,15 +126,20 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx3d_kernel(const Stenc
         };
         auto store = [&](int z) {
             if (!stage) return;
-            W[(z & 1) * np + tid] = fx_pack(M != Mode::F ? fma(eps, rv, ru) : ru);
+            W[(z & 1) * np + tid] = fx_pack(!ADJ && M != Mode::F ? fma(eps, rv, ru) : ru);
+            if (ADJ) V[(z & 1) * np + tid] = fx_pack(rv);
             // Dirichlet nodes: every output is zero
-            if (edge || z == 0 || z == n)
-                epilogue<double, M>(a, z * sz + sidx, false, 0.0, 0.0, ck, red);
+            if (edge || z == 0 || z == n) {
+                if (ADJ)
+                    epilogue_adj<double, M>(a, z * sz + sidx, false, 0.0, ck, red);
+                else
+                    epilogue<double, M>(a, z * sz + sidx, false, 0.0, 0.0, ck, red);
+            }
         };
-        fx_t p[8], carry[4] = {0, 0, 0, 0};  // corners; contributions to the upper face ...
-        int xl = 0, Xc = kFxTiny;            // ... times 2^Xc, or doubles (kFxFp64)
-        auto face = [&](int z, fx_t* q) -> int {
-            const fx_t* Wz = W + (z & 1) * np + corner;
+        fx_t p[8], pv[ADJ ? 8 : 1], carry[4] = {0, 0, 0, 0};  // corners; contributions to the upper face ...
+        int xl = 0, xvl = 0, Xc = kFxTiny;   // ... times 2^Xc, or doubles (kFxFp64)
+        auto face = [&](const fx_t* plane, int z, fx_t* q) -> int {
+            const fx_t* Wz = plane + (z & 1) * np + corner;
             q[0] = Wz[0];
             q[1] = Wz[1];
             q[2] = Wz[npx];
@@ -128,33 +151,39 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx3d_kernel(const Stenc
         fetch(za);
         store(za);
         __syncthreads();
-        if (elem) xl = face(za - 1, p);
+        if (elem) xl = face(W, za - 1, p);
+        if (ADJ && elem) xvl = face(V, za - 1, pv);
         __syncthreads();  // plane za - 1 is read before plane za + 1 takes its place
         for (int k = za - 1; k < zb; ++k) {
             if (k + 2 <= zb) fetch(k + 2);
             const bool out = node && k >= za;
             EpiIn1<double> e;
-            if (out) epi1_load<double, M>(a, (long long)k * sz + gidx, e);
+            if (!ADJ && out) epi1_load<double, M>(a, (long long)k * sz + gidx, e);
             double q = 0.0;
             if (elem) {
-                const int xu = face(k + 1, p + 4);
+                const int xu = face(W, k + 1, p + 4);
+                const int xvu = ADJ ? face(V, k + 1, pv + 4) : 0;
                 double kap = 1.0;
                 if (KAPPA) kap = a.kappa[JFNK_IDX(k * n * n + eidx, (long long)n * n * n)];
-                const int xm = max(xl, xu);
-                const bool fits = fx_exp_ok(xm) && (!KAPPA || fx_scale_ok(kap));
+                const int xm = max(xl, xu), xv = max(xvl, xvu);
+                const bool fits = (ADJ ? xm < kFxMaxExp && fx_exp_ok(xv) : fx_exp_ok(xm)) && (!KAPPA || fx_scale_ok(kap));
                 fx_t r[8];
                 int Xr = kFxTiny;
                 if (fits) {
-                    if (KAPPA)
-                        fx_nd3(p, xm, fx_scale_kappa(sc0, kap), r, Xr);
+                    const FxScale sc = KAPPA ? fx_scale_kappa(sc0, kap) : sc0;
+                    if (ADJ)
+                        fx_vjp3(p, xm, pv, xv, sc, r, Xr);
                     else
-                        fx_nd3(p, xm, sc0, r, Xr);
+                        fx_nd3(p, xm, sc, r, Xr);
                 } else {
 #pragma unroll
                     for (int c = 0; c < 8; ++c) r[c] = 0;
-                    if (xm != 0) {
+                    if (ADJ ? xv != 0 || xm == kFxBad : xm != 0) {
                         double rs[8];
-                        nd3_fp64<KAPPA, M != Mode::F>(a, eps, gx, gy, k, kap, rs);
+                        if (ADJ)
+                            vjp3_fp64<KAPPA>(a, gx, gy, k, kap, rs);
+                        else
+                            nd3_fp64<KAPPA, M != Mode::F>(a, eps, gx, gy, k, kap, rs);
 #pragma unroll
                         for (int c = 0; c < 8; ++c) r[c] = __double_as_longlong(rs[c]);
                         Xr = kFxFp64;
@@ -181,16 +210,21 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx3d_kernel(const Stenc
                 for (int c = 0; c < 4; ++c) {
                     carry[c] = r[4 + c];
                     p[c] = p[4 + c];
+                    if (ADJ) pv[c] = pv[4 + c];
                 }
                 Xc = Xr;
                 xl = xu;
+                xvl = xvu;
             }
             if (k + 2 <= zb) store(k + 2);
             __syncthreads();
             if (out) {
                 const double* Ck = C + (k & 1) * 3 * ne + tid;
                 const double val = (q + Ck[-1]) + (Ck[ne - t.ex] + Ck[2 * ne - t.ex - 1]);
-                epilogue_pf<double, M>(a, (long long)k * sz + gidx, true, val, inv_eps, ck, e, red);
+                if (ADJ)
+                    epilogue_adj<double, M>(a, (long long)k * sz + gidx, true, val, ck, red);
+                else
+                    epilogue_pf<double, M>(a, (long long)k * sz + gidx, true, val, inv_eps, ck, e, red);
             }
         }
     }
@@ -257,36 +291,41 @@ bool fx_outputs_alias(const StencilArgs<T>& a, Mode mode) {
 template bool fx_outputs_alias<double>(const StencilArgs<double>&, Mode);
 template bool fx_outputs_alias<float>(const StencilArgs<float>&, Mode);
 
-bool fx3d_use(const StencilArgs<double>& a, Mode mode) {
-    return a.fx.ctas > 0 && fx_scale_ok(a.node_scale) && !fx_outputs_alias(a, mode);
+bool fx3d_use(const StencilArgs<double>& a, Mode mode, bool adj) {
+    return a.fx.ctas > 0 && fx_scale_ok(a.node_scale) && !(adj && (a.dkout || mode == Mode::F)) &&
+           !fx_outputs_alias(a, mode);
 }
 
-template <Prob P, Mode M>
+template <Prob P, Mode M, bool ADJ>
 static jfnk_status launch_fx3d_pm(const StencilArgs<double>& a, cudaStream_t st) {
     const FxTiling& t = a.fx;
-    const size_t smem = sizeof(double) * (2 * (size_t)(t.ex + 1) * (t.ey + 1) + 6 * (size_t)t.ex * t.ey);
-    fx3d_kernel<P, M><<<t.ctas, t.threads, smem, st>>>(a);
+    const size_t smem = sizeof(double) * ((ADJ ? 4 : 2) * (size_t)(t.ex + 1) * (t.ey + 1) + 6 * (size_t)t.ex * t.ey);
+    fx3d_kernel<P, M, ADJ><<<t.ctas, t.threads, smem, st>>>(a);
     JFNK_LAUNCH_CHECK();
     return JFNK_OK;
 }
 
-template <Prob P>
+template <Prob P, bool ADJ>
 static jfnk_status launch_fx3d_p(Mode mode, const StencilArgs<double>& a, cudaStream_t st) {
     switch (mode) {
-        case Mode::F: return launch_fx3d_pm<P, Mode::F>(a, st);
-        case Mode::JV: return launch_fx3d_pm<P, Mode::JV>(a, st);
-        case Mode::BMJ: return launch_fx3d_pm<P, Mode::BMJ>(a, st);
-        case Mode::CHEB0: return launch_fx3d_pm<P, Mode::CHEB0>(a, st);
-        case Mode::CHEB: return launch_fx3d_pm<P, Mode::CHEB>(a, st);
-        case Mode::CHEBLAST: return launch_fx3d_pm<P, Mode::CHEBLAST>(a, st);
+        case Mode::F:
+            if constexpr (!ADJ) return launch_fx3d_pm<P, Mode::F, false>(a, st);
+            break;
+        case Mode::JV: return launch_fx3d_pm<P, Mode::JV, ADJ>(a, st);
+        case Mode::BMJ: return launch_fx3d_pm<P, Mode::BMJ, ADJ>(a, st);
+        case Mode::CHEB0: return launch_fx3d_pm<P, Mode::CHEB0, ADJ>(a, st);
+        case Mode::CHEB: return launch_fx3d_pm<P, Mode::CHEB, ADJ>(a, st);
+        case Mode::CHEBLAST: return launch_fx3d_pm<P, Mode::CHEBLAST, ADJ>(a, st);
     }
     set_error("unknown stencil mode");
     return JFNK_ERR_INVALID_ARG;
 }
 
-jfnk_status launch_fx3d(Prob prob, Mode mode, const StencilArgs<double>& a, cudaStream_t st) {
-    if (prob == Prob::ND3) return launch_fx3d_p<Prob::ND3>(mode, a, st);
-    if (prob == Prob::NDK3) return launch_fx3d_p<Prob::NDK3>(mode, a, st);
+jfnk_status launch_fx3d(Prob prob, Mode mode, bool adj, const StencilArgs<double>& a, cudaStream_t st) {
+    if (prob == Prob::ND3)
+        return adj ? launch_fx3d_p<Prob::ND3, true>(mode, a, st) : launch_fx3d_p<Prob::ND3, false>(mode, a, st);
+    if (prob == Prob::NDK3)
+        return adj ? launch_fx3d_p<Prob::NDK3, true>(mode, a, st) : launch_fx3d_p<Prob::NDK3, false>(mode, a, st);
     set_error("the fixed-point kernels evaluate the 3D diffusion problems only");
     return JFNK_ERR_INVALID_ARG;
 }

@@ -1,4 +1,4 @@
-// FP64 residual kernels of the 3D diffusion problems with the element
+// FP64 kernels of the 3D diffusion problems with the element
 // arithmetic in 64-bit fixed point (fx64.cuh): one launch per action, no
 // scratch.
 #pragma once
@@ -17,9 +17,10 @@ bool fx_outputs_alias(const StencilArgs<T>& a, Mode mode);
 
 // True when the fixed-point kernel takes this FP64 call: a.fx is set, and the
 // outputs are apart from the vectors whose neighbouring values other threads
-// still read.
-bool fx3d_use(const StencilArgs<double>& a, Mode mode);
+// still read.  adj: the vector-Jacobian product (not with the coefficient's
+// derivative).
+bool fx3d_use(const StencilArgs<double>& a, Mode mode, bool adj);
 
-jfnk_status launch_fx3d(Prob prob, Mode mode, const StencilArgs<double>& a, cudaStream_t st);
+jfnk_status launch_fx3d(Prob prob, Mode mode, bool adj, const StencilArgs<double>& a, cudaStream_t st);
 
 }  // namespace jfnk

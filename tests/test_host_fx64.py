@@ -1,6 +1,6 @@
 """Host-side checks of the fixed-point element arithmetic (no GPU): C++ programs
 compiled with overflow checks compare it with the FP64 elements and a long
-double quadrature (tests/host/fx64_check.cpp, fx_beam_check.cpp)."""
+double quadrature (tests/host/fx64_check.cpp, fx_vjp_check.cpp, fx_beam_check.cpp)."""
 import os
 import shutil
 import subprocess
@@ -10,7 +10,7 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-@pytest.mark.parametrize("check", ["fx64_check", "fx_beam_check"])
+@pytest.mark.parametrize("check", ["fx64_check", "fx_vjp_check", "fx_beam_check"])
 def test_fixed_point_element(check, tmp_path):
     gxx = shutil.which("g++")
     if gxx is None:
