@@ -4,10 +4,23 @@
 // residual estimate is <= tol ||r0|| (relative reading) or <= tol (absolute),
 // or after maxit iterations (Sec. 3: maxit = number of coarse unknowns).
 //
-// The coarse grid is tiny (<= JFNK_COARSE_MAX_NODES nodes), so the whole
-// solve runs in ONE CTA: the FD Jacobian action (element loop into shared
-// memory, node gather), classical Gram-Schmidt applied twice, Givens rotations
-// and the back-substitution, with no kernel launches or host round-trips.
+// The coarse grid is tiny (<= JFNK_COARSE_MAX_NODES nodes), so the whole solve
+// runs in ONE CTA, without kernel launches or host round trips, and an iteration
+// is a chain of latencies: barriers, shared-memory reads and dependent FP64
+// operations (64 clocks each for one thread).  Hence
+//   - the basis holds the unknowns only, and its vectors have unit norm, so
+//     that the FD step is the same for all of them;
+//   - 8 lanes form a dot product (32 on the larger coarse grids), so that one
+//     round of the warps covers a Gram-Schmidt pass;
+//   - the Givens rotations of column j, serial FP64 arithmetic, run in a warp of
+//     their own while the other warps form the products of iteration j + 1.  The
+//     solve stops one (discarded) iteration after the column that meets the
+//     tolerance;
+//   - six barriers an iteration, five of them among the computing warps only.
+// Measured (default tolerance; before: a block-wide norm per basis vector, warp-wide
+// dot products and the rotations by one thread between the barriers): 5^3 nodes 105
+// -> 33 us in FP32 and 171 -> 67 us in FP64, 9^2 nodes 299 -> 74 and 437 -> 140 us,
+// 10^3 nodes 670 -> 230 and 1798 -> 719 us.
 #include "coarse.cuh"
 #include "coarse_elem.cuh"
 #include "element.cuh"
@@ -16,130 +29,148 @@
 
 namespace jfnk {
 
-constexpr int kCoarseThreads = 512;
-
-// Threads of the one-CTA coarse solvers: about one per node, in whole warps,
-// 64 to 512 (block-wide reductions and barriers dominate on the small coarse
-// grids, and they are cheaper with fewer warps).
+// Threads of the one-CTA coarse solvers: the computing warps, one thread per
+// node, 256 (32 dot products of 8 lanes at once) to 480, and the warp of the
+// Givens rotations.
+constexpr int kCoarseMinThreads = 256, kCoarseMaxThreads = 480, kCoarseGivens = 32;
 static int coarse_threads(const Grid& g) {
     const long long t = ((g.size + 31) / 32) * 32;
-    return (int)(t < 64 ? 64 : (t > kCoarseThreads ? kCoarseThreads : t));
+    return (int)(t < kCoarseMinThreads ? kCoarseMinThreads : (t > kCoarseMaxThreads ? kCoarseMaxThreads : t)) +
+           kCoarseGivens;
 }
 
-template <typename T, Prob P>
-__device__ void coarse_apply_A(const Grid& g, const T* w, T* elemC, T* out, const T* kappa, T lh,
-                               T node_scale, const CoarseElem<T, P>& ce) {
-    // elemC: [nelem][npe];  out: A(w) scaled, full grid (boundary entries untouched)
-    const int n = g.n;
-    const int tid = threadIdx.x;
-    if (P == Prob::BEAM3) {
-        // lh = 1/h; 10n x n x n elements, 3 components per node
-        const int ex = 10 * n, ne = ex * n * n;
-        for (int e = tid; e < ne; e += blockDim.x) {
-            const int x = e % ex, y = (e / ex) % n, z = e / (ex * n);
-            coarse_element<T, P>(g, w, x, y, z, T(1), lh, ce, elemC + e * 24);
-        }
-        __syncthreads();
-        for (long long k = tid; k < g.size; k += blockDim.x) {
-            const int i = (int)(k % 3);
-            const int node = (int)(k / 3);
-            const int X = node % g.nx, Y = (node / g.nx) % g.ny, Z = node / (g.nx * g.ny);
-            T acc = T(0);
+// Barrier of the nc computing threads.
+__device__ __forceinline__ void coarse_sync(int nc) { asm volatile("bar.sync 1, %0;" ::"r"(nc) : "memory"); }
+
+// Element contributions of the coarse grid, C[c * ne + e]: of A(w), or (ADJ) of
+// J(x)^T w.  eoff[e]: where the element's first node is
+// in the vectors.
+template <typename T, Prob P, bool ADJ>
+__device__ __forceinline__ void coarse_elements(const Grid& g, const T* x, const T* w, const unsigned short* eoff, T* C,
+                                                int ne, const T* kappa, T lh, const CoarseElem<T, P>& ce, int nc) {
+    for (int e = threadIdx.x; e < ne; e += nc) {
+        const T kap = P == Prob::NDK3 ? kappa[e] : T(1);
+        if constexpr (ADJ) {
+            const int sy = (int)g.sy, sz = (int)g.sz;
+            T ue[8], ve[8], r[8], dk;
+#pragma unroll
             for (int c = 0; c < 8; ++c) {
-                const int xe = X - (c & 1), ye = Y - ((c >> 1) & 1), ze = Z - (c >> 2);
-                if (xe < 0 || xe >= ex || ye < 0 || ye >= n || ze < 0 || ze >= n) continue;
-                acc += elemC[((ze * n + ye) * ex + xe) * 24 + 3 * c + i];
+                const int i = eoff[e] + (c & 1) + ((c >> 1) & 1) * sy + (c >> 2) * sz;
+                ue[c] = x[i];
+                ve[c] = w[i];
             }
-            out[k] = acc;
-        }
-    } else if (is_2d(P)) {
-        const int ne = n * n;
-        for (int e = tid; e < ne; e += blockDim.x) {
-            const int ex = e % n, ey = e / n;
-            coarse_element<T, P>(g, w, ex, ey, 0, T(1), lh, ce, elemC + e * 4);
-        }
-        __syncthreads();
-        for (long long i = tid; i < g.size; i += blockDim.x) {
-            const int x = (int)(i % g.sy), y = (int)(i / g.sy);
-            T acc = T(0);
+            elem_vjp3<T>(ue, ve, kap, r, dk);
 #pragma unroll
-            for (int b = 0; b < 2; ++b)
-#pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    const int ex = x - 1 + a, ey = y - 1 + b;  // element with the node at local (1-a, 1-b)
-                    if (ex >= 0 && ex < n && ey >= 0 && ey < n) acc += elemC[(ey * n + ex) * 4 + (1 - a) + 2 * (1 - b)];
-                }
-            out[i] = acc * node_scale;
-        }
-    } else {
-        const int ne = n * n * n;
-        for (int e = tid; e < ne; e += blockDim.x) {
-            const int ex = e % n, ey = (e / n) % n, ez = e / (n * n);
-            coarse_element<T, P>(g, w, ex, ey, ez, P == Prob::NDK3 ? kappa[e] : T(1), lh, ce, elemC + e * 8);
-        }
-        __syncthreads();
-        for (long long i = tid; i < g.size; i += blockDim.x) {
-            const int x = (int)(i % g.sy);
-            const int y = (int)((i / g.sy) % g.ny);
-            const int z = (int)(i / g.sz);
-            T acc = T(0);
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int b = 0; b < 2; ++b)
-#pragma unroll
-                    for (int a = 0; a < 2; ++a) {
-                        const int ex = x - 1 + a, ey = y - 1 + b, ez = z - 1 + c;
-                        if (ex >= 0 && ex < n && ey >= 0 && ey < n && ez >= 0 && ez < n)
-                            acc += elemC[((ez * n + ey) * n + ex) * 8 + (1 - a) + 2 * (1 - b) + 4 * (1 - c)];
-                    }
-            out[i] = acc * node_scale;
+            for (int c = 0; c < 8; ++c) C[c * ne + e] = r[c];
+        } else {
+            coarse_element_at<T, P>(g, w + eoff[e], kap, lh, ce, C + e, ne);
         }
     }
-    __syncthreads();
 }
 
-// J(x)^T v on the coarse grid (3D diffusion problems), full grid out (boundary untouched)
+// Sum of the contributions to unknown i (eref: the element whose last corner it
+// is).  A scalar grid's unknown has all its elements; the beam's faces do not.
 template <typename T, Prob P>
-__device__ void coarse_apply_vjp(const Grid& g, const T* x, const T* v, T* elemC, T* out, const T* kappa,
-                                 T node_scale) {
+__device__ __forceinline__ T coarse_gather(const Grid& g, const T* C, int ne, int i, int eref) {
     const int n = g.n;
-    const int tid = threadIdx.x;
-    const int ne = n * n * n;
-    for (int e = tid; e < ne; e += blockDim.x) {
-        const int ex = e % n, ey = (e / n) % n, ez = e / (n * n);
-        const long long b = (long long)ez * g.sz + (long long)ey * g.sy + ex;
-        const long long o[8] = {0, 1, g.sy, g.sy + 1, g.sz, g.sz + 1, g.sz + g.sy, g.sz + g.sy + 1};
-        T ue[8], ve[8];
-#pragma unroll
+    T acc = T(0);
+    if constexpr (P == Prob::BEAM3) {
+        const int k = i % 3, node = i / 3, ex = 10 * n;
+        const int X = node % g.nx, Y = (node / g.nx) % g.ny, Z = node / (g.nx * g.ny);
         for (int c = 0; c < 8; ++c) {
-            ue[c] = x[b + o[c]];
-            ve[c] = v[b + o[c]];
+            const int xe = X - (c & 1), ye = Y - ((c >> 1) & 1), ze = Z - (c >> 2);
+            if (xe < 0 || xe >= ex || ye < 0 || ye >= n || ze < 0 || ze >= n) continue;
+            acc += C[(3 * c + k) * ne + (ze * n + ye) * ex + xe];
         }
-        T r[8], dk;
-        elem_vjp3<T>(ue, ve, P == Prob::NDK3 ? kappa[e] : T(1), r, dk);
+    } else if constexpr (is_2d(P)) {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) elemC[e * 8 + c] = r[c];
+        for (int c = 0; c < 4; ++c) acc += C[(3 - c) * ne + eref + (c & 1) + (c >> 1) * n];
+    } else {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc += C[(7 - c) * ne + eref + (c & 1) + ((c >> 1) & 1) * n + (c >> 2) * n * n];
     }
-    __syncthreads();
-    for (long long i = tid; i < g.size; i += blockDim.x) {
-        const int xx = (int)(i % g.sy);
-        const int yy = (int)((i / g.sy) % g.ny);
-        const int zz = (int)(i / g.sz);
-        T acc = T(0);
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int bb = 0; bb < 2; ++bb)
-#pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    const int ex = xx - 1 + a, ey = yy - 1 + bb, ez = zz - 1 + c;
-                    if (ex >= 0 && ex < n && ey >= 0 && ey < n && ez >= 0 && ez < n)
-                        acc += elemC[((ez * n + ey) * n + ex) * 8 + (1 - a) + 2 * (1 - bb) + 4 * (1 - c)];
-                }
-        out[i] = acc * node_scale;
+    return acc;
+}
+
+// 1 / sqrt(x) of a sum of squares.
+__device__ __forceinline__ float coarse_rsqrt(float x) { return 1.0f / sqrtf(x); }
+__device__ __forceinline__ double coarse_rsqrt(double x) {
+    return x >= 2.2250738585072014e-308 && x <= 1.7976931348623157e308 ? rsqrt_newton(x) : 1.0 / sqrt(x);
+}
+
+// The work of the Givens warp.  One column: the raw entries h1 + h2 (two
+// Gram-Schmidt passes) and the squared norm hn2 of what remains; applies the
+// earlier rotations, forms the new one and the residual estimate.  Returns
+// whether the iteration stops with this column.
+struct CoarseGivens {
+    double *H, *cs, *sn, *gv, *dinv, *work;  // H: column-major, m + 1 rows
+    int m;
+    double target;
+};
+template <typename T>
+__device__ bool coarse_givens(const CoarseGivens& s, int j, const T* h1, const T* h2, double hn2) {
+    const int lane = threadIdx.x & 31;
+    double* const Hj = s.H + (size_t)j * (s.m + 1);
+    // r_0 = x_0, r_(i+1) = c_i x_(i+1) - s_i r_i; the rotated entries are c_i r_i + s_i x_(i+1)
+    for (int i = lane; i <= j; i += 32) {
+        const double x = (double)h1[i] + (double)h2[i];
+        Hj[i] = x;
+        s.work[i] = i > 0 ? s.cs[i - 1] * x : x;
     }
-    __syncthreads();
+    __syncwarp();
+    double r = s.work[0];
+    if (lane == 0 && j > 0) {
+        double p = s.work[1], q = s.sn[0];  // (loaded an entry ahead of the chain)
+        for (int i = 0; i < j; ++i) {
+            const int i1 = i + 1 < j ? i + 1 : i;
+            const double p1 = s.work[i1 + 1], q1 = s.sn[i1];
+            s.work[i] = r;
+            r = fma(-q, r, p);
+            p = p1;
+            q = q1;
+        }
+    }
+    __syncwarp();
+    r = __shfl_sync(0xffffffffu, r, 0);
+    for (int i0 = 0; i0 < j; i0 += 32) {
+        const int i = i0 + lane;
+        double t = 0.0;
+        if (i < j) t = fma(s.cs[i], s.work[i], s.sn[i] * Hj[i + 1]);
+        __syncwarp();
+        if (i < j) Hj[i] = t;  // (entry i0 + 32 is still the raw one the next round reads)
+    }
+    // 1 / hypot(r, hn), and in lane 1 1 / hn
+    const double q2 = lane == 1 ? hn2 : fma(r, r, hn2);
+    double ri, hn;
+    if (__all_sync(0xffffffffu, q2 >= 1e-280 && q2 <= 1e280)) {
+        const double qi = rsqrt_newton(q2);
+        ri = __shfl_sync(0xffffffffu, qi, 0);
+        hn = hn2 * __shfl_sync(0xffffffffu, qi, 1);
+    } else {
+        hn = sqrt(hn2);
+        ri = 1.0 / hypot(r, hn);
+    }
+    double c = 1.0, sg = 0.0, d = r, di = ri;
+    if (hn != 0.0) {
+        c = r * ri;
+        sg = hn * ri;
+        d = fma(c, r, sg * hn);
+    } else {
+        di = 1.0 / r;
+    }
+    const double g = s.gv[j], gn = -sg * g;
+    __syncwarp();
+    if (lane == 0) {
+        Hj[j] = d;
+        s.cs[j] = c;
+        s.sn[j] = sg;
+        s.dinv[j] = di;
+        s.gv[j + 1] = gn;
+        s.gv[j] = c * g;
+    }
+    __syncwarp();
+    const double res = fabs(gn);
+    return res <= s.target || !(hn > 0.0) || !isfinite(res);
 }
 
 // vsm: the Krylov basis V and the Hessenberg matrix H live in shared memory
@@ -147,171 +178,240 @@ __device__ void coarse_apply_vjp(const Grid& g, const T* x, const T* v, T* elemC
 template <typename T, Prob P, bool ADJ>
 __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_raw, bool vsm) {
     const Grid g = a.g;
-    const int N = (int)g.size;
+    const int N = (int)g.size, U = (int)g.interior();
     const int ne = (int)g.elements();
     const int npe = coarse_npe(g);
     const int m = a.maxit;
-    T* wv = reinterpret_cast<T*>(smem_raw);  // [N] work vector
-    T* xw = wv + N;                          // [N] x + eps v
-    T* Aw = xw + N;                          // [N] A(x + eps v)
-    T* elemC = Aw + N;                       // [ne * npe]
-    double* hcol = reinterpret_cast<double*>(
-        (reinterpret_cast<uintptr_t>(elemC + ne * npe) + 15) & ~uintptr_t(15));  // [m + 1]
-    double* cs = hcol + (m + 1);             // [m]
-    double* sn = cs + m;                     // [m]
-    double* gv = sn + m;                     // [m + 1]
-    double* red = gv + (m + 1);              // [32]
-    __shared__ double s_scalar[4];
-    __shared__ int s_flag;
-    const int tid = threadIdx.x;
-    const int nwarps = blockDim.x >> 5;
-    const int lane = tid & 31, wid = tid >> 5;
-    T* V = a.V;       // (m + 1) x N
-    double* H = a.H;  // (m + 1) x m, column-major: H[j * (m+1) + i]
+    CoarseGivens gs;
+    gs.m = m;
+    gs.cs = reinterpret_cast<double*>(smem_raw);  // [m]
+    gs.sn = gs.cs + m;                            // [m]
+    gs.dinv = gs.sn + m;                          // [m]
+    gs.gv = gs.dinv + m;                          // [m + 1]
+    gs.work = gs.gv + (m + 1);                    // [m + 1]
+    double* const red = gs.work + (m + 1);        // [32]
+    gs.H = a.H;
+    double* end = red + 32;
     if (vsm) {
-        H = red + 32;
-        V = reinterpret_cast<T*>(H + (size_t)(m + 1) * m);
+        gs.H = end;
+        end += (size_t)(m + 1) * m;
     }
+    T* const x = reinterpret_cast<T*>(end);  // [N] x_0
+    T* const xw = x + N;                     // [N] x_0 + eps v (ADJ: v)
+    T* const Ax = xw + N;                    // [U] A(x_0)
+    T* const wv = Ax + U;                    // [U] work vector
+    T* const hp = wv + U;                    // [2][2][m + 1] dot products by column parity and pass
+    T* const C = hp + 4 * (m + 1);           // [npe * ne]
+    T* const V = vsm ? C + npe * ne : a.V;   // [m + 1][U]
+    unsigned short* const idx = reinterpret_cast<unsigned short*>(vsm ? V + (size_t)(m + 1) * U : C + npe * ne);
+    unsigned short* const eref = idx + U;    // [U]
+    unsigned short* const eoff = eref + U;   // [ne]
+    __shared__ double s_hn2[2];
+    __shared__ int s_flag[2];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int nc = blockDim.x - kCoarseGivens, nw = nc >> 5;
+    const bool comp = tid < nc;
 
-    // ||b|| over interior; V_0 = b / ||b||
+    // ||b|| over the unknowns; V_0 = b / ||b||
     double acc = 0.0;
     for (int i = tid; i < N; i += blockDim.x)
         if (coarse_inner(g, i)) acc += (double)a.b[i] * (double)a.b[i];
-    double bn = block_sum(acc, red);
-    if (tid == 0) s_scalar[0] = sqrt(bn);
+    __shared__ double s_beta[2], s_eps[2];
+    if (tid == 32) {  // the FD step of a unit vector
+        const double e = eps_formula(a.eps_mode, a.n_unknowns, *a.xstat, 1.0);
+        s_eps[0] = e;
+        s_eps[1] = e > 0.0 ? 1.0 / e : 0.0;
+    }
+    const double bn = block_sum(acc, red);
+    if (tid == 0) {
+        s_beta[0] = sqrt(bn);
+        s_beta[1] = 1.0 / s_beta[0];
+    }
     __syncthreads();
-    const double beta = s_scalar[0];
+    const double beta = s_beta[0];
     const double target = a.tol_abs ? a.tol : a.tol * beta;
-    int k = 0;
+    gs.target = target;
     if (!(beta > 0.0) || beta <= target) {
         for (int i = tid; i < N; i += blockDim.x) a.s[i] = T(0);
         return;
     }
-    for (int i = tid; i < N; i += blockDim.x) V[i] = coarse_inner(g, i) ? (T)((double)a.b[i] / beta) : T(0);
-    if (tid == 0) {
-        gv[0] = beta;
-        for (int j = 1; j <= m; ++j) gv[j] = 0.0;
-        s_flag = 0;
+    if (wid == nw) {  // the unknowns in order
+        int base = 0;
+        for (int i0 = 0; i0 < N; i0 += 32) {
+            const int i = i0 + lane;
+            const bool in = i < N && coarse_inner(g, i);
+            const unsigned int mask = __ballot_sync(0xffffffffu, in);
+            if (in) {
+                const int u = base + __popc(mask & ((1u << lane) - 1));
+                const int X = i % g.nx, Y = (i / g.nx) % g.ny, Z = i / (g.nx * g.ny);
+                idx[u] = (unsigned short)i;
+                eref[u] = P == Prob::BEAM3 ? 0 : (unsigned short)(((g.d == 3 ? Z - 1 : 0) * g.n + Y - 1) * g.n + X - 1);
+            }
+            base += __popc(mask);
+        }
+        for (int j = lane; j <= m; j += 32) gs.gv[j] = j == 0 ? beta : 0.0;
+    } else {
+        const int ex = P == Prob::BEAM3 ? 10 * g.n : g.n;
+        for (int e = tid; e < ne; e += nc) {
+            const int X = e % ex, Y = (e / ex) % g.n, Z = e / (ex * g.n);
+            eoff[e] = (unsigned short)(P == Prob::BEAM3 ? 3 * ((Z * g.ny + Y) * g.nx + X) : Z * (int)g.sz + Y * (int)g.sy + X);
+        }
+        for (int i = tid; i < N; i += nc) {
+            x[i] = a.x[i];
+            xw[i] = ADJ ? T(0) : a.x[i];
+        }
     }
     __syncthreads();
-    const double xstat = *a.xstat;
+    const T eps = (T)s_eps[0], inv_eps = (T)s_eps[1];
+    if (comp) {
+        const double bi = s_beta[1];
+        for (int u = tid; u < U; u += nc) {
+            const int i = idx[u];
+            const T v = (T)((double)a.b[i] * bi);
+            V[u] = v;
+            if (!ADJ) Ax[u] = a.Ax[i];
+            xw[i] = ADJ ? v : x[i] + eps * v;
+        }
+    }
+    __syncthreads();
     const CoarseElem<T, P> ce(a.lh);
+    const int lg = U <= 128 ? 3 : 5, dl = 1 << lg;  // lanes of a dot product
+    constexpr int LU = sizeof(T) == 8 ? 2 : 1;      // lanes of an unknown's update
+    int k = 0;
+    // (dots and updates in the basis precision T: in an FP32 preconditioner the
+    // single CTA would otherwise spend its iterations on this SM's FP64 pipe,
+    // 1/74 of the FP32 rate; the Hessenberg entries are kept in FP64)
     for (int j = 0; j < m; ++j) {
-        const T* vj = V + (long long)j * N;
-        // ||v_j|| (unit up to rounding) and the FD step
-        T vacc = T(0);
-        for (int i = tid; i < N; i += blockDim.x)
-            if (coarse_inner(g, i)) vacc += vj[i] * vj[i];
-        double vn2 = block_sum(vacc, red);
-        if (tid == 0) {
-            double e = eps_formula(a.eps_mode, a.n_unknowns, xstat, sqrt(vn2));
-            s_scalar[1] = e;
-            s_scalar[2] = e > 0.0 ? 1.0 / e : 0.0;
-        }
-        __syncthreads();
-        if (ADJ) {
-            // adjoint operator: J(x_0)^T v_j, exact, element by element
-            for (int i = tid; i < N; i += blockDim.x) xw[i] = coarse_inner(g, i) ? vj[i] : T(0);
-            __syncthreads();
-            coarse_apply_vjp<T, P>(g, a.x, xw, elemC, Aw, a.kappa, a.node_scale);
-            for (int i = tid; i < N; i += blockDim.x) wv[i] = coarse_inner(g, i) ? Aw[i] : T(0);
-        } else {
-            const T eps = (T)s_scalar[1], inv_eps = (T)s_scalar[2];
-            for (int i = tid; i < N; i += blockDim.x) xw[i] = a.x[i] + (coarse_inner(g, i) ? eps * vj[i] : T(0));
-            __syncthreads();
-            coarse_apply_A<T, P>(g, xw, elemC, Aw, a.kappa, a.lh, a.node_scale, ce);
-            for (int i = tid; i < N; i += blockDim.x) wv[i] = coarse_inner(g, i) ? (Aw[i] - a.Ax[i]) * inv_eps : T(0);
-        }
-        __syncthreads();
-        // classical Gram-Schmidt, twice; h accumulated in hcol
-        for (int i = tid; i <= j; i += blockDim.x) hcol[i] = 0.0;
-        __syncthreads();
-        // (dots and updates in the basis precision T: in an FP32 preconditioner the
-        // single CTA would otherwise spend its iterations on this SM's FP64 pipe,
-        // 1/74 of the FP32 rate; the Hessenberg entries are kept in FP64)
-        for (int pass = 0; pass < 2; ++pass) {
-            for (int q = wid; q <= j; q += nwarps) {
-                const T* vq = V + (long long)q * N;
-                T d = T(0);
-                for (int i = lane; i < N; i += 32) d += wv[i] * vq[i];
-                d = warp_sum(d);
-                if (lane == 0) {
-                    hcol[q] += (double)d;
-                    H[(long long)j * (m + 1) + q] = (double)d;
+        T* const hj = hp + (j & 1) * 2 * (m + 1);
+        if (comp) {
+            coarse_elements<T, P, ADJ>(g, x, xw, eoff, C, ne, a.kappa, a.lh, ce, nc);
+            coarse_sync(nc);
+            for (int u = tid; u < U; u += nc) {
+                T w = coarse_gather<T, P>(g, C, ne, idx[u], eref[u]);
+                if (P != Prob::BEAM3) w *= a.node_scale;
+                wv[u] = ADJ ? w : (w - Ax[u]) * inv_eps;
+            }
+            coarse_sync(nc);
+            // classical Gram-Schmidt, twice
+            T n2 = T(0);
+            for (int pass = 0; pass < 2; ++pass) {
+                T* const h = hj + pass * (m + 1);
+                for (int q0 = wid * (32 >> lg); q0 <= j; q0 += nw * (32 >> lg)) {
+                    const int q = q0 + (lane >> lg);
+                    T d = T(0);
+                    if (q <= j) {
+                        const T* const vq = V + q * U;
+                        for (int u = lane & (dl - 1); u < U; u += dl) d += wv[u] * vq[u];
+                    }
+                    for (int o = dl >> 1; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+                    if (q <= j && (lane & (dl - 1)) == 0) h[q] = d;
+                }
+                coarse_sync(nc);
+                for (int u0 = 0; u0 < U; u0 += nc / LU) {
+                    const int u = u0 + tid / LU;
+                    if (u0 + wid * (32 / LU) >= U) continue;  // (whole warps)
+                    const T* const vu = V + (u < U ? u : 0);
+                    T s0 = T(0), s1 = T(0);
+                    int q = tid % LU;
+                    for (; q + LU <= j; q += 2 * LU) {
+                        s0 += h[q] * vu[q * U];
+                        s1 += h[q + LU] * vu[(q + LU) * U];
+                    }
+                    if (q <= j) s0 += h[q] * vu[q * U];
+                    s0 += s1;
+                    if (LU == 2) s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+                    if (u < U && tid % LU == 0) {
+                        const T w = wv[u] - s0;
+                        wv[u] = w;
+                        if (pass == 1) n2 += w * w;
+                    }
+                }
+                if (pass == 0) coarse_sync(nc);
+            }
+            // the squared norm of what remains
+            const int nwu = min(nw, (U * LU + 31) / 32);  // warps with unknowns
+            if (wid < nwu) {
+                n2 = warp_sum(n2);
+                if (lane == 0) red[wid] = (double)n2;
+            }
+            coarse_sync(nc);
+            T hn2;
+            if (sizeof(T) == 8) {
+                double t = red[0];
+                for (int w = 1; w < nwu; ++w) t += red[w];
+                hn2 = (T)t;
+            } else {
+                hn2 = (T)red[0];
+                for (int w = 1; w < nwu; ++w) hn2 += (T)red[w];
+            }
+            if (tid == 0) s_hn2[j & 1] = (double)hn2;
+            if (j + 1 < m && tid < U) {
+                const T hinv = coarse_rsqrt(hn2);
+                T* const vn = V + (j + 1) * U;
+                for (int u = tid; u < U; u += nc) {
+                    const int i = idx[u];
+                    const T v = wv[u] * hinv;
+                    vn[u] = v;
+                    xw[i] = ADJ ? v : x[i] + eps * v;
                 }
             }
-            __syncthreads();
-            for (int i = tid; i < N; i += blockDim.x) {
-                T w = wv[i];
-                for (int q = 0; q <= j; ++q) w -= (T)H[(long long)j * (m + 1) + q] * V[(long long)q * N + i];
-                wv[i] = w;
-            }
-            __syncthreads();
-        }
-        T accT = T(0);
-        for (int i = tid; i < N; i += blockDim.x) accT += wv[i] * wv[i];
-        double wn2 = block_sum(accT, red);
-        if (tid == 0) {
-            const double hn = sqrt(wn2);
-            hcol[j + 1] = hn;
-            // Givens: apply previous rotations to column j, then the new one
-            for (int i = 0; i < j; ++i) {
-                double t = cs[i] * hcol[i] + sn[i] * hcol[i + 1];
-                hcol[i + 1] = -sn[i] * hcol[i] + cs[i] * hcol[i + 1];
-                hcol[i] = t;
-            }
-            double aa = hcol[j], bb = hcol[j + 1];
-            double c = 1.0, s = 0.0;
-            if (bb != 0.0) {
-                double r = hypot(aa, bb);
-                c = aa / r;
-                s = bb / r;
-            }
-            cs[j] = c;
-            sn[j] = s;
-            hcol[j] = c * aa + s * bb;
-            hcol[j + 1] = 0.0;
-            gv[j + 1] = -s * gv[j];
-            gv[j] = c * gv[j];
-            for (int i = 0; i <= j; ++i) H[(long long)j * (m + 1) + i] = hcol[i];
-            const double res = fabs(gv[j + 1]);
-            s_flag = (res <= target || !(hn > 0.0) || !isfinite(res)) ? 1 : 0;
-            s_scalar[0] = hn;
+        } else if (j > 0) {
+            const int pj = (j - 1) & 1;
+            const T* const h = hp + pj * 2 * (m + 1);
+            const bool stop = coarse_givens<T>(gs, j - 1, h, h + m + 1, s_hn2[pj]);
+            if (lane == 0) s_flag[pj] = stop;
         }
         __syncthreads();
         k = j + 1;
-        if (s_flag) break;
-        const T hinv = (T)(1.0 / s_scalar[0]);
-        T* vn = V + (long long)(j + 1) * N;
-        for (int i = tid; i < N; i += blockDim.x) vn[i] = wv[i] * hinv;
-        __syncthreads();
-    }
-    // back-substitution (thread 0), y into gv
-    if (tid == 0) {
-        for (int i = k - 1; i >= 0; --i) {
-            double t = gv[i];
-            for (int q = i + 1; q < k; ++q) t -= H[(long long)q * (m + 1) + i] * gv[q];
-            gv[i] = t / H[(long long)i * (m + 1) + i];
+        if (j > 0 && s_flag[(j - 1) & 1]) {
+            k = j;
+            break;
         }
-        if (a.iters) *a.iters += k;
+    }
+    // the last column, if the loop ran to its end; back-substitution,
+    // y into hp
+    if (!comp) {
+        if (k == m) {
+            const int pj = (m - 1) & 1;
+            const T* const h = hp + pj * 2 * (m + 1);
+            coarse_givens<T>(gs, m - 1, h, h + m + 1, s_hn2[pj]);
+        }
+        for (int i = k - 1; i >= 0; --i) {
+            const double* const Hi = gs.H + (size_t)i * (m + 1);
+            const double y = gs.gv[i] * gs.dinv[i];
+            __syncwarp();
+            if (lane == 0) gs.gv[i] = y;
+            for (int q = lane; q < i; q += 32) gs.gv[q] = fma(-Hi[q], y, gs.gv[q]);
+            __syncwarp();
+        }
+        for (int q = lane; q < k; q += 32) hp[q] = (T)gs.gv[q];
+        if (lane == 0 && a.iters) *a.iters += k;
+    } else {
+        for (int i = tid; i < N; i += nc)
+            if (!coarse_inner(g, i)) a.s[i] = T(0);
     }
     __syncthreads();
-    for (int i = tid; i < N; i += blockDim.x) {
-        T sv = T(0);
-        for (int q = 0; q < k; ++q) sv += (T)gv[q] * V[(long long)q * N + i];
-        a.s[i] = coarse_inner(g, i) ? sv : T(0);
+    for (int u = tid; u < U; u += blockDim.x) {
+        T s0 = T(0), s1 = T(0);
+        int q = 0;
+        for (; q + 1 < k; q += 2) {
+            s0 += hp[q] * V[q * U + u];
+            s1 += hp[q + 1] * V[(q + 1) * U + u];
+        }
+        if (q < k) s0 += hp[q] * V[q * U + u];
+        a.s[idx[u]] = s0 + s1;
     }
 }
 
 template <typename T, Prob P, bool ADJ>
-__global__ void __launch_bounds__(kCoarseThreads) coarse_gmres_kernel(CoarseArgs<T> a, int vsm) {
+__global__ void __launch_bounds__(kCoarseMaxThreads + kCoarseGivens) coarse_gmres_kernel(CoarseArgs<T> a, int vsm) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     coarse_gmres_body<T, P, ADJ>(a, smem_raw, vsm != 0);
 }
 
 // one CTA per instance of a batch (all instances share the coarse grid size)
 template <typename T, Prob P, bool ADJ>
-__global__ void __launch_bounds__(kCoarseThreads) coarse_gmres_batched_kernel(const CoarseArgs<T>* args, int vsm) {
+__global__ void __launch_bounds__(kCoarseMaxThreads + kCoarseGivens) coarse_gmres_batched_kernel(const CoarseArgs<T>* args, int vsm) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const CoarseArgs<T> a = args[blockIdx.x];
     coarse_gmres_body<T, P, ADJ>(a, smem_raw, vsm != 0);
@@ -320,12 +420,11 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_gmres_batched_kernel(co
 // Shared memory of the GMRES kernel: work arrays, plus V and H when vsm.
 template <typename T>
 size_t coarse_smem_bytes(const Grid& g, int maxit, bool vsm) {
-    const int ne = (int)g.elements();
-    const int npe = coarse_npe(g);
-    size_t b = sizeof(T) * (3 * (size_t)g.size + (size_t)ne * npe);
-    b = (b + 15) & ~size_t(15);
-    b += sizeof(double) * (4 * (size_t)maxit + 2 + 32);
-    if (vsm) b += sizeof(double) * (size_t)(maxit + 1) * maxit + sizeof(T) * (size_t)(maxit + 1) * g.size;
+    const size_t ne = (size_t)g.elements(), u = (size_t)g.interior(), m = (size_t)maxit;
+    size_t b = sizeof(double) * (5 * m + 2 + 32);
+    b += sizeof(T) * (2 * (size_t)g.size + 2 * u + 4 * (m + 1) + ne * coarse_npe(g));
+    b += sizeof(unsigned short) * (2 * u + ne);
+    if (vsm) b += sizeof(double) * (m + 1) * m + sizeof(T) * (m + 1) * u;
     return b;
 }
 

@@ -72,37 +72,39 @@ __device__ __forceinline__ void coarse_element_plain(const T* ue, T kap, T lh, T
 }
 // out of line: elements outside the fixed-point range
 template <Prob P>
-__device__ __noinline__ void coarse_element_fp64(const Grid& g, const double* b, double kap, double lh, double* C) {
+__device__ __noinline__ void coarse_element_fp64(const Grid& g, const double* b, double kap, double lh, double* C,
+                                                 int cs) {
     constexpr int K = is_2d(P) ? 4 : 8;
     double ue[K], r[K];
     for (int c = 0; c < K; ++c) ue[c] = b[(c & 1) + ((c >> 1) & 1) * g.sy + (c >> 2) * g.sz];
     coarse_element_plain<double, P>(ue, kap, lh, r);
-    for (int c = 0; c < K; ++c) C[c] = r[c];
+    for (int c = 0; c < K; ++c) C[c * cs] = r[c];
 }
 
-// contributions of element (x, y, z) for the vector w into C[npe]
+// contributions of an element into C[k * cs], k < npe; b: the vector's entry at
+// the element's first node (of its first component)
 template <typename T, Prob P>
-__device__ __forceinline__ void coarse_element(const Grid& g, const T* w, int x, int y, int z, T kap, T lh,
-                                               const CoarseElem<T, P>& ce, T* C) {
+__device__ __forceinline__ void coarse_element_at(const Grid& g, const T* b, T kap, T lh, const CoarseElem<T, P>& ce,
+                                                  T* C, int cs) {
     if constexpr (P == Prob::BEAM3) {
         T ue[24], r[24];
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-            const int node = ((z + (c >> 2)) * g.ny + y + ((c >> 1) & 1)) * g.nx + x + (c & 1);
+            const int node = ((c >> 2) * g.ny + ((c >> 1) & 1)) * g.nx + (c & 1);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) ue[3 * c + i] = w[node * 3 + i];
+            for (int i = 0; i < 3; ++i) ue[3 * c + i] = b[node * 3 + i];
         }
         bool done = false;
         if constexpr (sizeof(T) == 8) done = ce.ok && coarse_beam_fx(ue, ce.b, r);
         if (!done) elem_neohooke<T>(ue, lh, r);
 #pragma unroll
-        for (int k = 0; k < 24; ++k) C[k] = r[k];
+        for (int k = 0; k < 24; ++k) C[k * cs] = r[k];
     } else {
         constexpr int K = is_2d(P) ? 4 : 8;
-        const T* b = w + (long long)z * g.sz + (long long)y * g.sy + x;
+        const int sy = (int)g.sy, sz = (int)g.sz;
         T ue[K];
 #pragma unroll
-        for (int c = 0; c < K; ++c) ue[c] = b[(c & 1) + ((c >> 1) & 1) * g.sy + (c >> 2) * g.sz];
+        for (int c = 0; c < K; ++c) ue[c] = b[(c & 1) + ((c >> 1) & 1) * sy + (c >> 2) * sz];
         if constexpr (sizeof(T) == 8) {
             fx_t p[K], q[K];
             int xm = 0, X = 0;
@@ -119,7 +121,7 @@ __device__ __forceinline__ void coarse_element(const Grid& g, const T* w, int x,
             } else {
                 if (xm == 0) {  // a zero element contributes zero
 #pragma unroll
-                    for (int c = 0; c < K; ++c) C[c] = T(0);
+                    for (int c = 0; c < K; ++c) C[c * cs] = T(0);
                     return;
                 }
                 if constexpr (P == Prob::MINSURF2) {
@@ -131,17 +133,25 @@ __device__ __forceinline__ void coarse_element(const Grid& g, const T* w, int x,
             }
             if (done) {
 #pragma unroll
-                for (int c = 0; c < K; ++c) C[c] = fx_to_double(q[c], X);
+                for (int c = 0; c < K; ++c) C[c * cs] = fx_to_double(q[c], X);
             } else {
-                coarse_element_fp64<P>(g, b, kap, lh, C);
+                coarse_element_fp64<P>(g, b, kap, lh, C, cs);
             }
         } else {
             T r[K];
             coarse_element_plain<T, P>(ue, kap, lh, r);
 #pragma unroll
-            for (int c = 0; c < K; ++c) C[c] = r[c];
+            for (int c = 0; c < K; ++c) C[c * cs] = r[c];
         }
     }
+}
+
+// contributions of element (x, y, z) for the vector w into C[npe]
+template <typename T, Prob P>
+__device__ __forceinline__ void coarse_element(const Grid& g, const T* w, int x, int y, int z, T kap, T lh,
+                                               const CoarseElem<T, P>& ce, T* C) {
+    const long long b = P == Prob::BEAM3 ? 3LL * ((z * g.ny + y) * g.nx + x) : z * g.sz + y * g.sy + x;
+    coarse_element_at<T, P>(g, w + b, kap, lh, ce, C, 1);
 }
 
 }  // namespace jfnk
