@@ -77,10 +77,8 @@ __device__ __forceinline__ uint64_t b_splitmix(uint64_t z) {
     return z ^ (z >> 31);
 }
 
-// A thread's running sum of |v| or v^2.  FP32 entries are summed as an FP32 pair
-// (Knuth's two-sum; squares as product and its FMA remainder), 44 bits or more
-// without the FP64 pipe, on which the conversion, product and sum of every
-// entry would run at 2 a clock and SM.
+// A thread's running sum of |v| or v^2 (FP32: squares as product and its FMA
+// remainder).
 template <typename T>
 struct BSum;
 template <>
@@ -92,18 +90,13 @@ struct BSum<double> {
 };
 template <>
 struct BSum<float> {
-    float h = 0.f, l = 0.f;
-    __device__ void add(float v, float rest) {
-        const float t = h + v, b = t - h;
-        l += ((h - (t - b)) + (v - b)) + rest;
-        h = t;
-    }
-    __device__ void abs(float v) { add(fabsf(v), 0.f); }
+    F2Sum s;
+    __device__ void abs(float v) { s.add(fabsf(v), 0.f); }
     __device__ void sq(float v) {
         const float p = v * v;
-        add(p, isfinite(p) ? fmaf(v, v, -p) : 0.f);
+        s.add(p, isfinite(p) ? fmaf(v, v, -p) : 0.f);
     }
-    __device__ double value() const { return isfinite(h) ? (double)h + (double)l : (double)h; }
+    __device__ F2Sum value() const { return s; }
 };
 
 // b times the FP64 scalar whose FP32 parts are th + tl, rounded once

@@ -11,10 +11,43 @@ __device__ __forceinline__ float warp_sum(float v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+// FP64 sums over a warp by integer additions: the significands at the largest
+// exponent with 5 bits below its last place (32 of them fit 63 bits), which an
+// FP64 addition of two lanes' values is not more accurate than.  Five shuffled
+// FP64 additions take the pipe 5 x 64 clocks a warp; this takes it 64.
 __device__ __forceinline__ double warp_sum(double v) {
+    const int hi = __double2hiint(v), be = (hi >> 20) & 0x7ff;
+    const int top = __reduce_max_sync(0xffffffffu, be);
+    if (top < 64 || top > 2040) {  // near underflow or overflow, or not finite
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    }
+    long long m = ((__double_as_longlong(v) & 0xfffffffffffffLL) | (be ? 0x10000000000000LL : 0LL)) << 5;
+    m >>= min(top - be, 63);
+    if (hi < 0) m = -m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+    const double d = __ll2double_rn(m);
+    return m ? __hiloint2double(__double2hiint(d) + (top - 1080) * (1 << 20), __double2loint(d)) : 0.0;
+}
+
+// A running sum as an FP32 pair (Knuth's two-sum): 44 bits or more without the
+// FP64 pipe, on which the conversion and sum of every entry would run at 2 a
+// clock and SM.
+struct F2Sum {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float v, float rest) {
+        const float t = h + v, b = t - h;
+        l += ((h - (t - b)) + (v - b)) + rest;
+        h = t;
+    }
+    __device__ __forceinline__ double value() const { return isfinite(h) ? (double)h + (double)l : (double)h; }
+};
+__device__ __forceinline__ F2Sum shfl_add(F2Sum s, int o) {
+    const float h = __shfl_xor_sync(0xffffffffu, s.h, o), l = __shfl_xor_sync(0xffffffffu, s.l, o);
+    s.add(h, l);
+    return s;
 }
 
 // Sum over the block of one double per warp-summed value.  All threads must
@@ -38,13 +71,41 @@ __device__ __forceinline__ double block_sum(TA v, double* sm) {
     return t;
 }
 
+// The same for FP32 pairs: converted to FP64 once a block.
+__device__ __forceinline__ double block_sum(F2Sum v, double* sm) {
+    const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+    const int nw = (blockDim.x * blockDim.y * blockDim.z + 31) / 32;
+    float2* const s2 = reinterpret_cast<float2*>(sm);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = shfl_add(v, o);
+    if ((tid & 31) == 0) s2[tid >> 5] = make_float2(v.h, v.l);
+    __syncthreads();
+    double t = 0.0;
+    if (tid < 32) {
+        F2Sum s;
+        if (tid < nw) {
+            s.h = s2[tid].x;
+            s.l = s2[tid].y;
+        }
+        for (int o = nw > 16 ? 16 : nw > 8 ? 8 : nw > 4 ? 4 : nw > 2 ? 2 : nw > 1 ? 1 : 0; o > 0; o >>= 1) s = shfl_add(s, o);
+        t = s.value();
+    }
+    __syncthreads();
+    return t;
+}
+
+// Orders this thread's memory accesses before and after for the GPU (with an
+// atomic after or before it: release, acquire).
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
 // Last-block completion over a segment of nb CTAs (bid = this CTA's index in
 // it).  Thread 0 of every block passes its block sum; returns true in every
 // thread of the last block of the segment, with the total in *total (thread
 // 0).  The completion counter is reset by the last block.  `early` runs in one
 // thread of the last block while the others sum the partials, and is visible to
-// thread 0 on return.  (At most 4 warps sum: an FP64 addition takes an SM
-// quarter 64 clocks a warp.  Blocks have at least one whole warp.)
+// thread 0 on return.  (One warp sums up to 128 partials and 4 warps more: an
+// FP64 addition takes an SM quarter 64 clocks a warp.  Blocks have at least one
+// whole warp.)
 template <typename F>
 __device__ __forceinline__ bool grid_sum_last_seg(double blocksum, double* partials, unsigned int* counter,
                                                   double* total, unsigned int bid, unsigned int nb, F early) {
@@ -61,25 +122,33 @@ __device__ __forceinline__ bool grid_sum_last_seg(double blocksum, double* parti
     __shared__ int s_last;
     if (tid == 0) {
         partials[bid] = blocksum;
-        __threadfence();
+        fence_gpu();
         unsigned int prev = atomicAdd(counter, 1u);
+        fence_gpu();
         s_last = (prev == nb - 1) ? 1 : 0;
     }
     __syncthreads();
     if (!s_last) return false;
-    __threadfence();
-    const int act = nt >= 128 ? 128 : nt & ~31;
+    const int act = nb <= 128 ? 32 : nt >= 128 ? 128 : nt & ~31;
+    double s = 0.0;
     if (tid < act) {
-        double s = 0.0;
-#pragma unroll 4
-        for (unsigned int i = tid; i < nb; i += act) s += __ldcg(&partials[i]);
+        double part[4];
+        unsigned int i = tid;
+        do {  // four loads in flight
+#pragma unroll
+            for (int k = 0; k < 4; ++k) part[k] = i + k * act < nb ? __ldcg(&partials[i + k * act]) : 0.0;
+            i += 4 * act;
+            if (act == 32 && nb <= 32)
+                s = part[0];
+            else
+                s += (part[0] + part[1]) + (part[2] + part[3]);
+        } while (i < nb);
         s = warp_sum(s);
-        if ((tid & 31) == 0) s_part[tid >> 5] = s;
+        if (act > 32 && (tid & 31) == 0) s_part[tid >> 5] = s;
     }
     if (tid == (act < nt ? act : 0)) early();
     __syncthreads();
     if (tid == 0) {
-        double s = s_part[0];
         for (int w = 1; w < act / 32; ++w) s += s_part[w];
         *total = s;
         *counter = 0u;

@@ -63,7 +63,7 @@ __global__ void masked_stat_kernel(Grid g, const T* x, int what, double* out, do
 // entries.  One warp per row, lanes along x, rows dealt to warps in a fixed
 // order (reproducible sums); one integer division per row instead of two per
 // entry, and one floating-point operation per entry.  FP32 vectors are summed
-// in FP32 within a row, then in FP64.  (The FP64 pipe runs at 1/64 of the
+// in FP32 within a row, then as FP32 pairs.  (The FP64 pipe runs at 1/64 of the
 // FP32 rate on this GPU: converting every entry to FP64, or FP64 compares and
 // predicated-off FP64 instructions of an unrolled loop, made these reductions
 // bound by that pipe.)
@@ -91,9 +91,9 @@ __device__ __forceinline__ float abs_bits(float v) { return __int_as_float(__flo
 // Sum over the interior entries x = 1 .. nx-2 of one row taken by lane `lane`
 // (every 32nd entry): |v| (WHAT = 0) or v^2 (WHAT = 1).  Exactly one
 // floating-point operation per entry; FP32 rows are summed in FP32 (at most
-// 16 entries a lane up to n = 512), then added in FP64.
+// 16 entries a lane up to n = 512), then added as FP32 pairs.
 template <typename T, int WHAT>
-__device__ __forceinline__ double row_stat(const T* __restrict__ row, int nx, int lane) {
+__device__ __forceinline__ T row_stat(const T* __restrict__ row, int nx, int lane) {
     T f = T(0);
 #pragma unroll 4
     for (int x = 1 + lane; x < nx - 1; x += 32) {
@@ -103,8 +103,22 @@ __device__ __forceinline__ double row_stat(const T* __restrict__ row, int nx, in
         else
             f = fma(v, v, f);
     }
-    return (double)f;
+    return f;
 }
+
+// A thread's sum over rows.
+template <typename T>
+struct RowSum;
+template <>
+struct RowSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double f) { s += f; }
+};
+template <>
+struct RowSum<float> {
+    F2Sum s;
+    __device__ __forceinline__ void add(float f) { s.add(f, 0.f); }
+};
 
 template <typename T, int WHAT>
 __global__ void __launch_bounds__(kVecThreads) masked_stat_rows_kernel(Grid g, const T* __restrict__ x, double* out,
@@ -115,11 +129,11 @@ __global__ void __launch_bounds__(kVecThreads) masked_stat_rows_kernel(Grid g, c
     const int lane = threadIdx.x & 31;
     const unsigned int nrows = (unsigned int)interior_rows(g);
     const unsigned int wstride = gridDim.x * kRowWarps;
-    double acc = 0.0;
+    RowSum<T> acc;
     for (unsigned int r = blockIdx.x * kRowWarps + (threadIdx.x >> 5); r < nrows; r += wstride)
-        acc += row_stat<T, WHAT>(x + JFNK_IDX(interior_row_base(g, r), g.size - g.nx + 1), g.nx, lane);
+        acc.add(row_stat<T, WHAT>(x + JFNK_IDX(interior_row_base(g, r), g.size - g.nx + 1), g.nx, lane));
     __shared__ EpsPre pre;
-    double bs = block_sum(acc, sm);
+    double bs = block_sum(acc.s, sm);
     double tot = 0.0;
     if (grid_sum_last(bs, partials, counter, &tot, [&] {
             if (slot) pre = eps_pre(ep);
@@ -127,18 +141,23 @@ __global__ void __launch_bounds__(kVecThreads) masked_stat_rows_kernel(Grid g, c
         finish_stat(WHAT, tot, out, norm_out, pre, ep, slot);
 }
 
-// at most kVecBlocks blocks (8 per SM); up to 2048 blocks, one row a warp at
-// 129^3, measured slower (30 against 24 us for two FP32 norms at 129^3)
+// blocks of the row kernels: 8 per SM at most in FP32, 4 in FP64, which is bound
+// by that pipe (norm at 129^3: FP64 13.6 us against 15.1 with 8 per SM and 14.4
+// with 2, 257^3 52.7 against 54.9; FP32 at 257^3 36 against 42 with 4 per SM).
+// With block sums by integers and FP32 pairs (reduce.cuh): 129^3 FP64 18.5 -> 12.9,
+// FP32 13.0 -> 8.5 us
+template <typename T>
 static int row_blocks(long long rows) {
-    long long b = (rows + kRowWarps - 1) / kRowWarps;
-    return (int)(b < kVecBlocks ? (b < 1 ? 1 : b) : kVecBlocks);
+    constexpr long long cap = sizeof(T) == 8 ? kVecBlocks / 2 : kVecBlocks;
+    const long long b = (rows + kRowWarps - 1) / kRowWarps;
+    return (int)(b < cap ? (b < 1 ? 1 : b) : cap);
 }
 
 template <typename T>
 static jfnk_status launch_masked_stat(const Grid& g, const T* x, int what, double* out, const EpsParams& ep,
                                       EpsSlot* slot, double* norm_out, RedScratch* red, cudaStream_t st) {
     if (g.nc == 1 && !g.beam && g.n >= 2 && g.size <= 0x7fffffffLL) {
-        const int nb = row_blocks(interior_rows(g));
+        const int nb = row_blocks<T>(interior_rows(g));
         if (what == 0)
             masked_stat_rows_kernel<T, 0><<<nb, kVecThreads, 0, st>>>(g, x, out, red->partial, &red->counter[0], ep,
                                                                       slot, norm_out);
@@ -218,18 +237,17 @@ __global__ void multi_dot_kernel(const double* __restrict__ w, const double* __r
         double s = 0.0;
         for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s += sm[threadIdx.x][q];
         partials[(long long)(g0 + threadIdx.x) * gridDim.x + blockIdx.x] = s;
-        __threadfence();
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
+        fence_gpu();
         unsigned int nb = gridDim.x * gridDim.y;
         unsigned int prev = atomicAdd(counter, 1u);
+        fence_gpu();
         s_last = (prev == nb - 1) ? 1 : 0;
     }
     __syncthreads();
     if (!s_last) return;
-    __threadfence();
     // last block: each warp sums one vector's partials in order
     for (int k = wid; k < m; k += blockDim.x >> 5) {
         double s = 0.0;
@@ -520,7 +538,7 @@ __global__ void __launch_bounds__(kVecThreads) cheb_start_zero_rows_kernel(
     const unsigned int nrows = (unsigned int)(g.ny * g.nz);
     const unsigned int wstride = gridDim.x * kRowWarps;
     const int nx = g.nx;
-    double acc = 0.0;
+    RowSum<T> acc;
     for (unsigned int row = blockIdx.x * kRowWarps + (threadIdx.x >> 5); row < nrows; row += wstride) {
         const unsigned int zz = row / (unsigned int)g.ny, yy = row - zz * (unsigned int)g.ny;
         const bool inner_row = yy > 0 && yy < (unsigned int)g.ny - 1 && (g.d == 2 || (zz > 0 && zz < (unsigned int)g.nz - 1));
@@ -538,10 +556,10 @@ __global__ void __launch_bounds__(kVecThreads) cheb_start_zero_rows_kernel(
             dr[x] = dv;
             f = fma(dv, dv, f);
         }
-        acc += (double)f;
+        acc.add(f);
     }
     __shared__ EpsPre pre;
-    double bs = block_sum(acc, sm);
+    double bs = block_sum(acc.s, sm);
     double tot = 0.0;
     if (grid_sum_last(bs, partials, counter, &tot, [&] { pre = eps_pre(ep); }) && threadIdx.x == 0)
         set_eps_slot<false>(slot, pre, tot, false, nullptr);
@@ -551,7 +569,7 @@ template <typename T>
 jfnk_status cheb_start_zero(const Grid& g, const T* b, T* r, T* d, const ChebTable* cheb, const EpsParams& ep,
                             EpsSlot* slot, RedScratch* red, cudaStream_t st) {
     if (g.nc == 1 && !g.beam && g.n >= 2 && g.size <= 0x7fffffffLL) {
-        cheb_start_zero_rows_kernel<T><<<row_blocks((long long)g.ny * g.nz), kVecThreads, 0, st>>>(
+        cheb_start_zero_rows_kernel<T><<<row_blocks<T>((long long)g.ny * g.nz), kVecThreads, 0, st>>>(
             g, b, r, d, cheb, ep, slot, red->partial, &red->counter[0]);
     } else {
         cheb_start_zero_kernel<T><<<vec_blocks(g.size), kVecThreads, 0, st>>>(g, b, r, d, cheb, ep, slot,
