@@ -243,8 +243,9 @@ static size_t plan(P& p, char* base, const jfnk_options* o) {
     if (const char* e = getenv("JFNK_EP3D_CLUSTER_MIN_N")) p.cl_min_n32 = atoi(e);
     if (const char* e = getenv("JFNK_EP3D_CLUSTER_MAX_N")) p.cl_max_n32 = atoi(e);
     // an explicit choice of another kernel stands
-    const bool fx = !getenv("JFNK_EP3D_MAX_N_F64") && !getenv("JFNK_ZM3D_MIN_N_F64") && !getenv("JFNK_V2_THREADS_F64");
-    bool t3 = true;
+    const bool tiled = p.d == 3 && p.desc.kind != JFNK_BEAM3D;
+    const bool fx = tiled && !getenv("JFNK_EP3D_MAX_N_F64") && !getenv("JFNK_ZM3D_MIN_N_F64") && !getenv("JFNK_V2_THREADS_F64");
+    bool t3 = tiled;
     for (const char* e : {"JFNK_EP3D_MAX_N_F32", "JFNK_ZM3D_MIN_N_F32", "JFNK_V2_THREADS_F32", "JFNK_V3_F32",
                           "JFNK_EP3D_CLUSTER_MIN_N", "JFNK_EP3D_CLUSTER_MAX_N"})
         t3 = t3 && !getenv(e);
