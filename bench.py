@@ -18,8 +18,10 @@ extras:  FP32-preconditioned solve of the same workload (FP32 vs FP64 PC),
 roofline: the dominant kernel (the FP64 element-residual kernel with the fused
          Chebyshev epilogue) timed with CUDA events on its stream during K more
          solves right after the timed ones (the value itself is timed without
-         per-launch events, V-cycles replayed from their CUDA graph); FP64-ALU
-         bound.
+         per-launch events, V-cycles replayed from their CUDA graph).  Its
+         elements run in 64-bit fixed point on the integer pipes: against HBM,
+         with its rate in element operations beside it as a multiple of the
+         FP64 pipe's.
 extras:  also the same problem on 257^3 nodes, FP32 vs FP64 preconditioner,
          the 64-instance batched Bratu solve vs the same instances one by
          one, the forward + adjoint solve of the coefficient problem, and the
@@ -78,14 +80,13 @@ def load_peaks():
 # instructions (add, mul or fma) per clock per SM (the per-SM peak ncu reports
 # for sm__sass_thread_inst_executed_op_dfma_pred_on) x the maximum SM clock;
 # 0.629e12 instructions/s at 2070 MHz (the nominal 1.25 TFLOP/s counts an FMA
-# as two flops).  The roofline uses the rate measured by jfnk_measure_peaks and
-# reports this one beside it as a cross-check.
+# as two flops).  Reported beside the rate measured by jfnk_measure_peaks.
 GB300_SMS = 152
 FP64_INST_PER_CLK_SM = 2
-# DRAM bytes (read + write) of one fused FP64 Chebyshev step at 129^3 nodes,
-# element + node phase: dram__bytes_read.sum + dram__bytes_write.sum of the two
-# kernels in one ncu capture of the same kernels (profiles/ holds the summary)
-EP_CHEB_N128_TRAFFIC = (33.854720 + 72.549632 + 198.806784 + 29.048064) * 1e6
+# DRAM bytes (read + write) of one fused FP64 Chebyshev step at 129^3 nodes:
+# dram__bytes_read.sum + dram__bytes_write.sum in one ncu capture of the same
+# kernel (profiles/ holds the summary)
+FX_CHEB_N128_TRAFFIC = (97.86 + 15.08) * 1e6
 
 
 def fp64_peak(peaks):
@@ -598,7 +599,8 @@ def main():
                        "pct_hbm": 100.0 * byts / t / 1e9 / hbm, "alu_ops_per_s": ops,
                        "pct_alu": 100.0 * ops / alu_peak,
                        "alu_basis": (f"{ND_OPS_PER_ELEMENT} element operations x {n}^3 elements / time, of the "
-                                     + ("measured FP64 FMA rate" if name == "f64" else
+                                     + ("measured FP64 FMA rate (fixed point runs on the integer pipes)"
+                                        if name == "f64" else
                                         "measured packed-FP32 (f32x2) FMA rate"))}
 
     # ---- batched workload and adjoint workload ---------------------------------
@@ -614,24 +616,26 @@ def main():
     if top:
         name, (cnt, tot, elems) = top
         avg_s = tot / cnt * 1e-3
-        ops = ND_OPS_PER_ELEMENT * elems
-        achieved = ops / avg_s / 1e12
-        peak = alu["fp64"] / 1e12
-        derived = fp64_peak(peaks) / 1e12
+        ops = ND_OPS_PER_ELEMENT * elems / avg_s
+        algorithmic = 8 * 8 * dof
+        achieved = algorithmic / avg_s / 1e9
+        derived = fp64_peak(peaks)
         total_ms_all = sum(v[1] for v in prof.values())
-        traffic = EP_CHEB_N128_TRAFFIC if name == "stencil_nd3d_f64_CHEB_n128" else None
-        roof = {"kernel": name, "bound": "alu", "achieved": achieved, "peak": peak,
-                "unit": "Top/s (fp64 pipe)", "frac": achieved / peak, "traffic": traffic,
-                "traffic_unit": "bytes per fused step (element + node phase)",
-                "traffic_source": "ncu capture of the same two kernels at 129^3 (dram__bytes_read.sum + "
+        traffic = FX_CHEB_N128_TRAFFIC if name == "stencil_nd3d_f64_CHEB_n128" else None
+        roof = {"kernel": name, "bound": "hbm", "achieved": achieved, "peak": hbm,
+                "unit": "GB/s", "frac": achieved / hbm, "traffic": traffic,
+                "traffic_unit": "bytes per fused step",
+                "traffic_source": "ncu capture of the same kernel at 129^3 (dram__bytes_read.sum + "
                                   "dram__bytes_write.sum), not measured in this run",
-                "algorithmic_bytes": 8 * 8 * dof,
+                "algorithmic_bytes": algorithmic,
+                "note": "64-bit fixed-point element: integer issue and dependent chains bound it, not HBM",
                 "avg_launch_ms": avg_s * 1e3, "launches": cnt,
                 "share_of_stencil_time": tot / total_ms_all if total_ms_all else None,
                 "timed_region": f"{args.steps} event-bracketed solves after the value's timed region "
                                 f"({ms_prof:.1f} ms per solve)",
-                "peak_source": "measured: jfnk_measure_peaks, FP64 FMA chains on every SM, in this run",
-                "peak_derived": derived, "frac_of_derived": achieved / derived}
+                "peak_source": f"{peaks_src}: device copy",
+                "element_ops_per_s": ops, "of_fp64_pipe_measured": ops / alu["fp64"],
+                "of_fp64_pipe_derived": ops / derived}
 
     cpu = None
     if rank == 0 and world == 1:

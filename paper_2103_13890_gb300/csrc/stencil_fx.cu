@@ -14,8 +14,9 @@
 // runs, so that the last wave is as full as the others.
 //
 // Bound by instruction issue and dependent chains of integer arithmetic (about
-// 700 instructions an element); measured against the FP64-pipe kernels
-// (stencil_ep.cu): residual 129^3 0.622 -> 0.129 ms, 257^3 4.89 -> 0.844 ms, FD
+// 1200 instructions an element, 700 of them its arithmetic; half of the issue
+// slots busy); measured against the FP64-pipe kernels
+// (stencil_ep.cu): residual 129^3 0.622 -> 0.127 ms, 257^3 4.89 -> 0.844 ms, FD
 // action with kappa 101^3 0.414 -> 0.075 ms.  CTAs of at most 288 threads, two
 // per SM, 96 registers: 257^3 residual 0.844 ms, against 0.903 (576 x 1), 1.035
 // (192 x 3) and 0.901 ms (256 x 2, 128 registers).
