@@ -1415,6 +1415,10 @@ jfnk_status jfnk_solve_batched(jfnk_problem* const* problems, int count, const j
             set_error("jfnk_solve_batched: instance %d is not a 2D Bratu problem (or has no iterate)", i);
             return JFNK_ERR_INVALID_ARG;
         }
+        if (fx2d_strips(p.n) > 2 * kMaxRedBlocks) {
+            set_error("jfnk_solve_batched: instance %d: 2D grid too large for the reduction scratch", i);
+            return JFNK_ERR_INVALID_ARG;
+        }
         if (p.lv[0].g.n != problems[0]->lv[0].g.n || p.coarse_maxit != problems[0]->coarse_maxit) {
             set_error("jfnk_solve_batched: all hierarchies must end at the same coarse grid");
             return JFNK_ERR_INVALID_ARG;

@@ -18,7 +18,8 @@ __global__ void __launch_bounds__(32 * kFx2Warps) fx2d_kernel(const StencilArgs<
 
 template <typename T>
 bool fx2d_use(Prob prob, const StencilArgs<T>& a, Mode mode) {
-    return is_2d(prob) && a.g.n >= 2 && (sizeof(T) == 4 || a.node_scale == T(1)) && !fx_outputs_alias(a, mode);
+    return is_2d(prob) && a.g.n >= 2 && (sizeof(T) == 4 || a.node_scale == T(1)) &&
+           (a.red == RedOut::NONE || fx2d_strips(a.g.n) <= 2 * kMaxRedBlocks) && !fx_outputs_alias(a, mode);
 }
 template bool fx2d_use<double>(Prob, const StencilArgs<double>&, Mode);
 template bool fx2d_use<float>(Prob, const StencilArgs<float>&, Mode);

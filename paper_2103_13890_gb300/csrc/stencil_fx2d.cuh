@@ -29,7 +29,9 @@ constexpr int kFx2Slots64 = 152 * 20, kFx2Slots32 = 152 * 40;
 __host__ __device__ inline int fx2d_strips(int n) { return (n - 1 + kFx2Strip - 1) / kFx2Strip; }
 
 // True when the kernels take this call: outputs apart from the vectors whose
-// neighbouring values other lanes still read, and (FP64) no node factor.
+// neighbouring values other lanes still read, (FP64) no node factor, and no more
+// strips (a CTA has one) than the reduction scratch holds partials where the
+// call reduces: n <= 61441, the row-segment kernel beyond.
 template <typename T>
 bool fx2d_use(Prob prob, const StencilArgs<T>& a, Mode mode);
 
