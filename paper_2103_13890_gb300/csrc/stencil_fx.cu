@@ -179,7 +179,8 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx3d_kernel(const Stenc
                 } else {
 #pragma unroll
                     for (int c = 0; c < 8; ++c) r[c] = 0;
-                    if (ADJ ? xv != 0 || xm == kFxBad : xm != 0) {
+                    // (a zero element has none, but for 0 x NaN and 0 x Inf)
+                    if ((ADJ ? xv != 0 || xm == kFxBad : xm != 0) || (KAPPA && !fx_finite(kap))) {
                         double rs[8];
                         if (ADJ)
                             vjp3_fp64<KAPPA>(a, gx, gy, k, kap, rs);
