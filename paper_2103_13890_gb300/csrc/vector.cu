@@ -3,6 +3,8 @@
 #include "reduce.cuh"
 #include "vector.cuh"
 
+#include <algorithm>
+
 namespace jfnk {
 
 constexpr int kVecThreads = 256;
@@ -63,7 +65,7 @@ __global__ void masked_stat_kernel(Grid g, const T* x, int what, double* out, do
 // entries.  One warp per row, lanes along x, rows dealt to warps in a fixed
 // order (reproducible sums); one integer division per row instead of two per
 // entry, and one floating-point operation per entry.  FP32 vectors are summed
-// in FP32 within a row, then as FP32 pairs.  (The FP64 pipe runs at 1/64 of the
+// in FP32 within a row, then in FP64.  (The FP64 pipe runs at 1/64 of the
 // FP32 rate on this GPU: converting every entry to FP64, or FP64 compares and
 // predicated-off FP64 instructions of an unrolled loop, made these reductions
 // bound by that pipe.)
@@ -91,9 +93,10 @@ __device__ __forceinline__ float abs_bits(float v) { return __int_as_float(__flo
 // Sum over the interior entries x = 1 .. nx-2 of one row taken by lane `lane`
 // (every 32nd entry): |v| (WHAT = 0) or v^2 (WHAT = 1).  Exactly one
 // floating-point operation per entry; FP32 rows are summed in FP32 (at most
-// 16 entries a lane up to n = 512), then added as FP32 pairs.
+// 16 entries a lane up to n = 512), then added in FP64, whose range the sum over
+// the rows needs.
 template <typename T, int WHAT>
-__device__ __forceinline__ T row_stat(const T* __restrict__ row, int nx, int lane) {
+__device__ __forceinline__ double row_stat(const T* __restrict__ row, int nx, int lane) {
     T f = T(0);
 #pragma unroll 4
     for (int x = 1 + lane; x < nx - 1; x += 32) {
@@ -103,22 +106,8 @@ __device__ __forceinline__ T row_stat(const T* __restrict__ row, int nx, int lan
         else
             f = fma(v, v, f);
     }
-    return f;
+    return (double)f;
 }
-
-// A thread's sum over rows.
-template <typename T>
-struct RowSum;
-template <>
-struct RowSum<double> {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double f) { s += f; }
-};
-template <>
-struct RowSum<float> {
-    F2Sum s;
-    __device__ __forceinline__ void add(float f) { s.add(f, 0.f); }
-};
 
 template <typename T, int WHAT>
 __global__ void __launch_bounds__(kVecThreads) masked_stat_rows_kernel(Grid g, const T* __restrict__ x, double* out,
@@ -129,11 +118,11 @@ __global__ void __launch_bounds__(kVecThreads) masked_stat_rows_kernel(Grid g, c
     const int lane = threadIdx.x & 31;
     const unsigned int nrows = (unsigned int)interior_rows(g);
     const unsigned int wstride = gridDim.x * kRowWarps;
-    RowSum<T> acc;
+    double acc = 0.0;
     for (unsigned int r = blockIdx.x * kRowWarps + (threadIdx.x >> 5); r < nrows; r += wstride)
-        acc.add(row_stat<T, WHAT>(x + JFNK_IDX(interior_row_base(g, r), g.size - g.nx + 1), g.nx, lane));
+        acc += row_stat<T, WHAT>(x + JFNK_IDX(interior_row_base(g, r), g.size - g.nx + 1), g.nx, lane);
     __shared__ EpsPre pre;
-    double bs = block_sum(acc.s, sm);
+    double bs = block_sum(acc, sm);
     double tot = 0.0;
     if (grid_sum_last(bs, partials, counter, &tot, [&] {
             if (slot) pre = eps_pre(ep);
@@ -144,13 +133,16 @@ __global__ void __launch_bounds__(kVecThreads) masked_stat_rows_kernel(Grid g, c
 // blocks of the row kernels: 8 per SM at most in FP32, 4 in FP64, which is bound
 // by that pipe (norm at 129^3: FP64 13.6 us against 15.1 with 8 per SM and 14.4
 // with 2, 257^3 52.7 against 54.9; FP32 at 257^3 36 against 42 with 4 per SM).
-// With block sums by integers and FP32 pairs (reduce.cuh): 129^3 FP64 18.5 -> 12.9,
-// FP32 13.0 -> 8.5 us
+// A block's sum costs a warp as many FP64 operations as its rows do, so FP32
+// blocks beyond two per SM take three rows a warp: 97^3 12.3 -> 8.2 us, 129^3 12.3
+// -> 11.1 us (launches back to back), 65^3 and below as with one row a warp,
+// 193^3 and above at the most blocks.
 template <typename T>
 static int row_blocks(long long rows) {
     constexpr long long cap = sizeof(T) == 8 ? kVecBlocks / 2 : kVecBlocks;
-    const long long b = (rows + kRowWarps - 1) / kRowWarps;
-    return (int)(b < cap ? (b < 1 ? 1 : b) : cap);
+    constexpr long long few = sizeof(T) == 8 ? cap : 2 * kNumSMs;
+    const long long one = (rows + kRowWarps - 1) / kRowWarps, three = (one + 2) / 3;
+    return (int)std::max(1LL, std::min(cap, std::max(three, std::min(one, few))));
 }
 
 template <typename T>
@@ -538,7 +530,7 @@ __global__ void __launch_bounds__(kVecThreads) cheb_start_zero_rows_kernel(
     const unsigned int nrows = (unsigned int)(g.ny * g.nz);
     const unsigned int wstride = gridDim.x * kRowWarps;
     const int nx = g.nx;
-    RowSum<T> acc;
+    double acc = 0.0;
     for (unsigned int row = blockIdx.x * kRowWarps + (threadIdx.x >> 5); row < nrows; row += wstride) {
         const unsigned int zz = row / (unsigned int)g.ny, yy = row - zz * (unsigned int)g.ny;
         const bool inner_row = yy > 0 && yy < (unsigned int)g.ny - 1 && (g.d == 2 || (zz > 0 && zz < (unsigned int)g.nz - 1));
@@ -556,10 +548,10 @@ __global__ void __launch_bounds__(kVecThreads) cheb_start_zero_rows_kernel(
             dr[x] = dv;
             f = fma(dv, dv, f);
         }
-        acc.add(f);
+        acc += (double)f;
     }
     __shared__ EpsPre pre;
-    double bs = block_sum(acc.s, sm);
+    double bs = block_sum(acc, sm);
     double tot = 0.0;
     if (grid_sum_last(bs, partials, counter, &tot, [&] { pre = eps_pre(ep); }) && threadIdx.x == 0)
         set_eps_slot<false>(slot, pre, tot, false, nullptr);
