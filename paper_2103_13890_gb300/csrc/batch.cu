@@ -77,27 +77,16 @@ __device__ __forceinline__ uint64_t b_splitmix(uint64_t z) {
     return z ^ (z >> 31);
 }
 
-// A thread's running sum of |v| or v^2 (FP32: squares as product and its FMA
-// remainder).
-template <typename T>
-struct BSum;
-template <>
-struct BSum<double> {
-    double s = 0.0;
-    __device__ void abs(double v) { s += fabs(v); }
-    __device__ void sq(double v) { s += v * v; }
-    __device__ double value() const { return s; }
-};
-template <>
-struct BSum<float> {
-    F2Sum s;
-    __device__ void abs(float v) { s.add(fabsf(v), 0.f); }
-    __device__ void sq(float v) {
-        const float p = v * v;
-        s.add(p, isfinite(p) ? fmaf(v, v, -p) : 0.f);
-    }
-    __device__ F2Sum value() const { return s; }
-};
+// The same value in FP64, on the integer pipe for zero and normal FP32 values: the
+// hardware conversion runs on the FP64 pipe, at the rate of the multiply-add that
+// follows it.
+__device__ __forceinline__ double b_wide(double v) { return v; }
+__device__ __forceinline__ double b_wide(float v) {
+    const unsigned int b = __float_as_uint(v), a = b & 0x7fffffffu;
+    if (a != 0u && a - 0x00800000u >= 0x7f000000u) return (double)v;  // subnormal, infinite or NaN
+    const unsigned int hi = (b & 0x80000000u) | (a ? (a >> 3) + ((1023u - 127u) << 20) : 0u);
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
 
 // b times the FP64 scalar whose FP32 parts are th + tl, rounded once
 __device__ __forceinline__ double b_scaled(double b, double ti, double, double) { return b * ti; }
@@ -142,30 +131,28 @@ __global__ void __launch_bounds__(kBThreads) bvec_kernel(const BVec* __restrict_
             ((T*)d.y)[i] = v;
         }
     } else if (OP == BOp::STAT || OP == BOp::CHEB_START) {
-        BSum<T> acc;
+        double acc = 0.0;
         const double ti = (OP == BOp::CHEB_START) ? d.cheb->theta_inv : 0.0;
         const T th = (T)ti, tl = (T)(ti - (double)th);
         for (long long i = i0; i < d.g.size; i += stride) {
             const bool in = b_inner(d.g, i);
             if (OP == BOp::STAT) {
                 if (!in) continue;
-                const T v = ((const T*)d.x)[i];
-                if (d.what == 0)
-                    acc.abs(v);
-                else
-                    acc.sq(v);
+                const double v = b_wide(((const T*)d.x)[i]);
+                acc += d.what == 0 ? fabs(v) : v * v;
             } else {
                 const T bv = in ? ((const T*)d.x)[i] : T(0);
                 const T dv = b_scaled(bv, ti, th, tl);
                 ((T*)d.y)[i] = bv;        // r
                 ((T*)d.y2)[i] = dv;       // d
                 ((T*)d.x2)[i] = T(0);     // s (written through x2's address)
-                acc.sq(dv);
+                const double v = b_wide(dv);
+                acc += v * v;
             }
         }
         __shared__ EpsPre pre;
         const bool norm = OP != BOp::STAT || d.what != 0;
-        const double bs = block_sum(acc.value(), sm);
+        const double bs = block_sum(acc, sm);
         double tot = 0.0;
         if (grid_sum_last_seg(bs, d.partials, d.counter, &tot, it.bid, it.nblk, [&] {
                 if (d.slot && norm) pre = eps_pre(d.ep);

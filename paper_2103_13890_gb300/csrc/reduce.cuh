@@ -32,24 +32,6 @@ __device__ __forceinline__ double warp_sum(double v) {
     return m ? __hiloint2double(__double2hiint(d) + (top - 1080) * (1 << 20), __double2loint(d)) : 0.0;
 }
 
-// A running sum as an FP32 pair (Knuth's two-sum): 44 bits or more without the
-// FP64 pipe, on which the conversion and sum of every entry would run at 2 a
-// clock and SM.
-struct F2Sum {
-    float h = 0.f, l = 0.f;
-    __device__ __forceinline__ void add(float v, float rest) {
-        const float t = h + v, b = t - h;
-        l += ((h - (t - b)) + (v - b)) + rest;
-        h = t;
-    }
-    __device__ __forceinline__ double value() const { return isfinite(h) ? (double)h + (double)l : (double)h; }
-};
-__device__ __forceinline__ F2Sum shfl_add(F2Sum s, int o) {
-    const float h = __shfl_xor_sync(0xffffffffu, s.h, o), l = __shfl_xor_sync(0xffffffffu, s.l, o);
-    s.add(h, l);
-    return s;
-}
-
 // Sum over the block of one double per warp-summed value.  All threads must
 // call it.  `sm` holds >= 32 doubles.  Result valid in thread 0.
 template <typename TA>
@@ -66,29 +48,6 @@ __device__ __forceinline__ double block_sum(TA v, double* sm) {
         t = (tid < nw) ? sm[tid] : 0.0;
         for (int o = nw > 16 ? 16 : nw > 8 ? 8 : nw > 4 ? 4 : nw > 2 ? 2 : nw > 1 ? 1 : 0; o > 0; o >>= 1)
             t += __shfl_xor_sync(0xffffffffu, t, o);
-    }
-    __syncthreads();
-    return t;
-}
-
-// The same for FP32 pairs: converted to FP64 once a block.
-__device__ __forceinline__ double block_sum(F2Sum v, double* sm) {
-    const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-    const int nw = (blockDim.x * blockDim.y * blockDim.z + 31) / 32;
-    float2* const s2 = reinterpret_cast<float2*>(sm);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = shfl_add(v, o);
-    if ((tid & 31) == 0) s2[tid >> 5] = make_float2(v.h, v.l);
-    __syncthreads();
-    double t = 0.0;
-    if (tid < 32) {
-        F2Sum s;
-        if (tid < nw) {
-            s.h = s2[tid].x;
-            s.l = s2[tid].y;
-        }
-        for (int o = nw > 16 ? 16 : nw > 8 ? 8 : nw > 4 ? 4 : nw > 2 ? 2 : nw > 1 ? 1 : 0; o > 0; o >>= 1) s = shfl_add(s, o);
-        t = s.value();
     }
     __syncthreads();
     return t;
