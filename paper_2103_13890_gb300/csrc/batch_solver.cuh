@@ -770,9 +770,11 @@ static jfnk_status bsetup(BCtx& b, const std::vector<int>& S, int newton_step) {
         }
         if (!any) break;
         if (o.power_tol > 0.0) {
-            std::vector<int> running;  // (an instance may be named once per level)
+            std::vector<int> running;  // the instances named on any level, once each
             for (int c = 1; c <= cmax; ++c)
                 running.insert(running.end(), Rl[c].begin(), Rl[c].end());
+            std::sort(running.begin(), running.end());
+            running.erase(std::unique(running.begin(), running.end()), running.end());
             std::vector<double> hr;
             JFNK_TRY(bgather(b, running, hr));
             for (int c = 1; c <= cmax; ++c)

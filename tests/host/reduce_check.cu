@@ -1,8 +1,11 @@
-// GPU check of the warp sum (csrc/reduce.cuh) and of the batched norms
-// (csrc/batch.cu), which no entry point reaches on chosen values:
+// GPU check of the reductions' device functions (csrc/reduce.cuh, stencil.cuh,
+// coarse.cuh) and of the batched norms (csrc/batch.cu), which no entry point
+// reaches on chosen values:
 //   1. warp_sum(double): mixed exponents, cancellation, zeros and subnormals, the
 //      ends of its integer path, NaN and infinities in one lane;
-//   2. batched FP32 norms over values whose squares leave FP32's range.
+//   2. set_eps_slot: the norm, the FD step and its reciprocal as IEEE square
+//      root and divisions give them, over the exponent range;
+//   3. batched FP32 norms over values whose squares leave FP32's range.
 // Prints one line per violation and "ok" at the end.
 #include <cmath>
 #include <cstdio>
@@ -11,7 +14,9 @@
 #include <vector>
 
 #include "batch.cuh"
+#include "coarse.cuh"
 #include "reduce.cuh"
+#include "stencil.cuh"
 
 using namespace jfnk;
 
@@ -104,6 +109,42 @@ static void check_warp_sum() {
 }
 
 // ---- 2 --------------------------------------------------------------------
+__global__ void eps_kernel(const double* tot, const double* k, int n, int unit, EpsSlot* slot, double* nrm) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) set_eps_slot(slot + i, EpsPre{k[i], 1.0 / k[i]}, tot[i], unit != 0, nullptr, nrm + i);
+}
+
+static void check_eps_slot() {
+    std::mt19937_64 rng(2);
+    std::uniform_real_distribution<double> u(1.0, 2.0);
+    std::vector<double> tot, k;
+    for (int i = 0; i < 400000; ++i) {
+        const int wide = i & 1;
+        tot.push_back(std::ldexp(u(rng), wide ? (int)(rng() % 2040) - 1020 : (int)(rng() % 60) - 30));
+        k.push_back(std::ldexp(u(rng), wide ? (int)(rng() % 60) - 40 : -26));
+    }
+    for (double t : {1.0, 4.0, 0x1.fffffffffffffp+1, 0x1.0000000000001p+0, 4.9406564584124654e-324}) {
+        tot.push_back(t);
+        k.push_back(1.4901161193847656e-08);
+    }
+    const int n = (int)tot.size();
+    Dev<double> dt(tot), dk(k), dn(n);
+    Dev<EpsSlot> ds(n);
+    for (int unit = 0; unit < 2; ++unit) {
+        eps_kernel<<<(n + 255) / 256, 256>>>(dt.p, dk.p, n, unit, ds.p, dn.p);
+        const std::vector<double> nrm = dn.get();
+        const std::vector<EpsSlot> s = ds.get();
+        for (int i = 0; i < n; ++i) {
+            const double r = std::sqrt(tot[i]), e = k[i] / r, inv = unit ? 1.0 / k[i] : 1.0 / e;
+            CHECK(nrm[i] == r, "norm of %a: %a instead of %a", tot[i], nrm[i], r);
+            CHECK(s[i].e == e, "step %a / %a: %a instead of %a", k[i], r, s[i].e, e);
+            CHECK(s[i].inv == inv, "reciprocal step: %a instead of %a", s[i].inv, inv);
+            CHECK(s[i].ef == (float)e && s[i].invf == (float)inv, "FP32 step of %a", e);
+        }
+    }
+}
+
+// ---- 3 --------------------------------------------------------------------
 static void check_batched_norms() {
     std::mt19937_64 rng(3);
     std::uniform_real_distribution<double> u(0.5, 1.0);
@@ -154,6 +195,7 @@ static void check_batched_norms() {
 
 int main() {
     check_warp_sum();
+    check_eps_slot();
     check_batched_norms();
     const cudaError_t e = cudaDeviceSynchronize();
     CHECK(e == cudaSuccess, "%s", cudaGetErrorString(e));
