@@ -169,25 +169,36 @@ __device__ inline double rsqrt_newton(double x) {
 // The FD-step slot of the action on a vector whose squares sum to tot, with its
 // reciprocal in both precisions, and the norm; unit: for the direction v/||v||
 // (see RedOut::EPS_UNIT).  GUARD: a non-finite step sets bit 1 of the status word
-// and 0.  (One thread runs this at the end of every smoothing step, and an FP64
-// operation of one thread takes as long as one of a warp, 64 clocks: 9 in place
-// of about 40 with a square root and two divisions.)
+// and 0.  One thread runs this at the end of every smoothing step, and an FP64
+// operation of one thread takes as long as one of a warp, 64 clocks: the square
+// root and the two quotients come from one reciprocal square root, each with one
+// correction by its exact remainder (Newton's step; the result is the correctly
+// rounded one but for about one argument in 2^49, and for quotients by a number
+// whose significand is all ones, which are divided).  15 operations, 12 of them
+// dependent, in place of about 40.
 template <bool GUARD = true>
 __device__ inline void set_eps_slot(EpsSlot* slot, const EpsPre& pre, double tot, bool unit, int* status,
                                     double* norm_out = nullptr, double* norm_out2 = nullptr) {
     double nrm = tot, e = 0.0, inv = 0.0;
-    if (tot > 0.0) {
-        double r;
-        const unsigned int ex = (unsigned int)__double2hiint(tot) >> 20;  // biased exponent (sign: 0)
-        if (ex != 0u && ex != 0x7ffu) {
-            r = rsqrt_newton(tot);
-            nrm = tot * r;
-        } else {  // subnormal or infinite
-            nrm = sqrt(tot);
-            r = 1.0 / nrm;
+    const unsigned int et = (unsigned int)__double2hiint(tot) >> 20, ek = (unsigned int)__double2hiint(pre.k) >> 20;
+    bool done = et - 123u < 1800u && ek - 523u < 1000u;  // in [2^-900, 2^900), k in [2^-500, 2^500): all normal
+    if (done) {
+        const double r = rsqrt_newton(tot), g = tot * r, q = pre.k * r;
+        nrm = fma(fma(-g, g, tot), 0.5 * r, g);
+        e = fma(fma(-nrm, q, pre.k), r, q);
+        if (unit) {
+            inv = pre.inv;
+        } else {
+            const double i0 = g * pre.inv;
+            inv = fma(fma(-e, i0, 1.0), i0, i0);
         }
-        e = pre.k * r;
-        inv = e > 0.0 ? (unit ? pre.inv : nrm * pre.inv) : 0.0;
+        auto ones = [](double x) { return (__double2hiint(x) | 0xfff00000) == -1 && __double2loint(x) == -1; };
+        done = !ones(nrm) && !ones(e);
+    }
+    if (!done && tot > 0.0) {
+        nrm = sqrt(tot);
+        e = pre.k / nrm;
+        inv = e > 0.0 ? (unit ? pre.inv : 1.0 / e) : 0.0;
         if (GUARD && !(isfinite(e) && isfinite(inv))) {
             if (status) atomicOr(status, 1);
             e = 0.0;
