@@ -19,8 +19,8 @@
 //   - six barriers an iteration, five of them among the computing warps only.
 // Measured (default tolerance; before: a block-wide norm per basis vector, warp-wide
 // dot products and the rotations by one thread between the barriers): 5^3 nodes 105
-// -> 33 us in FP32 and 171 -> 67 us in FP64, 9^2 nodes 299 -> 74 and 437 -> 140 us,
-// 10^3 nodes 670 -> 230 and 1798 -> 719 us.
+// -> 34 us in FP32 and 171 -> 73 us in FP64, 9^2 nodes 299 -> 72 and 437 -> 143 us,
+// 10^3 nodes 670 -> 191 and 1798 -> 780 us.
 #include "coarse.cuh"
 #include "coarse_elem.cuh"
 #include "element.cuh"
@@ -92,12 +92,6 @@ __device__ __forceinline__ T coarse_gather(const Grid& g, const T* C, int ne, in
     return acc;
 }
 
-// 1 / sqrt(x) of a sum of squares.
-__device__ __forceinline__ float coarse_rsqrt(float x) { return 1.0f / sqrtf(x); }
-__device__ __forceinline__ double coarse_rsqrt(double x) {
-    return x >= 2.2250738585072014e-308 && x <= 1.7976931348623157e308 ? rsqrt_newton(x) : 1.0 / sqrt(x);
-}
-
 // The work of the Givens warp.  One column: the raw entries h1 + h2 (two
 // Gram-Schmidt passes) and the squared norm hn2 of what remains; applies the
 // earlier rotations, forms the new one and the residual estimate.  Returns
@@ -145,7 +139,8 @@ __device__ bool coarse_givens(const CoarseGivens& s, int j, const T* h1, const T
     if (__all_sync(0xffffffffu, q2 >= 1e-280 && q2 <= 1e280)) {
         const double qi = rsqrt_newton(q2);
         ri = __shfl_sync(0xffffffffu, qi, 0);
-        hn = hn2 * __shfl_sync(0xffffffffu, qi, 1);
+        const double hi = __shfl_sync(0xffffffffu, qi, 1), h0 = hn2 * hi;
+        hn = fma(fma(-h0, h0, hn2), 0.5 * hi, h0);
     } else {
         hn = sqrt(hn2);
         ri = 1.0 / hypot(r, hn);
@@ -190,6 +185,7 @@ __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_ra
     gs.gv = gs.dinv + m;                          // [m + 1]
     gs.work = gs.gv + (m + 1);                    // [m + 1]
     double* const red = gs.work + (m + 1);        // [32]
+    T* const part = reinterpret_cast<T*>(red);    // [2][16] squared norms of the warps by column parity
     gs.H = a.H;
     double* end = red + 32;
     if (vsm) {
@@ -206,11 +202,14 @@ __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_ra
     unsigned short* const idx = reinterpret_cast<unsigned short*>(vsm ? V + (size_t)(m + 1) * U : C + npe * ne);
     unsigned short* const eref = idx + U;    // [U]
     unsigned short* const eoff = eref + U;   // [ne]
-    __shared__ double s_hn2[2];
     __shared__ int s_flag[2];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nc = blockDim.x - kCoarseGivens, nw = nc >> 5;
     const bool comp = tid < nc;
+    constexpr int LU = sizeof(T) == 8 ? 2 : 1;      // lanes of an unknown's update
+    const int nwu = min(nw, (U * LU + 31) / 32);    // warps with unknowns
+    // squared norm of what remains of column j, by the Givens warp
+    auto remains = [&](int j) { return warp_sum(lane < nwu ? (double)part[(j & 1) * 16 + lane] : 0.0); };
 
     // ||b|| over the unknowns; V_0 = b / ||b||
     double acc = 0.0;
@@ -267,7 +266,9 @@ __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_ra
         const double bi = s_beta[1];
         for (int u = tid; u < U; u += nc) {
             const int i = idx[u];
-            const T v = (T)((double)a.b[i] * bi);
+            double q = (double)a.b[i] * bi;
+            if (sizeof(T) == 8) q = fma(fma(-q, beta, (double)a.b[i]), bi, q);  // (the quotient's rounding alone)
+            const T v = (T)q;
             V[u] = v;
             if (!ADJ) Ax[u] = a.Ax[i];
             xw[i] = ADJ ? v : x[i] + eps * v;
@@ -276,7 +277,6 @@ __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_ra
     __syncthreads();
     const CoarseElem<T, P> ce(a.lh);
     const int lg = U <= 128 ? 3 : 5, dl = 1 << lg;  // lanes of a dot product
-    constexpr int LU = sizeof(T) == 8 ? 2 : 1;      // lanes of an unknown's update
     int k = 0;
     // (dots and updates in the basis precision T: in an FP32 preconditioner the
     // single CTA would otherwise spend its iterations on this SM's FP64 pipe,
@@ -329,24 +329,14 @@ __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_ra
                 if (pass == 0) coarse_sync(nc);
             }
             // the squared norm of what remains
-            const int nwu = min(nw, (U * LU + 31) / 32);  // warps with unknowns
+            T* const pj = part + (j & 1) * 16;
             if (wid < nwu) {
                 n2 = warp_sum(n2);
-                if (lane == 0) red[wid] = (double)n2;
+                if (lane == 0) pj[wid] = n2;
             }
             coarse_sync(nc);
-            T hn2;
-            if (sizeof(T) == 8) {
-                double t = red[0];
-                for (int w = 1; w < nwu; ++w) t += red[w];
-                hn2 = (T)t;
-            } else {
-                hn2 = (T)red[0];
-                for (int w = 1; w < nwu; ++w) hn2 += (T)red[w];
-            }
-            if (tid == 0) s_hn2[j & 1] = (double)hn2;
             if (j + 1 < m && tid < U) {
-                const T hinv = coarse_rsqrt(hn2);
+                const T hinv = coarse_rsqrt(pj, nwu);
                 T* const vn = V + (j + 1) * U;
                 for (int u = tid; u < U; u += nc) {
                     const int i = idx[u];
@@ -358,7 +348,7 @@ __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_ra
         } else if (j > 0) {
             const int pj = (j - 1) & 1;
             const T* const h = hp + pj * 2 * (m + 1);
-            const bool stop = coarse_givens<T>(gs, j - 1, h, h + m + 1, s_hn2[pj]);
+            const bool stop = coarse_givens<T>(gs, j - 1, h, h + m + 1, remains(j - 1));
             if (lane == 0) s_flag[pj] = stop;
         }
         __syncthreads();
@@ -374,7 +364,7 @@ __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_ra
         if (k == m) {
             const int pj = (m - 1) & 1;
             const T* const h = hp + pj * 2 * (m + 1);
-            coarse_givens<T>(gs, m - 1, h, h + m + 1, s_hn2[pj]);
+            coarse_givens<T>(gs, m - 1, h, h + m + 1, remains(m - 1));
         }
         for (int i = k - 1; i >= 0; --i) {
             const double* const Hi = gs.H + (size_t)i * (m + 1);

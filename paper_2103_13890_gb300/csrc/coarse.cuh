@@ -51,6 +51,29 @@ struct CoarseArgs {
     LbfgsState* lb;
 };
 
+#ifdef __CUDACC__
+// 1 / sqrt of the sum of n squared norms >= 0.  FP32: summed as a pair (two-sum), and
+// one Newton step on the pair, which leaves the rounding of the result (in FP64 the
+// sum and root would hold every computing warp for their latencies).
+__device__ __forceinline__ float coarse_rsqrt(const float* p, int n) {
+    float h = p[0], l = 0.f;
+    for (int w = 1; w < n; ++w) {
+        const float v = p[w], t = h + v, b = t - h;
+        l += (h - (t - b)) + (v - b);
+        h = t;
+    }
+    if (!(h >= 0x1p-100f && h <= 0x1p100f)) return (float)(1.0 / sqrt((double)h + (double)l));
+    const float y = rsqrtf(h), q = y * y, qe = fmaf(y, y, -q);
+    const float e = fmaf(-l, q, fmaf(-h, qe, fmaf(-h, q, 1.f)));  // 1 - (h + l) y^2
+    return fmaf(0.5f * y, e, y);
+}
+__device__ __forceinline__ double coarse_rsqrt(const double* p, int n) {
+    double t = p[0];
+    for (int w = 1; w < n; ++w) t += p[w];
+    return t >= 2.2250738585072014e-308 && t <= 1.7976931348623157e308 ? rsqrt_newton(t) : 1.0 / sqrt(t);
+}
+#endif
+
 // method 1 (coarse_cg.cu)
 template <typename T>
 jfnk_status launch_coarse_cgqn(Prob prob, const CoarseArgs<T>& a, cudaStream_t st);

@@ -192,7 +192,7 @@ __device__ inline void set_eps_slot(EpsSlot* slot, const EpsPre& pre, double tot
             const double i0 = g * pre.inv;
             inv = fma(fma(-e, i0, 1.0), i0, i0);
         }
-        auto ones = [](double x) { return (__double2hiint(x) | 0xfff00000) == -1 && __double2loint(x) == -1; };
+        auto ones = [](double x) { return (__double2hiint(x) | ~0xfffff) == -1 && __double2loint(x) == -1; };
         done = !ones(nrm) && !ones(e);
     }
     if (!done && tot > 0.0) {

@@ -5,7 +5,8 @@
 //      ends of its integer path, NaN and infinities in one lane;
 //   2. set_eps_slot: the norm, the FD step and its reciprocal as IEEE square
 //      root and divisions give them, over the exponent range;
-//   3. batched FP32 norms over values whose squares leave FP32's range.
+//   3. batched FP32 norms over values whose squares leave FP32's range;
+//   4. coarse_rsqrt in FP32: 1 / sqrt of a sum of squared norms, rounded once.
 // Prints one line per violation and "ok" at the end.
 #include <cmath>
 #include <cstdio>
@@ -193,7 +194,42 @@ static void check_batched_norms() {
     }
 }
 
+// ---- 4 --------------------------------------------------------------------
+__global__ void rsqrt_kernel(const float* p, int n, int count, float* out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < count) out[i] = coarse_rsqrt(p + (size_t)i * n, n);
+}
+
+static void check_coarse_rsqrt() {
+    std::mt19937_64 rng(4);
+    std::uniform_real_distribution<double> u(0.0, 1.0);
+    const int count = 100000;
+    for (int n : {1, 2, 7, 15}) {
+        std::vector<float> p;
+        for (int i = 0; i < count; ++i) {
+            const int e = (int)(rng() % 240) - 130;
+            for (int w = 0; w < n; ++w) p.push_back((float)std::ldexp(u(rng), e - (int)(rng() % 8)));
+            p.back() = std::fmax(p.back(), 0x1p-126f);
+        }
+        Dev<float> dp(p), dy(count);
+        rsqrt_kernel<<<(count + 255) / 256, 256>>>(dp.p, n, count, dy.p);
+        const std::vector<float> y = dy.get();
+        for (int i = 0; i < count; ++i) {
+            long double s = 0;
+            for (int w = 0; w < n; ++w) s += (long double)p[(size_t)i * n + w];
+            const long double want = 1 / std::sqrt(s);
+            int e;
+            std::frexp((double)want, &e);
+            // the start is within 2 ulp (e below 2^-21): the step leaves 3/8 e^2 and three
+            // roundings of e, together below 2^-43 of the result
+            const long double ulp = std::ldexp(1.0L, e - 24);
+            CHECK(std::fabs(y[i] - want) <= (0.5L + 0x1p-18L) * ulp, "1/sqrt of %Lg: off by %Lg ulp", s, (y[i] - want) / ulp);
+        }
+    }
+}
+
 int main() {
+    check_coarse_rsqrt();
     check_warp_sum();
     check_eps_slot();
     check_batched_norms();
