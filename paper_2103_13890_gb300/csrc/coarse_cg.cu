@@ -11,12 +11,13 @@
 //
 // One thread-block cluster runs the whole solve.  Every CTA owns a contiguous
 // slice of the unknowns, in its shared memory: the CG vectors and its part of
-// the kept pairs.  x_0 + eps p is pushed to every CTA's copy of the full vector
-// (distributed shared memory), each CTA evaluates the elements that touch its
-// slice, and sums are exchanged by pushing every CTA's partial sums to all
+// the kept pairs.  p is pushed to every CTA's copy of the full vector
+// (distributed shared memory); each CTA sums p.p for the FD step and the Rayleigh
+// quotient, forms x_0 + eps p, and evaluates the elements that touch its slice.
+// The other sums are exchanged by pushing every CTA's partial sums to all
 // CTAs, which add them in rank order: all CTAs hold the same scalars and take
-// the same branches.  Four cluster barriers an iteration: x_0 + eps p; p.q; r.r
-// with S^T r and Y^T r; r.z with z.z and z.p (p.p follows by recurrence).
+// the same branches.  Four cluster barriers an iteration: p; p.q; r.r
+// with S^T r and Y^T r; r.z.
 // The compact L-BFGS form is applied as one 2k x 2k matrix, formed when the
 // pairs are chosen, instead of two triangular solves by one thread.
 //
@@ -51,7 +52,7 @@ struct CgOut {
 // Shared memory of a CTA: doubles first, then the T arrays.
 struct CgLayout {
     int sl;                                   // slice length
-    size_t slots, tot, mat, coef, scal;       // doubles
+    size_t slots, tot, mat, coef, scal, part, step;  // doubles
     size_t x, r, z, p, q, x0, ax, S, Y, xw, ec, mask;
     size_t bytes;
 };
@@ -71,8 +72,11 @@ __host__ __device__ inline CgLayout cg_layout(int N, int ne, int npe, int ctas, 
     l.mat = take((size_t)4 * k * k, 8);
     l.coef = take(2 * k, 8);
     l.scal = take(8, 8);
-    size_t* v[] = {&l.x, &l.r, &l.z, &l.p, &l.q, &l.x0, &l.ax};
+    l.part = take(kCgThreads / 32, 8);
+    l.step = take(1, sizeof(EpsSlot));
+    size_t* v[] = {&l.x, &l.r, &l.z, &l.p, &l.q, &l.ax};
     for (size_t* a : v) *a = take(l.sl, esz);
+    l.x0 = take(N, esz);
     l.S = take((size_t)k * l.sl, esz);
     l.Y = take((size_t)k * l.sl, esz);
     l.xw = take(N, esz);
@@ -91,7 +95,8 @@ struct CgCta {
     unsigned char* sm;
     int rank, ctas, N, i0, n;  // owned entries [i0, i0 + n)
     int buf = 0;               // slot buffer of the next exchange
-    double xstat, gamma = 1.0;
+    double gamma = 1.0;
+    EpsPre pre;
 
     __device__ CgCta(const CoarseArgs<T>& args, const CgLayout& lay, unsigned char* smem)
         : a(args), cluster(cg::this_cluster()), l(lay), ce(args.lh), sm(smem) {
@@ -100,12 +105,14 @@ struct CgCta {
         N = (int)a.g.size;
         i0 = rank * l.sl;
         n = max(0, min(l.sl, N - i0));
-        xstat = *a.xstat;
+        const EpsParams ep = {a.eps_mode, a.n_unknowns, a.xstat};
+        pre = eps_pre(ep);
     }
     __device__ double* dbl(size_t o) const { return reinterpret_cast<double*>(sm + o); }
     __device__ T* vec(size_t o) const { return reinterpret_cast<T*>(sm + o); }
     __device__ bool inner(int i) const { return sm[l.mask + i] != 0; }
     __device__ double& scal(int i) const { return dbl(l.scal)[i]; }
+    __device__ EpsSlot& slot() const { return *reinterpret_cast<EpsSlot*>(sm + l.step); }
 
     // sum v of this CTA's slice of u . w, by one warp, to every CTA
     __device__ void dot_push(int v, const T* u, const T* w) {
@@ -137,29 +144,41 @@ struct CgCta {
         __syncthreads();
     }
 
-    // FD step for a direction of squared norm pp: scal 0 = eps, 1 = 1 / eps (eps 0: none)
-    __device__ void step(double pp) {
-        const double e = eps_formula(a.eps_mode, a.n_unknowns, xstat, sqrt(pp));
-        const bool ok = e > 0.0 && isfinite(e);
-        scal(0) = ok ? e : 0.0;
-        scal(1) = ok ? 1.0 / e : 0.0;
-    }
-    // q = A_s p = (A(x_0 + eps p) - A(x_0)) / eps - shift p on the slice, with the step in scal 0 / 1
+    // FD step for a direction of squared norm pp (0: none)
+    __device__ void step(double pp) { set_eps_slot(&slot(), pre, pp, false, nullptr); }
+    // q = A_s p = (A(x_0 + eps p) - A(x_0)) / eps - shift p on the slice; p.p in
+    // scal 4, the step in the slot
     __device__ void apply(const T* p, double shift) {
         const Grid& g = a.g;
         T* q = vec(l.q);
-        const T eps = (T)scal(0), inv = (T)scal(1), sh = (T)shift;
-        if (!(scal(0) > 0.0)) {
+        T* xw = vec(l.xw);
+        for (int t = threadIdx.x; t < n * ctas; t += blockDim.x) {
+            const int c = t / n, i = t - c * n;
+            *cluster.map_shared_rank(xw + i0 + i, c) = p[i];
+        }
+        cluster.sync();
+        // every CTA has all of p and sums p.p in the same order
+        double d = 0.0;
+        for (int i = threadIdx.x; i < N; i += blockDim.x) d += (double)xw[i] * (double)xw[i];
+        d = warp_sum(d);
+        if ((threadIdx.x & 31) == 0) dbl(l.part)[threadIdx.x >> 5] = d;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            d = warp_sum(threadIdx.x < kCgThreads / 32 ? dbl(l.part)[threadIdx.x] : 0.0);
+            if (threadIdx.x == 0) {
+                scal(4) = d;
+                step(d);
+            }
+        }
+        __syncthreads();
+        const T eps = (T)slot().e, inv = (T)slot().inv, sh = (T)shift;
+        if (!(slot().e > 0.0)) {
             for (int i = threadIdx.x; i < n; i += blockDim.x) q[i] = T(0);
             __syncthreads();
             return;
         }
-        T* xw = vec(l.xw);
-        for (int t = threadIdx.x; t < n * ctas; t += blockDim.x) {
-            const int c = t / n, i = t - c * n;
-            *cluster.map_shared_rank(xw + i0 + i, c) = vec(l.x0)[i] + eps * p[i];
-        }
-        cluster.sync();
+        for (int i = threadIdx.x; i < N; i += blockDim.x) xw[i] = vec(l.x0)[i] + eps * xw[i];
+        __syncthreads();
         // elements touching the nodes of the slice
         T* ec = vec(l.ec);
         const int nc = g.nc;
@@ -248,8 +267,6 @@ struct CgCta {
         const int tid = threadIdx.x, wid = tid >> 5, nw = blockDim.x >> 5;
         CgOut o = {0.0, 0, 0, 0};
         if (warm) {
-            if (wid == 0) dot_push(0, x, x);
-            exchange(1, [&](double* t) { step(t[0]); });
             apply(x, shift);
             o.fd++;
         }
@@ -261,22 +278,16 @@ struct CgCta {
                 dot_push(v, r, v == 0 ? r : v <= k ? S + (v - 1) * l.sl : Y + (v - 1 - k) * l.sl);
             exchange(1 + 2 * k, [&](double* t) { scal(2) = sqrt(t[0]); });
         };
-        // r.z, z.z, z.p
-        auto direction_sums = [&]() {
-            if (wid < 3) dot_push(wid, z, wid == 0 ? r : wid == 1 ? z : p);
-        };
         residual_sums();
         double res = scal(2);
         if (!(res > 0.0) || res <= target || !isfinite(res)) return o;
         precond(k);
         for (int i = tid; i < n; i += blockDim.x) p[i] = T(0);
         __syncthreads();
-        direction_sums();
-        exchange(3, [&](double* t) {
+        if (wid == 0) dot_push(0, r, z);
+        exchange(1, [&](double* t) {
             scal(3) = t[0];  // r.z
-            scal(4) = t[1];  // p.p of p = z
             scal(5) = 0.0;   // beta
-            step(t[1]);
         });
         for (int it = 1; it <= a.maxit; ++it) {
             const T beta = (T)scal(5);
@@ -310,14 +321,10 @@ struct CgCta {
             res = scal(2);
             if (res <= target || !isfinite(res)) return o;
             precond(k);
-            direction_sums();
-            exchange(3, [&](double* t) {
-                const double b = t[0] / scal(3);
+            if (wid == 0) dot_push(0, r, z);
+            exchange(1, [&](double* t) {
+                scal(5) = t[0] / scal(3);
                 scal(3) = t[0];
-                scal(5) = b;
-                const double pp = t[1] + b * (2.0 * t[2] + b * scal(4));  // |z + b p|^2
-                scal(4) = pp > 0.0 ? pp : 0.0;
-                step(scal(4));
             });
         }
         return o;
@@ -428,10 +435,10 @@ __global__ void __launch_bounds__(kCgThreads) coarse_cgqn_kernel(const CoarseArg
         const bool in = coarse_inner(a.g, c.i0 + i);
         smem_raw[l.mask + i] = in ? 1 : 0;
         c.vec(l.x)[i] = T(0);
-        c.vec(l.x0)[i] = a.x[c.i0 + i];
         c.vec(l.ax)[i] = a.Ax[c.i0 + i];
         c.vec(l.z)[i] = in ? a.b[c.i0 + i] : T(0);
     }
+    for (int i = tid; i < c.N; i += blockDim.x) c.vec(l.x0)[i] = a.x[i];
     const int count = __ldcg(&a.lb->count);
     const bool collect = count < 0;
     int k = collect ? 0 : count;
