@@ -167,11 +167,12 @@ __host__ __device__ __forceinline__ void elem_nd3(const T u[8], T kap, T r[8]) {
 // The same element for kernels that march along z, in 131 operations a layer:
 // the x/y butterflies of a face's corner values are shared by the elements on
 // both sides, and on the test side the two elements' face modes are added
-// before the x/y butterflies.  No mode is scaled by itself: with the gradients
-// taken over A, the powers of A enter the butterflies as multiply-adds, and the
-// common factors 1/8 (gradient), 1/64 (coefficient, formed as 64 + (8u)^2) and
-// A^2 = 1/3 are left to the node factor (kNd3FaceScale).
-constexpr double kNd3FaceScale = 1.0 / (8.0 * 64.0 * 3.0);
+// before the x/y butterflies.  No mode is scaled by itself: the gradients are
+// taken over A, whose powers enter the butterflies as multiply-adds, and the corner
+// values are given over 16, so that half a point's u falls out of the butterflies
+// and the coefficient is 1/4 + (u/2)^2.  The contributions are 3/8 of elem_nd3's:
+// no larger, so that FP32's range is elem_nd3's too (kNd3FaceScale undoes it).
+constexpr double kNd3FaceCorner = 1.0 / 16.0, kNd3FaceScale = 8.0 / 3.0;
 
 // face corners q[a + 2b] -> modes m[p + 2q] (8 operations)
 template <typename T>
@@ -208,9 +209,9 @@ __host__ __device__ __forceinline__ void nd3_faces(const T a[4], const T b[4], T
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const T p = madd(Y0z[k], j ? A : B, P0z[k]);
-            const T um = madd(GX[j][k], B, p), up8 = madd(GX[j][k], A, p);  // 8 u
-            c[0][j][k] = madd(um, um, T(64));
-            c[1][j][k] = madd(up8, up8, T(64));
+            const T um = madd(GX[j][k], B, p), uq = madd(GX[j][k], A, p);  // u / 2
+            c[0][j][k] = madd(um, um, T(0.25));
+            c[1][j][k] = madd(uq, uq, T(0.25));
         }
     T FX[2][2], FY[2][2], FZ[2][2];
 #pragma unroll

@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kT3Threads, 1) t3d_kernel(const StencilArgs<fl
     const int n = a.g.n;
     const int sy = (int)a.g.sy, sz = (int)a.g.sz;
     const int npx = t.ex + 1, npy = t.ey + 1, np = npx * npy, eyp = t.ey >> 1;
-    float* const W = reinterpret_cast<float*>(smem_raw);  // [2][np]: w
+    float* const W = reinterpret_cast<float*>(smem_raw);  // [2][np]: w (not ADJ: times kNd3FaceCorner)
     float* const V = W + (ADJ ? 2 * np : 0);              // [2][np]: direction (ADJ)
     const int cb = (eyp + 1) * npx;
     float* const CA = V + 2 * np;                         // [2][np]: rows 2 ty, 2 ty + 1 from the left column
@@ -96,7 +96,12 @@ __global__ void __launch_bounds__(kT3Threads, 1) t3d_kernel(const StencilArgs<fl
                 if (in2) v2 = dir2 && zin ? pv[JFNK_IDX(j2, sz)] : 0.f;
             }
         };
-        auto wv = [&](float u, float v) { return (!ADJ && M != Mode::F) ? u + eps * v : u; };
+        // (the scaling of the corner values is exact)
+        auto wv = [&](float u, float v) {
+            if (ADJ) return u;
+            const float c = (float)kNd3FaceCorner * u;
+            return M != Mode::F ? fmaf((float)kNd3FaceCorner * eps, v, c) : c;
+        };
         auto store = [&](int z) {
             float* Wz = W + (z & 1) * np;
             float* Vz = V + (z & 1) * np;

@@ -3,13 +3,19 @@
 Norms: an FP32 vector's norm is summed in FP64 beyond a row, so scaling the
 vector by 2^k, with every row's FP32 sum of squares finite and normal, scales the
 norm exactly, the FD step by 2^-k exactly, and leaves u + eps v and so the action's
-bits as they are, also where the sum over all rows exceeds FP32's range."""
+bits as they are, also where the sum over all rows exceeds FP32's range.
+
+Elements: the 3D diffusion terms are formed without a common factor, so F(u) is
+right wherever its largest terms, u^3 times the corners' stiffness, are in FP32's
+range.  Tolerance: 64 roundings of those terms, as in test_gpu_fp32_tiles.py."""
 import numpy as np
 import pytest
 
-from gpu_common import dev, jf, kernel_path, torch
+from gpu_common import dev, host, jf, kernel_path, torch
 
 pytestmark = pytest.mark.gpu
+
+EPS = 2.0 ** -24
 
 
 # squares of N(0, 1) 2^60 stay below 2^125; 29791 and 65025 of them exceed 2^128
@@ -46,3 +52,17 @@ def test_sweep_of_a_scaled_right_hand_side(monkeypatch):
     s = [p.smooth(dev(np.ldexp(b, e)), torch.zeros(p.shape(), device="cuda"), s_is_zero=True) for e in (0, k)]
     assert torch.any(s[0] != 0)
     assert torch.equal(torch.ldexp(s[1], torch.tensor(-k, device="cuda")), s[0])
+
+
+@pytest.mark.parametrize("kind", ["nd3d", "ndk3d"])
+@pytest.mark.parametrize("n", [17, 40])
+def test_large_values(kind, n, monkeypatch):
+    kernel_path(monkeypatch, "default")
+    rng = np.random.default_rng(n)
+    m = 2.0 ** 40  # u^3 = 2^120
+    u = (m * rng.uniform(-1, 1, size=(n + 1,) * 3)).astype(np.float32)
+    kap = torch.ones((n,) * 3, dtype=torch.float64) if kind == "ndk3d" else None
+    p = jf().Problem(kind, n, 1, kappa=kap)
+    F, G = host(p.residual(dev(u))), host(p.residual(dev(u.astype(np.float64))))
+    assert np.all(np.isfinite(F))
+    assert np.max(np.abs(F - G)) <= 64 * EPS * 64 / (3.0 * n) * m * (1 + m * m)
