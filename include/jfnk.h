@@ -138,7 +138,9 @@ typedef struct {
     int coarse_negcurv;                  /* coarse CG calls ended by negative curvature */
     int outer_negcurv;                   /* outer CG solves ended by negative curvature */
     long long nJv[JFNK_MAX_LEVELS];      /* FD Jacobian actions per level (part of nF; the
-                                            coarse Krylov iterations count on level 0) */
+                                            coarse Krylov products count on level 0: GMRES
+                                            stopped by its tolerance has formed one beyond
+                                            its last column) */
     int ls_hist[JFNK_MAX_HIST];          /* residual evaluations of the line search per Newton
                                             step; when none gives a sufficient decrease the
                                             step is not taken (alpha_hist 0, u and ||F||

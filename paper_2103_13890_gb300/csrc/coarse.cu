@@ -14,8 +14,8 @@
 //     round of the warps covers a Gram-Schmidt pass;
 //   - the Givens rotations of column j, serial FP64 arithmetic, run in a warp of
 //     their own while the other warps form the products of iteration j + 1.  The
-//     solve stops one (discarded) iteration after the column that meets the
-//     tolerance;
+//     solve stops one (discarded, but counted) iteration after the column that
+//     meets the tolerance;
 //   - six barriers an iteration, five of them among the computing warps only.
 // Measured (default tolerance; before: a block-wide norm per basis vector, warp-wide
 // dot products and the rotations by one thread between the barriers): 5^3 nodes 105
@@ -277,7 +277,7 @@ __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_ra
     __syncthreads();
     const CoarseElem<T, P> ce(a.lh);
     const int lg = U <= 128 ? 3 : 5, dl = 1 << lg;  // lanes of a dot product
-    int k = 0;
+    int k = 0, formed = 0;  // columns, products
     // (dots and updates in the basis precision T: in an FP32 preconditioner the
     // single CTA would otherwise spend its iterations on this SM's FP64 pipe,
     // 1/74 of the FP32 rate; the Hessenberg entries are kept in FP64)
@@ -352,7 +352,7 @@ __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_ra
             if (lane == 0) s_flag[pj] = stop;
         }
         __syncthreads();
-        k = j + 1;
+        k = formed = j + 1;
         if (j > 0 && s_flag[(j - 1) & 1]) {
             k = j;
             break;
@@ -375,7 +375,7 @@ __device__ void coarse_gmres_body(const CoarseArgs<T>& a, unsigned char* smem_ra
             __syncwarp();
         }
         for (int q = lane; q < k; q += 32) hp[q] = (T)gs.gv[q];
-        if (lane == 0 && a.iters) *a.iters += k;
+        if (lane == 0 && a.iters) *a.iters += formed;
     } else {
         for (int i = tid; i < N; i += nc)
             if (!coarse_inner(g, i)) a.s[i] = T(0);

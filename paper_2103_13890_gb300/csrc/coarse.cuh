@@ -38,7 +38,7 @@ struct CoarseArgs {
     int maxit;
     T* V;                  // (maxit + 1) * g.size scratch
     double* H;             // (maxit + 1) * maxit scratch
-    long long* iters;      // device accumulator of GMRES iterations (GE count), nullable
+    long long* iters;      // device accumulator of products formed (GE count), nullable
     int adjoint;           // 1: solve with J(x_0)^T (exact VJP) instead of the FD action
     // CG with the L-BFGS preconditioner and the spectral shift (method 1)
     int method;            // 0: GMRES, 1: CG-QN with shift (Alg. 1)
