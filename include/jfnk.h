@@ -163,9 +163,9 @@ void jfnk_paper_options(jfnk_options* opts);
  * Allocates only host memory.  INVALID_ARG on bad kind/sizes/levels.
  * The 3D kernel choice per level is read from the environment here; it
  * changes speed only (results differ at rounding level).  Unless one of the
- * variables of its precision is set (CLUSTER and V3: FP32), actions of the
- * diffusion problems run the z-marching kernels (one launch, no scratch; FP64 in
- * fixed point, FP32 from n = 17 on):
+ * variables of its precision is set (V3: FP32), actions of the diffusion problems
+ * run the z-marching kernels (one launch, no scratch; FP64 in fixed point, FP32
+ * from n = 17 on, but for levels in the CLUSTER range):
  *   JFNK_EP3D_MAX_N_F64 / _F32  levels with n <= this run the element-parallel
  *                               kernels (defaults 2^20 / 64)
  *   JFNK_V2_THREADS_F64 / _F32  CTA-size cap of the halo-free kernel (default

@@ -242,19 +242,19 @@ static size_t plan(P& p, char* base, const jfnk_options* o) {
     if (const char* e = getenv("JFNK_ZM3D_MIN_N_F32")) p.zm_min_n32 = atoi(e);
     if (const char* e = getenv("JFNK_EP3D_CLUSTER_MIN_N")) p.cl_min_n32 = atoi(e);
     if (const char* e = getenv("JFNK_EP3D_CLUSTER_MAX_N")) p.cl_max_n32 = atoi(e);
-    // an explicit choice of another kernel stands
+    // the cluster kernels' attributes are set here, outside any graph capture
+    if (p.cl_max_n32 > 0 && !ep3d_cluster_init()) p.cl_max_n32 = 0;
+    // an explicit choice of another kernel stands: for its precision, or (cluster) for its levels
     const bool tiled = p.d == 3 && p.desc.kind != JFNK_BEAM3D;
     const bool fx = tiled && !getenv("JFNK_EP3D_MAX_N_F64") && !getenv("JFNK_ZM3D_MIN_N_F64") && !getenv("JFNK_V2_THREADS_F64");
     bool t3 = tiled;
-    for (const char* e : {"JFNK_EP3D_MAX_N_F32", "JFNK_ZM3D_MIN_N_F32", "JFNK_V2_THREADS_F32", "JFNK_V3_F32",
-                          "JFNK_EP3D_CLUSTER_MIN_N", "JFNK_EP3D_CLUSTER_MAX_N"})
+    for (const char* e : {"JFNK_EP3D_MAX_N_F32", "JFNK_ZM3D_MIN_N_F32", "JFNK_V2_THREADS_F32", "JFNK_V3_F32"})
         t3 = t3 && !getenv(e);
     for (Level& L : p.lv) {
+        const bool cluster = L.g.n >= p.cl_min_n32 && L.g.n <= std::min(p.cl_max_n32, kEpClusterMaxN);
         L.fx = fx ? fx3d_tiling(L.g) : FxTiling{};
-        L.t3 = t3 ? t3d_tiling(L.g) : FxTiling{};
+        L.t3 = t3 && !cluster ? t3d_tiling(L.g) : FxTiling{};
     }
-    // the cluster kernels' attributes are set here, outside any graph capture
-    if (p.cl_max_n32 > 0 && !ep3d_cluster_init()) p.cl_max_n32 = 0;
     if (const char* e = getenv("JFNK_V2_THREADS_F64")) p.v2_threads64 = atoi(e);
     if (const char* e = getenv("JFNK_V2_THREADS_F32")) p.v2_threads32 = atoi(e);
     if (const char* e = getenv("JFNK_V3_F32")) p.v3_f32 = atoi(e);

@@ -400,7 +400,6 @@ __global__ void __launch_bounds__(kEpSmallThreads) ep3d_small_kernel(const Stenc
 // of the element-parallel pair.
 constexpr int kEpClusterThreads = 1024;
 constexpr int kEpClusterMaxCtas = 16;
-constexpr int kEpClusterMaxN = 32;  // S <= 2: 8 S n^2 words = 64 KB of shared memory at n = 32
 
 __host__ __device__ inline int ep3d_cluster_slices(int n) { return (n + kEpClusterMaxCtas - 1) / kEpClusterMaxCtas; }
 __host__ __device__ inline int ep3d_cluster_ctas(int n) {

@@ -33,6 +33,10 @@ inline bool ep3d_use(const StencilArgs<T>& a, bool adj = false) {
            ep3d_scratch_need(a.g, zm) <= a.face_cap;
 }
 
+// Largest level of the cluster kernels (S <= 2 layers a CTA: 8 S n^2 words = 64 KB of
+// shared memory).
+constexpr int kEpClusterMaxN = 32;
+
 // Sets the cluster kernels' attributes on the current device (once) and
 // returns whether a cluster of their largest size fits there.  Called by the
 // launcher; callers that capture launches into a graph call it first.
