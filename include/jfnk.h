@@ -258,8 +258,9 @@ jfnk_status jfnk_smooth(jfnk_problem* p, const jfnk_options* opts, int level, co
                         int s_is_zero, void* stream);
 
 /* Coarse solve of Algorithm 1 on level 0 (Sec. 2, "The coarse level solver"),
- * in one CTA: GMRES (opts->coarse_method = JFNK_COARSE_GMRES) or the paper's
- * CG preconditioned by L-BFGS with the spectral shift (JFNK_COARSE_CGQN): the
+ * in one launch: GMRES in one CTA (opts->coarse_method = JFNK_COARSE_GMRES) or
+ * the paper's CG preconditioned by L-BFGS with the spectral shift in one
+ * thread-block cluster (JFNK_COARSE_CGQN): the
  * first call after jfnk_mg_setup(newton_step = 0) collects the secant pairs and
  * keeps opts->lbfgs_pairs of them (uniform sampling) for every later call; a
  * CG run that meets negative curvature is repeated on A - lambda_c+ I with
@@ -334,7 +335,7 @@ jfnk_status jfnk_jvp_noalloc(int kind, int n_elem, double lambda, const void* ka
                              const void* u, const void* Fu, const void* v, void* Jv, double eps, int eps_mode,
                              void* stream);
 
-/* Limits of the single-CTA coarse solver and of FGMRES. */
+/* Limits of the coarse solvers and of FGMRES. */
 #define JFNK_COARSE_MAX_NODES 1024
 #define JFNK_COARSE_MAX_IT 1024
 #define JFNK_MAX_RESTART 64

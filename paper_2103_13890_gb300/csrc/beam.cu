@@ -54,7 +54,7 @@ template <typename T, Mode M>
 __global__ void __launch_bounds__(kBeamElemThreads, 4) beam_elem_kernel(const StencilArgs<T> a) {
     const Grid g = a.g;
     const int ex = 10 * g.n, ey = g.n, ez = g.n;
-    const int ne = ex * ey * ez;  // (at most 10 x 256^3)
+    const int ne = ex * ey * ez;  // (at most 10 x 414^3 < 2^31: 30 (n + 1)^3 entries are, see jfnk_problem_create)
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= ne) return;
     const int x = e % ex, yz = e / ex, y = yz % ey, z = yz / ey;

@@ -16,7 +16,7 @@
 //     their own while the other warps form the products of iteration j + 1.  The
 //     solve stops one (discarded, but counted) iteration after the column that
 //     meets the tolerance;
-//   - six barriers an iteration, five of them among the computing warps only.
+//   - seven barriers an iteration, six of them among the computing warps only.
 // Measured (default tolerance; before: a block-wide norm per basis vector, warp-wide
 // dot products and the rotations by one thread between the barriers): 5^3 nodes 105
 // -> 34 us in FP32 and 171 -> 73 us in FP64, 9^2 nodes 299 -> 72 and 437 -> 143 us,

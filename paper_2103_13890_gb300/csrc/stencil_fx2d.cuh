@@ -24,7 +24,7 @@ namespace jfnk {
 constexpr int kFx2Strip = 30;     // node columns a warp completes
 constexpr int kFx2Warps = 4;      // per CTA
 // warps a launch is cut into, about what is resident: FP64 96 registers a thread
-constexpr int kFx2Slots64 = 152 * 20, kFx2Slots32 = 152 * 40;
+constexpr int kFx2Slots64 = kNumSMs * 20, kFx2Slots32 = kNumSMs * 40;
 
 __host__ __device__ inline int fx2d_strips(int n) { return (n - 1 + kFx2Strip - 1) / kFx2Strip; }
 

@@ -31,7 +31,11 @@
 
 namespace jfnk {
 
-constexpr int kT3MinN = 17;      // below, one CTA or one cluster does a level in less time (stencil_ep.cu)
+// Smaller levels run in one CTA (n <= 8), in one cluster (n = 16) or, 9 to 15, in the
+// element-parallel pair (stencil_ep.cu).  A smoothing step with its norm takes 8.3-8.4
+// us here and in a cluster for n = 10 to 20 alike, 10.4 us in the pair; the pair on 9 to
+// 15 predates both and is the slower one.
+constexpr int kT3MinN = 17;
 constexpr int kT3Threads = 512;  // largest CTA (128 registers a thread)
 
 template <Prob P, Mode M, bool ADJ>
