@@ -119,7 +119,7 @@ __device__ __forceinline__ void coarse_element_at(const Grid& g, const T* b, T k
                 done = ce.ok && fx_bratu_exp_ok(xe);
                 if (done) fx_bratu2(p, xe, ce.b, q, X);
             } else {
-                if (xm == 0 && (P != Prob::NDK3 || fx_finite(kap))) {  // a zero element contributes zero
+                if (xm == 0 && (P != Prob::NDK3 || fx_scale_ok(kap))) {  // contributes zero (kappa is finite)
 #pragma unroll
                     for (int c = 0; c < K; ++c) C[c * cs] = T(0);
                     return;

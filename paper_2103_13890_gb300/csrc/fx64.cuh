@@ -218,14 +218,13 @@ __host__ __device__ __forceinline__ fx_t fx_pack(double w) {
 }
 __host__ __device__ __forceinline__ int fx_exp(fx_t p) { return (int)fx_lo(p) & kFxMask; }
 // the largest exponent field of an element's corners: 0 for a zero element,
-// which has zero contributions where kappa is finite; in range for fx_nd3 or not
+// which has zero contributions (0 x NaN and 0 x Inf apart); in range for fx_nd3 or not
 __host__ __device__ __forceinline__ bool fx_exp_ok(int x) { return x >= kFxMinExp && x < kFxMaxExp; }
 // a scale (node factor, kappa) fx_nd3 takes: in [2^-300, 2^300)
 __host__ __device__ __forceinline__ bool fx_scale_ok(double scale) {
     const int h = dbl_hi(scale);  // (negative: sign bit set, fails the first test)
     return h >= ((1023 - 300) << 20) && h < ((1023 + 300) << 20);
 }
-__host__ __device__ __forceinline__ bool fx_finite(double x) { return (dbl_hi(x) & 0x7ff00000) != 0x7ff00000; }
 
 // 2-point butterflies of element.cuh (exact here)
 __host__ __device__ __forceinline__ void fx_h2_fwd(fx_t v00, fx_t v10, fx_t v01, fx_t v11, fx_t out[2][2]) {

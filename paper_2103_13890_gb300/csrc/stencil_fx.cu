@@ -167,7 +167,8 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx3d_kernel(const Stenc
                 double kap = 1.0;
                 if (KAPPA) kap = a.kappa[JFNK_IDX(k * n * n + eidx, (long long)n * n * n)];
                 const int xm = max(xl, xu), xv = max(xvl, xvu);
-                const bool fits = (ADJ ? xm < kFxMaxExp && fx_exp_ok(xv) : fx_exp_ok(xm)) && (!KAPPA || fx_scale_ok(kap));
+                const bool kap_ok = !KAPPA || fx_scale_ok(kap);
+                const bool fits = (ADJ ? xm < kFxMaxExp && fx_exp_ok(xv) : fx_exp_ok(xm)) && kap_ok;
                 fx_t r[8];
                 int Xr = kFxTiny;
                 if (fits) {
@@ -179,8 +180,8 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx3d_kernel(const Stenc
                 } else {
 #pragma unroll
                     for (int c = 0; c < 8; ++c) r[c] = 0;
-                    // (a zero element has none, but for 0 x NaN and 0 x Inf)
-                    if ((ADJ ? xv != 0 || xm == kFxBad : xm != 0) || (KAPPA && !fx_finite(kap))) {
+                    // (a zero element has none, but kappa may be NaN or Inf)
+                    if ((ADJ ? xv != 0 || xm == kFxBad : xm != 0) || !kap_ok) {
                         double rs[8];
                         if (ADJ)
                             vjp3_fp64<KAPPA>(a, gx, gy, k, kap, rs);
